@@ -315,23 +315,39 @@ __device__ __forceinline__ StepTime step_time(const StepParams &P, const float2 
 }
 
 // Step times of a launch are the same for every particle: each block computes those of
-// steps [k0, k0 + STEP_TAB) once with step_time and keeps them in shared memory as they
-// are (h0, f, t_k, h1 and the offset); step_time_tab rebuilds a step's StepTime from its
-// entry (measured: the per-particle step_time cost 3.5 % of the step).
+// steps [k0, k0 + STEP_TAB) once with step_time and keeps them in shared memory (the pair's
+// address, fraction and t_k in one 16-byte entry, the offset, the hour); step_time_tab
+// reads a step's StepTime back (measured: the per-particle step_time cost 3.5 % of the step).
 constexpr int STEP_TAB = 128;
 
-__device__ __forceinline__ StepTime step_time_tab(const StepParams &P, const float4 *ta,
-                                                  const float2 *tb, int i, int k)
+struct StepTable {
+    float4 a[STEP_TAB];              // pair address (64 bits), f, t_k
+    float2 off[STEP_TAB];            // du, dv
+    int h0[STEP_TAB];
+};
+
+__device__ __forceinline__ void step_table_set(StepTable &tab, int i, const StepTime &T)
 {
-    const float4 a = ta[i];
-    const float2 b = tb[i];
+    const unsigned long long p = reinterpret_cast<unsigned long long>(T.pair);
+    tab.a[i] = make_float4(__uint_as_float((unsigned int)p), __uint_as_float((unsigned int)(p >> 32)),
+                           T.ts.f, T.tk);
+    tab.off[i] = make_float2(T.du, T.dv);
+    tab.h0[i] = T.ts.h0;
+}
+
+__device__ __forceinline__ StepTime step_time_tab(const StepParams &P, const StepTable &tab, int i,
+                                                  int k)
+{
+    const float4 a = tab.a[i];
+    const float2 b = tab.off[i];
     StepTime T;
     T.k = k;
-    T.tk = a.z;
-    T.ts.h0 = __float_as_int(a.x);
-    T.ts.h1 = __float_as_int(a.w);
-    T.ts.f = a.y;
-    T.pair = P.pair + (long long)T.ts.h0 * P.slab * 2;
+    T.tk = a.w;
+    T.ts.h0 = tab.h0[i];
+    T.ts.h1 = min(T.ts.h0 + 1, P.n_t - 1);
+    T.ts.f = a.z;
+    T.pair = reinterpret_cast<const float4 *>((unsigned long long)__float_as_uint(a.x) |
+                                              ((unsigned long long)__float_as_uint(a.y) << 32));
     T.khp = P.khpair ? P.khpair + (long long)T.ts.h0 * P.slab : nullptr;
     T.blp = P.blpair ? P.blpair + (long long)T.ts.h0 * P.nx * P.ny * 2 : nullptr;
     T.du = b.x;
@@ -393,33 +409,45 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
         zn = z + m.w * P.dt + n2 * sig_z;
         if (P.drift) zn += P.k_scale * m.dkz * P.dt;
     }
-    // 5. reflection, at most 4 folds, then clamp
-    float fs = 1.0f;
+    // 5. reflection, at most 4 folds, then clamp: the first fold by selects (near the ground
+    // most warps hold a lane that folds once), the rest of the loop only where that leaves a
+    // height outside [zf_lo, zf_hi] (0 and z_top, or infinite where nothing reflects)
+    const bool g0 = zn < P.zf_lo, t0 = zn > P.zf_hi;
+    float fs = g0 || t0 ? -1.0f : 1.0f;
+    zn = g0 ? -zn : t0 ? 2.0f * P.z_top - zn : zn;
+    if (zn < P.zf_lo || zn > P.zf_hi) {
 #pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-        if (P.reflect_ground && zn < 0.0f) { zn = -zn; fs = -fs; }
-        else if (P.reflect_top && zn > P.z_top) { zn = 2.0f * P.z_top - zn; fs = -fs; }
-        else break;
+        for (int it = 1; it < 4; ++it) {
+            if (P.reflect_ground && zn < 0.0f) { zn = -zn; fs = -fs; }
+            else if (P.reflect_top && zn > P.z_top) { zn = 2.0f * P.z_top - zn; fs = -fs; }
+            else break;
+        }
+        if (P.reflect_ground && zn < 0.0f) { zn = 0.0f; fs = 0.0f; }
+        if (P.reflect_top && zn > P.z_top) { zn = P.z_top; fs = 0.0f; }
     }
-    if (P.reflect_ground && zn < 0.0f) { zn = 0.0f; fs = 0.0f; }
-    if (P.reflect_top && zn > P.z_top) { zn = P.z_top; fs = 0.0f; }
     if (fold) *fold = fs;
     if (EXT && wv) *wv *= fs;            // a reflection reverses the turbulent velocity
     x = xn; y = yn; z = zn;
-    if (!isfinite(xn + yn + zn)) {
-        atomicOr(P.err, ERR_NAN);
-        return ST_EXITED;
-    }
-    // lateral boundary
-    if (P.lateral_exit && (xn < P.x_lo || xn > P.x_hi || yn < P.y_lo || yn > P.y_hi)) {
-        if (GRIDS)
-            atomicAdd(scg->ctr + C_EXITED * P.ctr_stride, to_fixed(mass_at(P, sc, sp, k), sc.scale));
-        return ST_EXITED;
+    // lateral boundary and non-finite positions: one test of the box [fx_lo, fx_hi] x
+    // [fy_lo, fy_hi] x |z| <= 1e30 (the domain, cut at 1e30) clears a particle of both (a NaN
+    // fails it)
+    if (!((xn >= P.fx_lo) & (xn <= P.fx_hi) & (yn >= P.fy_lo) & (yn <= P.fy_hi) &
+          (fabsf(zn) <= 1e30f))) {
+        if (!isfinite(xn + yn + zn)) {
+            atomicOr(P.err, ERR_NAN);
+            return ST_EXITED;
+        }
+        if (P.lateral_exit && (xn < P.x_lo || xn > P.x_hi || yn < P.y_lo || yn > P.y_hi)) {
+            if (GRIDS)
+                atomicAdd(scg->ctr + C_EXITED * P.ctr_stride, to_fixed(mass_at(P, sc, sp, k), sc.scale));
+            return ST_EXITED;
+        }
     }
     if (!(P.t_dry | P.t_wet)) return ST_ACTIVE;
     // 6. dry deposition below the mixing height, then wet where it rains
     uint32_t w_dry, w_wet;
     dep_words(P, gid, k, dc, w_dry, w_wet);
+    if (!((w_dry < P.t_dry) | (w_wet < P.t_wet))) return ST_ACTIVE;
     int kind = -1;
     if (w_dry < P.t_dry && zn < P.h_mix) kind = 0;
     if (kind < 0 && w_wet < P.t_wet && P.rain) {
@@ -457,20 +485,27 @@ struct MinBlocks {
     static constexpr int value = per_sm_threads / BLOCK > 0 ? per_sm_threads / BLOCK : 1;
 };
 
-// Advance: each thread keeps PPT particles in registers and runs steps [k0, k1) over the
+// Advance: each thread keeps a particle in registers and runs steps [k0, k1) over the
 // launch's tiles (Ranges): sorted tiles of A and release-ordered tiles of B, handed out by
-// block index (grid over all tiles) or by an atomic queue (persistent grid). With MIXED the
-// lanes of a tile may belong to different scenarios (the sorted particles of a batched
-// context): each lane finds its scenario from its home slot and carries its own wind
-// offset; the results are bit-identical to the per-scenario path. EXT adds, as uniform
-// run-time options, the dosage samples (every P.dose_every steps) inside the time loop,
-// K_z from Eq. 3 (P.blpair), the daughters of a decay chain (P.n_species > 1), the
-// Langevin variant and the scenarios' perturbation modes (P.n_modes > 0); MODES without
-// EXT carries the modes alone. The default instantiations carry none of that code.
-template <int BLOCK, int PPT, int OCC, bool MIXED, bool EXT, bool MODES>
+// block index (grid over all tiles) or by an atomic queue (persistent grid); a tile holds ppt
+// particles per thread, one after the other. With MIXED the lanes of a tile may belong to
+// different scenarios (the sorted particles of a batched context): each lane finds its
+// scenario from its home slot and carries its own wind offset; the results are bit-identical
+// to the per-scenario path. EXT adds, as uniform run-time options, the dosage samples (every
+// P.dose_every steps) inside the time loop, K_z from Eq. 3 (P.blpair), the daughters of a
+// decay chain (P.n_species > 1), the Langevin variant and the scenarios' perturbation modes
+// (P.n_modes > 0); MODES without EXT carries the modes alone. The default instantiations
+// carry none of that code.
+//
+// Bound by issued instructions (32 warps an SM keep the schedulers 75 % busy, DRAM idle), so
+// the step is kept short of branches and constant loads. A lane's time loop starts at its own
+// release step and ends with the particle: no status is tested inside it, and the lanes of a
+// tile of late releases all work from the loop's first turn. (The dosage samples gather a
+// warp's lanes at the same step, so with them the loop runs over common steps.)
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
 __global__ void __launch_bounds__(BLOCK, (MinBlocks<BLOCK, OCC>::value))
 advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *queue, int k0,
-               int k1, int do_bin)
+               int k1, int do_bin, int ppt)
 {
     extern __shared__ float4 s_adv_dyn[];            // the level table, sized by the launch
     __shared__ unsigned long long s_acc[BLOCK];
@@ -479,18 +514,13 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
     const Levels LV = load_levels(P, reinterpret_cast<unsigned char *>(s_adv_dyn));
     unsigned long long *s_warp = s_acc + (threadIdx.x & ~31);
     const long long n_cells = (long long)P.cx * P.cy * P.cz;
-    constexpr int TILE = BLOCK * PPT;
     // the uniform horizontal diffusivity gives one displacement scale for the run
     const float sig_h_uniform = sqrtf(2.0f * P.k_scale * fmaxf(P.kh_uniform, 0.0f) * P.dt);
     // the launch's step times (the first barrier of the tile loop publishes them)
-    __shared__ float4 s_ta[STEP_TAB];
-    __shared__ float2 s_tb[STEP_TAB];
+    __shared__ StepTable s_tab;
     const int n_tab = min(k1 - k0, STEP_TAB);
-    for (int i = threadIdx.x; i < n_tab; i += BLOCK) {
-        const StepTime T = step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k0 + i);
-        s_ta[i] = make_float4(__int_as_float(T.ts.h0), T.ts.f, T.tk, __int_as_float(T.ts.h1));
-        s_tb[i] = make_float2(T.du, T.dv);
-    }
+    for (int i = threadIdx.x; i < n_tab; i += BLOCK)
+        step_table_set(s_tab, i, step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k0 + i));
 
     int iter = 0;
     for (;;) {
@@ -510,8 +540,8 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
         int count, tscen;
         if (in_a) {
             state = R.state_a;
-            first = (long long)t * TILE;
-            count = (int)max(0LL, min((long long)TILE, (long long)*R.a_live - first));
+            first = (long long)t * BLOCK * ppt;
+            count = (int)max(0LL, min((long long)BLOCK * ppt, (long long)*R.a_live - first));
             tscen = 0;
         } else {
             const Tile tl = R.b_tiles[R.b_first + (t - R.tiles_a)];
@@ -525,218 +555,147 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
         }
         if (count <= 0) continue;                       // the whole block skips
         const ScenDev &scg = P.scen[tscen];
-        const ScenDev sc = scg;                         // (unused when MIXED)
 
-        // ---- load particles ---------------------------------------------------------
-        float x[PPT], y[PPT], z[PPT];
-        uint32_t tag[PPT];
-        unsigned long long gid[PPT];
-        int sj[PPT];                                    // scenario of each particle (MIXED)
-        float wv[PPT];                                  // Langevin w' (EXT)
-        float *wsrc = in_a ? R.w_a : R.w_b;
-        const bool lang = EXT && P.langevin && wsrc;
-        const bool modes = MODES && P.n_modes > 0 && P.mode_sc;
-        int live = 0;
-#pragma unroll
-        for (int j = 0; j < PPT; ++j) {
+#pragma unroll 1
+        for (int j = 0; j < ppt; ++j) {
+            // ---- load the particle ------------------------------------------------------
             const int local = j * BLOCK + threadIdx.x;
             const long long slot = first + local;
-            sj[j] = tscen;
-            gid[j] = 0ull;
+            float *wsrc = in_a ? R.w_a : R.w_b;
+            const bool lang = EXT && P.langevin && wsrc;
+            const bool modes = MODES && P.n_modes > 0 && P.mode_sc;
+            float x = 0.0f, y = 0.0f, z = 0.0f, wv = 0.0f;   // wv: Langevin w' (EXT)
+            uint32_t st = ST_EXITED;
+            int sp = 0, sj = tscen;                          // sj: scenario of the particle
+            unsigned long long gid = 0ull;
             if (local < count) {
                 long long home = in_a ? (long long)__ldg(R.pidx + slot) : slot;
                 if (!LPM_IN_BOUNDS(P.err, home >= 0 && home < P.slot_cap)) home = 0;
-                if (MIXED) {
-                    if (in_a) sj[j] = scen_of(P, home);
-                    if (!LPM_IN_BOUNDS(P.err, sj[j] >= 0 && sj[j] < P.n_scen)) sj[j] = 0;
-                    const ScenDev &q = P.scen[sj[j]];
-                    gid[j] = (unsigned long long)(__ldg(&q.id0) + (home - __ldg(&q.first_slot)));
-                } else {
-                    gid[j] = (unsigned long long)(sc.id0 + (home - sc.first_slot));
-                }
+                if (MIXED && in_a) sj = scen_of(P, home);
+                if (MIXED && !LPM_IN_BOUNDS(P.err, sj >= 0 && sj < P.n_scen)) sj = 0;
+                const ScenDev &q = P.scen[sj];
+                gid = (unsigned long long)(__ldg(&q.id0) + (home - __ldg(&q.first_slot)));
                 const float4 s = state[slot];
-                x[j] = s.x; y[j] = s.y; z[j] = s.z;
-                tag[j] = __float_as_uint(s.w);
-                wv[j] = lang ? wsrc[slot] : 0.0f;
-                const uint32_t st = tag[j] >> TAG_SHIFT;
-                const int sp = (int)(tag[j] & TAG_STEP);
-                if (st == ST_ACTIVE || (st == ST_UNRELEASED && sp < k1)) ++live;
-            } else {
-                x[j] = y[j] = z[j] = 0.0f;
-                tag[j] = ST_EXITED << TAG_SHIFT;
-                wv[j] = 0.0f;
+                x = s.x; y = s.y; z = s.z;
+                const uint32_t tag = __float_as_uint(s.w);
+                st = tag >> TAG_SHIFT;
+                sp = (int)(tag & TAG_STEP);
+                wv = lang ? wsrc[slot] : 0.0f;
             }
-        }
+            const ScenDev &sc = P.scen[sj];
+            const float *msc = modes ? P.mode_sc + 8 * sj : nullptr;
 
-        // ---- time loop --------------------------------------------------------------
-        unsigned long long steps = 0;
-        unsigned int nst[PPT];                          // active steps per particle (MIXED)
-        float2 o0[PPT], o1[PPT];                        // lane wind offsets at h0, h1 (MIXED)
-        DepCache dc[PPT];                               // odd-step deposition words
-        int cur_h = -1;
-#pragma unroll
-        for (int j = 0; j < PPT; ++j) {
-            nst[j] = 0u;
-            o0[j] = o1[j] = make_float2(0.0f, 0.0f);
-            dc[j].pair = -1;
-        }
+            // ---- time loop --------------------------------------------------------------
+            unsigned int steps = 0u;                        // active steps of this particle
+            float2 o0 = make_float2(0.f, 0.f), o1 = o0;     // wind offsets at h0, h1 (MIXED)
+            int cur_h = -1;
+            DepCache dc;                                    // odd-step deposition words
+            dc.pair = -1;
+            int k = k0;
+            if (st == ST_UNRELEASED && sp >= k0 && sp < k1) {
+                x = __ldg(&sc.src_x); y = __ldg(&sc.src_y); z = __ldg(&sc.src_z);
+                st = ST_ACTIVE;
+                k = sp;
+            }
+            auto advance = [&](int k) {
+                const StepTime T = k - k0 < n_tab
+                                       ? step_time_tab(P, s_tab, k - k0, k)
+                                       : step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k);
+                float du = T.du, dv = T.dv;
+                if (MIXED && P.woff) {
+                    if (T.ts.h0 != cur_h) {
+                        cur_h = T.ts.h0;
+                        const float2 *w = P.woff + (long long)sj * P.n_t;
+                        o0 = __ldg(w + T.ts.h0);
+                        o1 = __ldg(w + T.ts.h1);
+                    }
+                    // the same expression as step_time's, so sorting changes no bit
+                    du = P.bias_u + fmaf(T.ts.f, o1.x - o0.x, o0.x);
+                    dv = P.bias_v + fmaf(T.ts.f, o1.y - o0.y, o0.y);
+                }
+                ++steps;
+                st = particle_step<true, EXT, Levels, MODES>(P, LV, T, sc, &sc, gid, sp,
+                                                             sig_h_uniform, du, dv, x, y, z,
+                                                             nullptr, lang ? &wv : nullptr, msc,
+                                                             &dc);
+            };
+            if (!EXT || !P.dose_every) {
 #pragma unroll 1
-        for (int k = k0; k < k1; ++k) {
-            if (EXT && P.dose_every) {
-                // with dosage sampling the warp stays together (the samples are warp-collective)
-                if (!__any_sync(0xffffffffu, live > 0)) break;
-            } else if (live <= 0) {
-                break;
-            }
-            const StepTime T = k - k0 < n_tab
-                                   ? step_time_tab(P, s_ta, s_tb, k - k0, k)
-                                   : step_time(P, MIXED ? nullptr : sc.wind_offset, k);
-            if (MIXED && P.woff && T.ts.h0 != cur_h) {
-                cur_h = T.ts.h0;
-#pragma unroll
-                for (int j = 0; j < PPT; ++j) {
-                    const float2 *w = P.woff + (long long)sj[j] * P.n_t;
-                    o0[j] = __ldg(w + T.ts.h0);
-                    o1[j] = __ldg(w + T.ts.h1);
-                }
-            }
-            live = 0;
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                uint32_t st = tag[j] >> TAG_SHIFT;
-                const int sp = (int)(tag[j] & TAG_STEP);
-                if (st == ST_UNRELEASED && sp == k) {
-                    st = ST_ACTIVE;
-                    if (MIXED) {
-                        const ScenDev &q = P.scen[sj[j]];
-                        x[j] = __ldg(&q.src_x); y[j] = __ldg(&q.src_y); z[j] = __ldg(&q.src_z);
-                    } else {
-                        x[j] = sc.src_x; y[j] = sc.src_y; z[j] = sc.src_z;
-                    }
-                }
-                if (st != ST_ACTIVE) {
-                    if (st == ST_UNRELEASED && sp < k1) ++live;
-                    continue;
-                }
-                if (MIXED) {
-                    ++nst[j];
-                    float du = T.du, dv = T.dv;
-                    if (P.woff) {
-                        // the same expression as step_time's, so sorting changes no bit
-                        du = P.bias_u + fmaf(T.ts.f, o1[j].x - o0[j].x, o0[j].x);
-                        dv = P.bias_v + fmaf(T.ts.f, o1[j].y - o0[j].y, o0[j].y);
-                    }
-                    st = particle_step<true, EXT, Levels, MODES>(P, LV, T, P.scen[sj[j]], P.scen + sj[j], gid[j],
-                                                  sp, sig_h_uniform, du, dv, x[j], y[j], z[j],
-                                                  nullptr, lang ? &wv[j] : nullptr,
-                                                  modes ? P.mode_sc + 8 * sj[j] : nullptr, &dc[j]);
-                } else {
-                    ++steps;
-                    st = particle_step<true, EXT, Levels, MODES>(P, LV, T, sc, &scg, gid[j], sp, sig_h_uniform,
-                                                  T.du, T.dv, x[j], y[j], z[j], nullptr,
-                                                  lang ? &wv[j] : nullptr,
-                                                  modes ? P.mode_sc + 8 * tscen : nullptr, &dc[j]);
-                }
-                tag[j] = (st << TAG_SHIFT) | (uint32_t)sp;
-                if (st == ST_ACTIVE) ++live;
-            }
-            // time-integrated dosage: every dose_every-th step, the decayed masses at t_{k+1}
-            if (EXT && P.dose_every && (k + 1) % P.dose_every == 0) {
-#pragma unroll
-                for (int j = 0; j < PPT; ++j) {
-                    const int local = j * BLOCK + threadIdx.x;
-                    const bool on = local < count && (tag[j] >> TAG_SHIFT) == ST_ACTIVE;
-                    const int sp = (int)(tag[j] & TAG_STEP);
-                    const int cell = on ? grid_cell(P, x[j], y[j], z[j]) : KEY_NONE;
-                    unsigned long long v = 0ull;
-                    if (on) {
+                for (; st == ST_ACTIVE && k < k1; ++k) advance(k);
+            } else {
+                const int k_own = k;                        // this lane's first step
+#pragma unroll 1
+                for (k = k0; k < k1; ++k) {
+                    // the samples are warp-collective: the warp stays together
+                    if (!__any_sync(0xffffffffu, st == ST_ACTIVE)) break;
+                    if (st == ST_ACTIVE && k >= k_own) advance(k);
+                    // every dose_every-th step, the decayed masses at t_{k+1}
+                    if ((k + 1) % P.dose_every == 0) {
+                        const bool on = st == ST_ACTIVE && k >= k_own;
+                        const int cell = on ? grid_cell(P, x, y, z) : KEY_NONE;
+                        unsigned long long v = 0ull;
+                        if (on) v = to_fixed(mass_at(P, sc, sp, k), __ldg(&sc.scale) * P.dose_mul);
                         if (MIXED) {
-                            const ScenDev &q = P.scen[sj[j]];
-                            v = to_fixed(mass_at(P, q, sp, k), __ldg(&q.scale) * P.dose_mul);
+                            long long key = -1;
+                            if (on) key = cell >= 0 ? (long long)sj * n_cells + cell : -2LL - sj;
+                            warp_accumulate_scen(key, v, P, P.dose_all, C_DOSE_OUT, s_warp, n_cells);
                         } else {
-                            v = to_fixed(mass_at(P, sc, sp, k), sc.scale * P.dose_mul);
+                            warp_accumulate(cell, v, P.dose_all + (long long)tscen * n_cells,
+                                            scg.ctr + C_DOSE_OUT * P.ctr_stride, s_warp, n_cells,
+                                            P.err);
                         }
                     }
-                    if (MIXED) {
-                        long long key = -1;
-                        if (on) key = cell >= 0 ? (long long)sj[j] * n_cells + cell : -2LL - sj[j];
-                        warp_accumulate_scen(key, v, P, P.dose_all, C_DOSE_OUT, s_warp, n_cells);
-                    } else {
-                        warp_accumulate(cell, v, P.dose_all + (long long)tscen * n_cells,
-                                        scg.ctr + C_DOSE_OUT * P.ctr_stride, s_warp, n_cells,
-                                        P.err);
-                    }
                 }
             }
-        }
 
-        // ---- store ------------------------------------------------------------------
-#pragma unroll
-        for (int j = 0; j < PPT; ++j) {
-            const int local = j * BLOCK + threadIdx.x;
+            // ---- store ------------------------------------------------------------------
+            const bool on = local < count && st == ST_ACTIVE;
             if (local < count) {
-                state[first + local] = make_float4(x[j], y[j], z[j], __uint_as_float(tag[j]));
+                state[first + local] = make_float4(x, y, z, __uint_as_float((st << TAG_SHIFT) |
+                                                                            (uint32_t)sp));
                 // only a moving particle has a turbulent velocity (0 once deposited or
                 // exited, and before its release)
-                if (lang) wsrc[first + local] = (tag[j] >> TAG_SHIFT) == ST_ACTIVE ? wv[j] : 0.0f;
+                if (lang) wsrc[first + local] = on ? wv : 0.0f;
             }
-        }
 
-        // ---- sort keys for the sort that follows (its inputs: A slots, then B lanes) ----
-        if (R.keys) {
-            const unsigned int dead_key = (unsigned int)sort_key_range(P.nx, P.ny, P.nz);
-            const int lane = threadIdx.x & 31;
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                const int local = j * BLOCK + threadIdx.x;
+            // ---- sort keys for the sort that follows (its inputs: A slots, then B lanes) ----
+            if (R.keys) {
+                const unsigned int dead_key = (unsigned int)sort_key_range(P.nx, P.ny, P.nz);
+                const int lane = threadIdx.x & 31;
                 long long idx = -1;
                 unsigned int key = KEY_NONE_U;
                 if (in_a) {
                     if (local < count) idx = first + local;
                 } else {
-                    idx = (long long)*R.a_live + (long long)(t - R.tiles_a) * TILE + local;
+                    idx = (long long)*R.a_live + (long long)(t - R.tiles_a) * BLOCK * ppt + local;
                 }
-                if (local < count) {
-                    if ((tag[j] >> TAG_SHIFT) == ST_ACTIVE) {
-                        int ix, jy, kz;
-                        float fa, fb, fc;
-                        axis(x[j], P.x0, P.inv_dx, P.nx, ix, fa);
-                        axis(y[j], P.y0, P.inv_dy, P.ny, jy, fb);
-                        level(P, LV, z[j], kz, fc);
-                        key = cell_key(P, ix, jy, kz);
-                    } else {
-                        key = dead_key;
-                    }
+                if (on) {
+                    int ix, jy, kz;
+                    float fa, fb, fc;
+                    axis(x, P.x0, P.inv_dx, P.nx, ix, fa);
+                    axis(y, P.y0, P.inv_dy, P.ny, jy, fb);
+                    level(P, LV, z, kz, fc);
+                    key = cell_key(P, ix, jy, kz);
+                } else if (local < count) {
+                    key = dead_key;
                 }
                 if (idx >= 0) R.keys[idx] = key;
                 const unsigned int peers = __match_any_sync(0xffffffffu, key);
                 if (key != KEY_NONE_U && lane == __ffs(peers) - 1)
                     atomicAdd(R.hist + key, (unsigned int)__popc(peers));
             }
-        }
 
-        // ---- end-of-segment concentration snapshot (every n-th step, Sec. 3.2) --------
-        if (do_bin) {
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                const int local = j * BLOCK + threadIdx.x;
-                const uint32_t st = tag[j] >> TAG_SHIFT;
-                const bool on = local < count && st == ST_ACTIVE;
+            // ---- end-of-segment concentration snapshot (every n-th step, Sec. 3.2) --------
+            if (do_bin) {
                 int cell = KEY_NONE;
                 unsigned long long v = 0ull;
                 if (on) {
-                    const int sp = (int)(tag[j] & TAG_STEP);
-                    if (MIXED) {
-                        const ScenDev &q = P.scen[sj[j]];
-                        v = to_fixed(mass_at(P, q, sp, k1 - 1), __ldg(&q.scale));
-                    } else {
-                        v = to_fixed(mass_at(P, sc, sp, k1 - 1), sc.scale);
-                    }
-                    cell = grid_cell(P, x[j], y[j], z[j]);
+                    v = to_fixed(mass_at(P, sc, sp, k1 - 1), __ldg(&sc.scale));
+                    cell = grid_cell(P, x, y, z);
                 }
                 if (MIXED) {
                     long long key = -1;
-                    if (on) key = cell >= 0 ? (long long)sj[j] * n_cells + cell : -2LL - sj[j];
+                    if (on) key = cell >= 0 ? (long long)sj * n_cells + cell : -2LL - sj;
                     warp_accumulate_scen(key, v, P, P.conc_all, C_BIN_OUT, s_warp, n_cells);
                 } else {
                     warp_accumulate(cell, v, scg.conc, scg.ctr + C_BIN_OUT * P.ctr_stride, s_warp,
@@ -746,16 +705,14 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
                 for (int d = 1; EXT && d < P.n_species; ++d) {
                     unsigned long long vd = 0ull;
                     if (on) {
-                        const int sp = (int)(tag[j] & TAG_STEP);
-                        const ScenDev &q = MIXED ? P.scen[sj[j]] : scg;
-                        const float m0 = m0_of(P, q, sp);
+                        const float m0 = m0_of(P, sc, sp);
                         vd = to_fixed(m0 * chain_amount(P, d, (float)(k1 - sp) * P.dt),
-                                      __ldg(&q.scale));
+                                      __ldg(&sc.scale));
                     }
                     unsigned long long *base = P.sp_conc_all + (long long)(d - 1) * P.n_scen * n_cells;
                     if (MIXED) {
                         long long key = -1;
-                        if (on) key = cell >= 0 ? (long long)sj[j] * n_cells + cell : -2LL - sj[j];
+                        if (on) key = cell >= 0 ? (long long)sj * n_cells + cell : -2LL - sj;
                         warp_accumulate_scen(key, vd, P, base, C_SP_OUT + d - 1, s_warp, n_cells);
                     } else {
                         warp_accumulate(cell, vd, base + (long long)tscen * n_cells,
@@ -764,18 +721,16 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
                     }
                 }
             }
-        }
 
-        // ---- active particle-steps of the tile -----------------------------------------
-        if (MIXED) {
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                const int local = j * BLOCK + threadIdx.x;
-                warp_count_scen(local < count ? sj[j] : -1, nst[j], C_ACTIVE_STEPS, P, s_warp);
+            // ---- active particle-steps --------------------------------------------------
+            if (MIXED) {
+                warp_count_scen(local < count ? sj : -1, steps, C_ACTIVE_STEPS, P, s_warp);
+            } else {
+                const unsigned int sum = __reduce_add_sync(0xffffffffu, steps);
+                if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&s_steps, (unsigned long long)sum);
             }
-        } else {
-            for (int o = 16; o > 0; o >>= 1) steps += __shfl_xor_sync(0xffffffffu, steps, o);
-            if ((threadIdx.x & 31) == 0 && steps) atomicAdd(&s_steps, steps);
+        }
+        if (!MIXED) {
             __syncthreads();
             if (threadIdx.x == 0 && s_steps)
                 atomicAdd(scg.ctr + C_ACTIVE_STEPS * P.ctr_stride, s_steps);
@@ -783,73 +738,66 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
     }
 }
 
-template <int BLOCK, int PPT, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
 void adv_prefer_l1()
 {
     // the kernel needs a few KB of shared memory per block: ask for a small carve-out so the
     // rest of the SM's unified L1 serves the weather gathers (measured +0.7 to +1.7 %)
-    cudaFuncSetAttribute(advance_kernel<BLOCK, PPT, OCC, MIXED, EXT, MODES>,
+    cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES>,
                          cudaFuncAttributePreferredSharedMemoryCarveout, 10);
     (void)cudaGetLastError();
 }
 
-template <int BLOCK, int PPT, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
 cudaError_t launch_adv(const AdvanceLaunch &L)
 {
     static std::once_flag once;          // per instantiation; contexts may use several threads
-    std::call_once(once, adv_prefer_l1<BLOCK, PPT, OCC, MIXED, EXT, MODES>);
+    std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES>);
     const size_t smem = adv_dyn_smem(L.params->n_lut);
-    advance_kernel<BLOCK, PPT, OCC, MIXED, EXT, MODES><<<L.grid, BLOCK, smem, L.stream>>>(
-        *L.params, L.ranges, L.n_tiles(), L.queue, L.k0, L.k1, L.do_bin);
+    advance_kernel<BLOCK, OCC, MIXED, EXT, MODES><<<L.grid, BLOCK, smem, L.stream>>>(
+        *L.params, L.ranges, L.n_tiles(), L.queue, L.k0, L.k1, L.do_bin, L.ppt);
     return cudaGetLastError();
 }
 
-template <int BLOCK, int PPT, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
 int occ_adv(size_t smem)
 {
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, advance_kernel<BLOCK, PPT, OCC, MIXED, EXT, MODES>, BLOCK, smem);
+        &n, advance_kernel<BLOCK, OCC, MIXED, EXT, MODES>, BLOCK, smem);
     return n;
 }
 
-// (particles per thread, occupancy variant, mixed scenarios, options: 0 none, 1 extended,
-// 2 perturbation modes alone) -> instantiation, for one block size; the extended options
-// and the modes run with 1 particle per thread
-#define LPM_ADV_CASE(FN, BLOCK, PPT, OCC, MIX, EX, ...)                                \
-    case PPT * 1000 + OCC * 100 + MIX * 10 + EX:                                       \
-        return FN<BLOCK, PPT, OCC, (MIX != 0), (EX == 1), (EX != 0)>(__VA_ARGS__);
-#define LPM_ADV_CASES2(FN, BLOCK, PPT, OCC, EX, ...)                                   \
-    LPM_ADV_CASE(FN, BLOCK, PPT, OCC, 0, EX, __VA_ARGS__)                              \
-    LPM_ADV_CASE(FN, BLOCK, PPT, OCC, 1, EX, __VA_ARGS__)
+// (occupancy variant, mixed scenarios, options: 0 none, 1 extended, 2 perturbation modes
+// alone) -> instantiation, for one block size
+#define LPM_ADV_CASE(FN, BLOCK, OCC, MIX, EX, ...)                                     \
+    case OCC * 100 + MIX * 10 + EX:                                                    \
+        return FN<BLOCK, OCC, (MIX != 0), (EX == 1), (EX != 0)>(__VA_ARGS__);
+#define LPM_ADV_CASES2(FN, BLOCK, OCC, EX, ...)                                        \
+    LPM_ADV_CASE(FN, BLOCK, OCC, 0, EX, __VA_ARGS__)                                   \
+    LPM_ADV_CASE(FN, BLOCK, OCC, 1, EX, __VA_ARGS__)
 #define LPM_ADV_CASES(FN, BLOCK, ...)                                                  \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 0, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 1, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 2, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 0, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 1, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 2, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 4, 0, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 4, 1, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 4, 2, 0, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 0, 1, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 1, 1, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 2, 1, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 0, 2, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 1, 2, __VA_ARGS__)                                    \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 2, 2, __VA_ARGS__)
+    LPM_ADV_CASES2(FN, BLOCK, 0, 0, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 1, 0, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 2, 0, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 0, 1, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 1, 1, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 2, 1, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 0, 2, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 1, 2, __VA_ARGS__)                                       \
+    LPM_ADV_CASES2(FN, BLOCK, 2, 2, __VA_ARGS__)
 
 #define LPM_ADVANCE_TU(BLOCK)                                                          \
     cudaError_t launch_advance_b##BLOCK(const AdvanceLaunch &L)                         \
     {                                                                                  \
-        switch (L.ppt * 1000 + L.occ * 100 + (L.mixed ? 10 : 0) + L.variant()) {       \
+        switch (L.occ * 100 + (L.mixed ? 10 : 0) + L.variant()) {                      \
             LPM_ADV_CASES(launch_adv, BLOCK, L)                                        \
         }                                                                              \
         return cudaErrorInvalidValue;                                                  \
     }                                                                                  \
-    int occupancy_b##BLOCK(int ppt, int occ, bool mixed, int variant, size_t smem)     \
+    int occupancy_b##BLOCK(int occ, bool mixed, int variant, size_t smem)              \
     {                                                                                  \
-        switch (ppt * 1000 + occ * 100 + (mixed ? 10 : 0) + variant) {                 \
+        switch (occ * 100 + (mixed ? 10 : 0) + variant) {                              \
             LPM_ADV_CASES(occ_adv, BLOCK, smem)                                        \
         }                                                                              \
         return 0;                                                                      \

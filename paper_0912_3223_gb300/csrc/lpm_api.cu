@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <string>
 #include <vector>
 #include <algorithm>
@@ -351,6 +352,13 @@ void fill_params(const lpm_ctx *c, StepParams &P)
     P.reflect_top = g.reflect_top;
     P.lateral_exit = g.lateral_exit;
     P.drift = g.drift_correction;
+    const float inf = std::numeric_limits<float>::infinity();
+    P.zf_lo = g.reflect_ground ? 0.0f : -inf;
+    P.zf_hi = g.reflect_top ? P.z_top : inf;
+    P.fx_lo = g.lateral_exit ? std::max(P.x_lo, -1e30f) : -1e30f;
+    P.fx_hi = g.lateral_exit ? std::min(P.x_hi, 1e30f) : 1e30f;
+    P.fy_lo = g.lateral_exit ? std::max(P.y_lo, -1e30f) : -1e30f;
+    P.fy_hi = g.lateral_exit ? std::min(P.y_hi, 1e30f) : 1e30f;
     P.cx = g.cx; P.cy = g.cy; P.cz = g.cz;
     P.gx0 = g.cx0; P.gy0 = g.cy0; P.gz0 = g.cz0;
     P.ginv_dx = 1.0 / g.cdx; P.ginv_dy = 1.0 / g.cdy; P.ginv_dz = 1.0 / g.cdz;
@@ -1397,7 +1405,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
         const bool ext_opts = P.dose_every > 0 || P.blpair != nullptr || P.n_species > 1 ||
                               P.langevin;
         const int occ_blocks = std::max(1, advance_occupancy(
-            c->block, c->ppt, c->occ, false, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
+            c->block, c->occ, false, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
             adv_dyn_smem(P.n_lut)));
         st = run_segments(c, P, plan, c->stream, c->sorted_upto, c->cur, kernels, true,
                           occ_blocks);
@@ -1418,7 +1426,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
             const bool ext_opts = P.dose_every > 0 || P.blpair != nullptr || P.n_species > 1 ||
                                   P.langevin;
             const int occ_blocks = std::max(1, advance_occupancy(
-                c->block, c->ppt, c->occ, true, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
+                c->block, c->occ, true, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
                 adv_dyn_smem(P.n_lut)));
             lpm_ctx::Graph ng{};
             ng.k0 = c->k;

@@ -140,13 +140,13 @@ inline size_t adv_dyn_smem(int n_lut)
 }
 
 cudaError_t launch_advance(const AdvanceLaunch &L);
-int advance_occupancy(int block, int ppt, int occ, bool mixed, int variant, size_t smem);
+int advance_occupancy(int block, int occ, bool mixed, int variant, size_t smem);
 cudaError_t launch_advance_b128(const AdvanceLaunch &L);
 cudaError_t launch_advance_b256(const AdvanceLaunch &L);
 cudaError_t launch_advance_b512(const AdvanceLaunch &L);
-int occupancy_b128(int ppt, int occ, bool mixed, int variant, size_t smem);
-int occupancy_b256(int ppt, int occ, bool mixed, int variant, size_t smem);
-int occupancy_b512(int ppt, int occ, bool mixed, int variant, size_t smem);
+int occupancy_b128(int occ, bool mixed, int variant, size_t smem);
+int occupancy_b256(int occ, bool mixed, int variant, size_t smem);
+int occupancy_b512(int occ, bool mixed, int variant, size_t smem);
 cudaError_t launch_pack(cudaStream_t s, const float4 *a, const float4 *b, const float *ka,
                         const float *kb, float4 *pair, float2 *khpair, int nx, int ny, int nz);
 cudaError_t launch_sort(cudaStream_t s, const StepParams &P, const SortSource &in,
