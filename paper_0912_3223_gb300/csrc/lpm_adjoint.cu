@@ -30,35 +30,37 @@ __device__ __forceinline__ void sample_met_grad(const StepParams &P, const LEV &
 {
     int i, j, k;
     float a, b, c;
-    axis(x, P.x0, P.inv_dx, P.nx, i, a);
-    axis(y, P.y0, P.inv_dy, P.ny, j, b);
+    axis(x, P.x0, P.inv_dx, P.nx2, i, a);
+    axis(y, P.y0, P.inv_dy, P.ny2, j, b);
     level(P, L, z, k, c);
     const float fx = (x - P.x0) * P.inv_dx, fy = (y - P.y0) * P.inv_dy;
     const float gx = (fx >= 0.0f && fx <= (float)(P.nx - 1)) ? P.inv_dx : 0.0f;
-    const float gy = (fy >= 0.0f && fy <= (float)(P.ny - 1)) ? P.inv_dy : 0.0f;
-    const float gz = (z >= L.z_lo && z <= L.z_hi) ? level_entry(P, L, k).y : 0.0f;
-    const int n00 = col_node(P, i, j, k);
-    float4 q[8];
+    const float gy0 = (fy >= 0.0f && fy <= (float)(P.ny - 1)) ? P.inv_dy : 0.0f;
+    const float gz0 = (z >= L.z_lo && z <= L.z_hi) ? level_entry(P, L, k).y : 0.0f;
+    const Corners q = cell_corners(P, i, j, k, b, c);
+    const F2 ff = pack2(T.f, T.f), aa = pack2(a, a), bb = pack2(q.b, q.b), cc = pack2(q.c, q.c);
+    Rec4 yl[2], dx[2], dy[2];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        const int off = corner_off(P, m);
-        float4 lo, dt;
-        ld_pair(T.pair + 2 * (n00 + off), lo, dt);
-        q[m] = tlerp4(lo, dt, T.ts.f);
+    for (int l = 0; l < 2; ++l) {
+        Rec4 xr[2], df[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const float4 *p = record_at<32>(T.pair, q.rec[2 * l + m]);
+            const Rec4 v0 = ld_blend(p, ff), v1 = ld_blend(p + 8, ff);
+            df[m] = sub4(v1, v0);
+            xr[m] = lerp4(v0, v1, aa);
+        }
+        yl[l] = lerp4s(xr[0], xr[1], bb, q.sy);
+        dx[l] = lerp4s(df[0], df[1], bb, q.sy);
+        dy[l] = sub4(xr[1], xr[0]);
     }
-    const float4 x00 = lerp4(q[0], q[1], a), x10 = lerp4(q[2], q[3], a);
-    const float4 x01 = lerp4(q[4], q[5], a), x11 = lerp4(q[6], q[7], a);
-    const float4 y0 = lerp4(x00, x10, b), y1 = lerp4(x01, x11, b);
-    const float4 r = lerp4(y0, y1, c);
-    // d/dx: x-differences blended in y and z; d/dy: y-differences blended in z
-    float4 dx0 = lerp4(make_float4(q[1].x - q[0].x, q[1].y - q[0].y, q[1].z - q[0].z, q[1].w - q[0].w),
-                       make_float4(q[3].x - q[2].x, q[3].y - q[2].y, q[3].z - q[2].z, q[3].w - q[2].w), b);
-    float4 dx1 = lerp4(make_float4(q[5].x - q[4].x, q[5].y - q[4].y, q[5].z - q[4].z, q[5].w - q[4].w),
-                       make_float4(q[7].x - q[6].x, q[7].y - q[6].y, q[7].z - q[6].z, q[7].w - q[6].w), b);
-    const float4 ddx = lerp4(dx0, dx1, c);
-    const float4 ddy = lerp4(make_float4(x10.x - x00.x, x10.y - x00.y, x10.z - x00.z, x10.w - x00.w),
-                             make_float4(x11.x - x01.x, x11.y - x01.y, x11.z - x01.z, x11.w - x01.w), c);
-    const float4 ddz = make_float4(y1.x - y0.x, y1.y - y0.y, y1.z - y0.z, y1.w - y0.w);
+    const float4 r = unpack4(lerp4s(yl[0], yl[1], cc, q.sz));
+    // d/dx: x-differences blended in y and z; d/dy: y-differences blended in z; a swapped
+    // axis negates its differences (exactly), and so does its sign here
+    const float4 ddx = unpack4(lerp4s(dx[0], dx[1], cc, q.sz));
+    const float4 ddy = unpack4(lerp4s(dy[0], dy[1], cc, q.sz));
+    const float4 ddz = unpack4(sub4(yl[1], yl[0]));
+    const float gy = q.sy ? -gy0 : gy0, gz = q.sz ? -gz0 : gz0;
     val[0] = r.x; val[1] = r.y; val[2] = r.z; val[3] = r.w;
     g[0][0] = ddx.x * gx; g[0][1] = ddy.x * gy; g[0][2] = ddz.x * gz;
     g[1][0] = ddx.y * gx; g[1][1] = ddy.y * gy; g[1][2] = ddz.y * gz;
@@ -68,23 +70,28 @@ __device__ __forceinline__ void sample_met_grad(const StepParams &P, const LEV &
         val[3] = 0.0f;
         g[3][0] = g[3][1] = g[3][2] = 0.0f;
     }
-    if (KHG && T.khp) {
-        float e[8];
+    if (KHG && P.khpair) {
+        const float2 *khp = P.khpair + (long long)T.h0 * P.slab;
+        float ey[2], lx[2], dk[2];
 #pragma unroll
-        for (int mm = 0; mm < 8; ++mm) {
-            const int off = corner_off(P, mm);
-            const float2 v = __ldg(T.khp + n00 + off);
-            e[mm] = fmaf(T.ts.f, v.y, v.x);
+        for (int l = 0; l < 2; ++l) {
+            float ex[2], de[2];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const float2 *p = record_at<8>(khp, q.rec[2 * l + m]);
+                const float2 v0 = __ldg(p), v1 = __ldg(p + 4);
+                const float e0 = fmaf(T.f, v0.y, v0.x), e1 = fmaf(T.f, v1.y, v1.x);
+                de[m] = e1 - e0;
+                ex[m] = fmaf(a, de[m], e0);
+            }
+            ey[l] = lerps(ex[0], ex[1], q.b, q.sy);
+            lx[l] = lerps(de[0], de[1], q.b, q.sy);
+            dk[l] = ex[1] - ex[0];
         }
-        const float ex0 = fmaf(a, e[1] - e[0], e[0]), ex1 = fmaf(a, e[3] - e[2], e[2]);
-        const float ex2 = fmaf(a, e[5] - e[4], e[4]), ex3 = fmaf(a, e[7] - e[6], e[6]);
-        const float ey0 = fmaf(b, ex1 - ex0, ex0), ey1 = fmaf(b, ex3 - ex2, ex2);
-        val[4] = fmaf(c, ey1 - ey0, ey0);
-        const float l01 = fmaf(b, (e[3] - e[2]) - (e[1] - e[0]), e[1] - e[0]);
-        const float l23 = fmaf(b, (e[7] - e[6]) - (e[5] - e[4]), e[5] - e[4]);
-        g[4][0] = fmaf(c, l23 - l01, l01) * gx;
-        g[4][1] = fmaf(c, (ex3 - ex2) - (ex1 - ex0), ex1 - ex0) * gy;
-        g[4][2] = (ey1 - ey0) * gz;
+        val[4] = lerps(ey[0], ey[1], q.c, q.sz);
+        g[4][0] = lerps(lx[0], lx[1], q.c, q.sz) * gx;
+        g[4][1] = lerps(dk[0], dk[1], q.c, q.sz) * gy;
+        g[4][2] = (ey[1] - ey[0]) * gz;
         if (!(val[4] > 0.0f)) {
             val[4] = 0.0f;
             g[4][0] = g[4][1] = g[4][2] = 0.0f;
@@ -96,36 +103,29 @@ __device__ __forceinline__ void sample_met_grad(const StepParams &P, const LEV &
     (void)sig_h_uniform;
 }
 
-// The time parts of step k (time pair h0 / h1, fraction, t_k) as step_time computes them,
-// packed for a per-block table: the steps of a segment are the same for every particle.
+// The time parts of step k as step_time computes them (without an offset), packed for a
+// per-block table: the steps of a segment are the same for every particle.
 __device__ __forceinline__ float4 step_time_parts(const StepParams &P, int k)
 {
     const StepTime T = step_time(P, nullptr, k);
-    return make_float4(__int_as_float(T.ts.h0), T.ts.f, T.tk, __int_as_float(T.ts.h1));
+    const unsigned long long p = reinterpret_cast<unsigned long long>(T.pair);
+    return make_float4(__uint_as_float((unsigned int)p), __uint_as_float((unsigned int)(p >> 32)),
+                       T.f, __int_as_float(T.h0));
 }
 
-// step_time(P, wind_offset, k) from the packed time parts of step k (the same values: the
-// parts are step_time's own, the pointers and the offset follow its expressions).
+// step_time(P, wind_offset, k) from the packed time parts of step k.
 __device__ __forceinline__ StepTime step_time_from(const StepParams &P, const float2 *wind_offset,
                                                    float4 a, int k)
 {
     StepTime T;
     T.k = k;
-    T.tk = a.z;
-    T.ts.h0 = __float_as_int(a.x);
-    T.ts.h1 = __float_as_int(a.w);
-    T.ts.f = a.y;
-    T.pair = P.pair + (long long)T.ts.h0 * P.slab * 2;
-    T.khp = P.khpair ? P.khpair + (long long)T.ts.h0 * P.slab : nullptr;
-    T.blp = P.blpair ? P.blpair + (long long)T.ts.h0 * P.nx * P.ny * 2 : nullptr;
-    T.du = P.bias_u;
-    T.dv = P.bias_v;
-    if (wind_offset) {
-        const float2 o0 = __ldg(wind_offset + T.ts.h0);
-        const float2 o1 = __ldg(wind_offset + T.ts.h1);
-        T.du += fmaf(T.ts.f, o1.x - o0.x, o0.x);
-        T.dv += fmaf(T.ts.f, o1.y - o0.y, o0.y);
-    }
+    T.pair = reinterpret_cast<const float4 *>((unsigned long long)__float_as_uint(a.x) |
+                                              ((unsigned long long)__float_as_uint(a.y) << 32));
+    T.f = a.z;
+    T.h0 = __float_as_int(a.w);
+    const float2 d = step_offset(P, wind_offset, T.h0, min(T.h0 + 1, P.n_t - 1), T.f);
+    T.du = d.x;
+    T.dv = d.y;
     return T;
 }
 

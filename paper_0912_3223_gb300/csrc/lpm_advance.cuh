@@ -120,96 +120,6 @@ __device__ __forceinline__ void mode_wind(const StepParams &P, const float *msc,
     dv = pz * sv;
 }
 
-// Weather at a point from the time-paired records: 8 spatial corners, each one 32-byte
-// load of (slab h, slab h+1 - slab h), blended in time, then in x, y and z. With the
-// boundary-layer columns (EXT and blp), K_z and its derivative come from Eq. 3 instead
-// (4 more 32-byte loads of the time-paired (u*, 1/L, H_z) at the cell's corner columns,
-// bilinear in x, y); with msc (MODES) the scenario's perturbation modes are added to
-// (u, v). Only the EXT or MODES instantiations carry that code.
-template <bool EXT, class LEV, bool MODES = EXT>
-__device__ __forceinline__ Met sample_met_pair(const StepParams &P, const LEV &L,
-                                               const float4 *__restrict__ pair,
-                                               const float2 *__restrict__ khp,
-                                               const float4 *__restrict__ blp, float f,
-                                               float x, float y, float z, float tk = 0.0f,
-                                               const float *msc = nullptr)
-{
-    int i, j, k;
-    float a, b, c;
-    axis(x, P.x0, P.inv_dx, P.nx, i, a);
-    axis(y, P.y0, P.inv_dy, P.ny, j, b);
-    level(P, L, z, k, c);
-    if (!LPM_IN_BOUNDS(P.err, i >= 0 && i <= P.nx - 2 && j >= 0 && j <= P.ny - 2 && k >= 0 &&
-                                  k <= P.nz - 2))
-        i = j = k = 0;
-    // the corners as two x-adjacent records at four bases: (y, z), (y+1, z), (y, z+1),
-    // (y+1, z+1); the x + 1 record is the next 32 bytes
-    const float4 *b00 = pair + 2 * (long long)col_node(P, i, j, k);
-    const float4 *b10 = b00 + 2 * P.nx;
-    const float4 *b01 = b00 + 2 * (long long)P.nx * P.ny;
-    const float4 *b11 = b01 + 2 * P.nx;
-    const float4 *base[4] = {b00, b10, b01, b11};
-    float4 q[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        float4 lo, dt;
-        ld_pair(base[m >> 1] + 2 * (m & 1), lo, dt);
-        q[m] = tlerp4(lo, dt, f);
-    }
-    const float4 x00 = lerp4(q[0], q[1], a), x10 = lerp4(q[2], q[3], a);
-    const float4 x01 = lerp4(q[4], q[5], a), x11 = lerp4(q[6], q[7], a);
-    const float4 y0 = lerp4(x00, x10, b), y1 = lerp4(x01, x11, b);
-    const float4 r = lerp4(y0, y1, c);
-    Met m;
-    m.u = r.x;
-    m.v = r.y;
-    m.w = r.z;
-    if (MODES && msc) {
-        float du, dv;
-        mode_wind(P, msc, k, c, x, y, tk, du, dv);
-        m.u += du;
-        m.v += dv;
-    }
-    if (EXT && blp) {
-        float4 cq[4];
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) {
-            float4 lo, dt;
-            ld_pair(blp + 2 * ((j + ((mm >> 1) & 1)) * P.nx + i + (mm & 1)), lo, dt);
-            cq[mm] = tlerp4(lo, dt, f);
-        }
-        const float4 c0 = lerp4(cq[0], cq[1], a), c1 = lerp4(cq[2], cq[3], a);
-        const float4 col = lerp4(c0, c1, b);
-        kz_eq3(col.x, col.y, col.z, P.kz_min, z, m.kz, m.dkz);
-    } else {
-        m.kz = fmaxf(r.w, 0.0f);
-        // the vertical derivative only where a drift term reads it (the drift-corrected
-        // walk and the Langevin variant)
-        m.dkz = 0.0f;
-        if (P.drift || (EXT && P.langevin)) {
-            const bool inside = z >= L.z_lo && z <= L.z_hi;
-            m.dkz = inside ? (y1.w - y0.w) * level_entry(P, L, k).y : 0.0f;
-        }
-    }
-    if (khp) {
-        const int n00 = col_node(P, i, j, k);
-        float e[8];
-#pragma unroll
-        for (int mm = 0; mm < 8; ++mm) {
-            const int off = corner_off(P, mm);
-            const float2 v = __ldg(khp + n00 + off);
-            e[mm] = fmaf(f, v.y, v.x);
-        }
-        const float ex0 = fmaf(a, e[1] - e[0], e[0]), ex1 = fmaf(a, e[3] - e[2], e[2]);
-        const float ex2 = fmaf(a, e[5] - e[4], e[4]), ex3 = fmaf(a, e[7] - e[6], e[6]);
-        const float ey0 = fmaf(b, ex1 - ex0, ex0), ey1 = fmaf(b, ex3 - ex2, ex2);
-        m.kh = fmaxf(fmaf(c, ey1 - ey0, ey0), 0.0f);
-    } else {
-        m.kh = 0.0f;
-    }
-    return m;
-}
-
 // Concentration-grid cell of a position, or KEY_OUT outside the grid.
 __device__ __forceinline__ int grid_cell(const StepParams &P, float x, float y, float z)
 {
@@ -252,107 +162,207 @@ static __device__ __noinline__ void deposit_species(const StepParams &P, const S
 
 // The deposition words of a particle: one Philox block (stream 1) serves a pair of steps,
 // words 0 and 1 for the even step, 2 and 3 for the odd one (dry, then wet test). A step
-// runner may keep the odd step's words from the even step in a DepCache.
+// runner may keep the odd step's words from the even step in a DepCache; it has to fill it
+// (dep_begin) before a first step that is odd.
 struct DepCache {
-    uint32_t c, d;                   // words of the odd step of pair `pair`
-    int pair;                        // -1: nothing kept
+    uint32_t c, d;                   // words of the odd step of the current pair
 };
+
+__device__ __forceinline__ U4 dep_block(const StepParams &P, unsigned long long gid, int k)
+{
+    return philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)(k >> 1), 1u, P.rk);
+}
+
+__device__ __forceinline__ void dep_begin(const StepParams &P, unsigned long long gid, int k,
+                                          DepCache &dc)
+{
+    dc.c = dc.d = 0u;
+    if ((P.t_dry | P.t_wet) && (k & 1)) {
+        const U4 w = dep_block(P, gid, k);
+        dc.c = w.c;
+        dc.d = w.d;
+    }
+}
 
 __device__ __forceinline__ void dep_words(const StepParams &P, unsigned long long gid, int k,
                                           DepCache *dc, uint32_t &w_dry, uint32_t &w_wet)
 {
-    const int pair = k >> 1;
-    if (dc && (k & 1) && dc->pair == pair) {
+    const bool odd = (k & 1) != 0;
+    if (dc) {
         w_dry = dc->c;
         w_wet = dc->d;
-        return;
-    }
-    const U4 d = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)pair, 1u, P.rk);
-    if (k & 1) {
-        w_dry = d.c;
-        w_wet = d.d;
-    } else {
-        w_dry = d.a;
-        w_wet = d.b;
-        if (dc) {
-            dc->c = d.c;
-            dc->d = d.d;
-            dc->pair = pair;
+        if (!odd) {
+            const U4 w = dep_block(P, gid, k);
+            w_dry = w.a;
+            w_wet = w.b;
+            dc->c = w.c;
+            dc->d = w.d;
         }
+    } else {
+        const U4 w = dep_block(P, gid, k);
+        w_dry = odd ? w.c : w.a;
+        w_wet = odd ? w.d : w.b;
     }
 }
 
 // Per-step quantities shared by every particle of a tile.
 struct StepTime {
     int k;
-    float tk;                        // t_k
-    TimeSlab ts;
+    int h0;                          // first slab of the time pair (not read by the plain step)
+    float f;                         // fraction between the slabs
     const float4 *pair;              // time pair of the step
-    const float2 *khp;               // K_h time pair or nullptr
-    const float4 *blp;               // boundary-layer column pair or nullptr
     float du, dv;                    // wind offset of the scenario + bias
 };
+
+// The wind offset of (hourly) row `wo` between slabs h0 and h1, plus the bias.
+__device__ __forceinline__ float2 step_offset(const StepParams &P, const float2 *wo, int h0, int h1,
+                                              float f)
+{
+    float2 d = make_float2(P.bias_u, P.bias_v);
+    if (wo) {
+        const float2 o0 = __ldg(wo + h0);
+        const float2 o1 = __ldg(wo + h1);
+        d.x += fmaf(f, o1.x - o0.x, o0.x);
+        d.y += fmaf(f, o1.y - o0.y, o0.y);
+    }
+    return d;
+}
 
 __device__ __forceinline__ StepTime step_time(const StepParams &P, const float2 *wind_offset, int k)
 {
     StepTime T;
     T.k = k;
-    T.tk = (float)k * P.dt;
-    T.ts = time_slab(P, T.tk);
-    if (!LPM_IN_BOUNDS(P.err, T.ts.h0 >= 0 && T.ts.h0 < P.n_pair)) T.ts.h0 = 0;
-    T.pair = P.pair + (long long)T.ts.h0 * P.slab * 2;
-    T.khp = P.khpair ? P.khpair + (long long)T.ts.h0 * P.slab : nullptr;
-    T.blp = P.blpair ? P.blpair + (long long)T.ts.h0 * P.nx * P.ny * 2 : nullptr;
-    T.du = P.bias_u;
-    T.dv = P.bias_v;
-    if (wind_offset) {
-        const float2 o0 = __ldg(wind_offset + T.ts.h0);
-        const float2 o1 = __ldg(wind_offset + T.ts.h1);
-        T.du += fmaf(T.ts.f, o1.x - o0.x, o0.x);
-        T.dv += fmaf(T.ts.f, o1.y - o0.y, o0.y);
-    }
+    TimeSlab ts = time_slab(P, (float)k * P.dt);
+    if (!LPM_IN_BOUNDS(P.err, ts.h0 >= 0 && ts.h0 < P.n_pair)) ts.h0 = 0;
+    T.h0 = ts.h0;
+    T.f = ts.f;
+    T.pair = P.pair + (long long)ts.h0 * P.slab * 2;
+    const float2 d = step_offset(P, wind_offset, ts.h0, ts.h1, ts.f);
+    T.du = d.x;
+    T.dv = d.y;
     return T;
 }
 
-// Step times of a launch are the same for every particle: each block computes those of
-// steps [k0, k0 + STEP_TAB) once with step_time and keeps them in shared memory (the pair's
-// address, fraction and t_k in one 16-byte entry, the offset, the hour); step_time_tab
-// reads a step's StepTime back (measured: the per-particle step_time cost 3.5 % of the step).
-constexpr int STEP_TAB = 128;
-
+// Step times of a launch are the same for every particle: each block computes those of its
+// (at most STEP_TAB) steps once with step_time and keeps them in shared memory, 24 bytes a
+// step; step_time_tab reads one back (measured: the per-particle step_time cost 3.5 % of the
+// step). HOUR: h0 is read too (gridded K_h, Eq. 3 columns, scenarios' wind offsets).
 struct StepTable {
-    float4 a[STEP_TAB];              // pair address (64 bits), f, t_k
-    float2 off[STEP_TAB];            // du, dv
-    int h0[STEP_TAB];
+    float4 a[STEP_TAB];              // pair address (64 bits), f, du
+    float2 b[STEP_TAB];              // dv, h0
 };
 
 __device__ __forceinline__ void step_table_set(StepTable &tab, int i, const StepTime &T)
 {
     const unsigned long long p = reinterpret_cast<unsigned long long>(T.pair);
     tab.a[i] = make_float4(__uint_as_float((unsigned int)p), __uint_as_float((unsigned int)(p >> 32)),
-                           T.ts.f, T.tk);
-    tab.off[i] = make_float2(T.du, T.dv);
-    tab.h0[i] = T.ts.h0;
+                           T.f, T.du);
+    tab.b[i] = make_float2(T.dv, __int_as_float(T.h0));
 }
 
-__device__ __forceinline__ StepTime step_time_tab(const StepParams &P, const StepTable &tab, int i,
-                                                  int k)
+template <bool HOUR>
+__device__ __forceinline__ StepTime step_time_tab(uint32_t tab, int i, int k)
 {
-    const float4 a = tab.a[i];
-    const float2 b = tab.off[i];
+    const float4 a = ld_shared4(tab + 16 * i);
+    const float2 b = ld_shared2(tab + 16 * STEP_TAB + 8 * i);
     StepTime T;
     T.k = k;
-    T.tk = a.w;
-    T.ts.h0 = tab.h0[i];
-    T.ts.h1 = min(T.ts.h0 + 1, P.n_t - 1);
-    T.ts.f = a.z;
+    T.f = a.z;
     T.pair = reinterpret_cast<const float4 *>((unsigned long long)__float_as_uint(a.x) |
                                               ((unsigned long long)__float_as_uint(a.y) << 32));
-    T.khp = P.khpair ? P.khpair + (long long)T.ts.h0 * P.slab : nullptr;
-    T.blp = P.blpair ? P.blpair + (long long)T.ts.h0 * P.nx * P.ny * 2 : nullptr;
-    T.du = b.x;
-    T.dv = b.y;
+    T.du = a.w;
+    T.dv = b.x;
+    T.h0 = HOUR ? __float_as_int(b.y) : 0;
     return T;
+}
+
+// Weather at a point from the time-paired records: 8 spatial corners, each one 32-byte
+// load of (slab h, slab h+1 - slab h), blended in time, then in x, y and z. With the
+// boundary-layer columns (EXT and blp), K_z and its derivative come from Eq. 3 instead
+// (4 more 32-byte loads of the time-paired (u*, 1/L, H_z) at the cell's corner columns,
+// bilinear in x, y); with msc (MODES) the scenario's perturbation modes are added to
+// (u, v). Only the EXT or MODES instantiations carry that code.
+template <bool EXT, class LEV, bool MODES, bool FIELDS>
+__device__ __forceinline__ Met sample_met_pair(const StepParams &P, const LEV &L, const StepTime &T,
+                                               float x, float y, float z, const float *msc)
+{
+    const float4 *pair = T.pair;
+    const float f = T.f;
+    int i, j, k;
+    float a, b, c;
+    axis(x, P.x0, P.inv_dx, P.nx2, i, a);
+    axis(y, P.y0, P.inv_dy, P.ny2, j, b);
+    level(P, L, z, k, c);
+    if (!LPM_IN_BOUNDS(P.err, i >= 0 && i <= P.nx - 2 && j >= 0 && j <= P.ny - 2 && k >= 0 &&
+                                  k <= P.nz - 2))
+        i = j = k = 0;
+    // x first (the x + 1 record is the next line), then the two slots of rows and of levels
+    const Corners q = cell_corners(P, i, j, k, b, c);
+    const F2 ff = pack2(f, f), aa = pack2(a, a), bb = pack2(q.b, q.b);
+    Rec4 yl[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        Rec4 xr[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const float4 *p = record_at<32>(pair, q.rec[2 * l + m]);
+            xr[m] = lerp4(ld_blend(p, ff), ld_blend(p + 8, ff), aa);
+        }
+        yl[l] = lerp4s(xr[0], xr[1], bb, q.sy);
+    }
+    const float4 r = unpack4(lerp4s(yl[0], yl[1], pack2(q.c, q.c), q.sz));
+    Met m;
+    m.u = r.x;
+    m.v = r.y;
+    m.w = r.z;
+    if (MODES && msc) {
+        float du, dv;
+        mode_wind(P, msc, k, c, x, y, (float)T.k * P.dt, du, dv);
+        m.u += du;
+        m.v += dv;
+    }
+    if (EXT && P.blpair) {
+        const float4 *blp = P.blpair + (long long)T.h0 * P.nx * P.ny * 2;
+        const F2 b2 = pack2(b, b);
+        Rec4 xr[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const float4 *p = record_at<32>(blp, (unsigned int)((j + m) * P.nx + i));
+            xr[m] = lerp4(ld_blend(p, ff), ld_blend(p + 2, ff), aa);
+        }
+        const float4 col = unpack4(lerp4(xr[0], xr[1], b2));
+        kz_eq3(col.x, col.y, col.z, P.kz_min, z, m.kz, m.dkz);
+    } else {
+        m.kz = fmaxf(r.w, 0.0f);
+        // the vertical derivative only where a drift term reads it (the drift-corrected
+        // walk and the Langevin variant)
+        m.dkz = 0.0f;
+        if ((FIELDS && P.drift) || (EXT && P.langevin)) {
+            const bool inside = z >= L.z_lo && z <= L.z_hi;
+            const float d = unpack2(sub2(yl[1].zw, yl[0].zw)).y;
+            m.dkz = inside ? (q.sz ? -d : d) * level_entry(P, L, k).y : 0.0f;
+        }
+    }
+    if (FIELDS && P.khpair) {
+        const float2 *khp = P.khpair + (long long)T.h0 * P.slab;
+        float ey[2];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            float ex[2];
+#pragma unroll
+            for (int mm = 0; mm < 2; ++mm) {
+                const float2 *p = record_at<8>(khp, q.rec[2 * l + mm]);
+                const float2 v0 = __ldg(p), v1 = __ldg(p + 4);
+                const float e0 = fmaf(f, v0.y, v0.x), e1 = fmaf(f, v1.y, v1.x);
+                ex[mm] = fmaf(a, e1 - e0, e0);
+            }
+            ey[l] = lerps(ex[0], ex[1], q.b, q.sy);
+        }
+        m.kh = fmaxf(lerps(ey[0], ey[1], q.c, q.sz), 0.0f);
+    } else {
+        m.kh = 0.0f;
+    }
+    return m;
 }
 
 // One step of one active particle (Sec. 3.2 main loop: weather at the old position, K,
@@ -360,7 +370,8 @@ __device__ __forceinline__ StepTime step_time_tab(const StepParams &P, const Ste
 // Updates (x, y, z) and returns the new status. (du, dv) is the wind offset of the
 // particle's scenario plus the bias at t_k. With GRIDS, deposition and exit add their mass
 // to the scenario's grids and counters; *fold receives dz/dz_pre (+-1, 0 when clamped).
-template <bool GRIDS, bool EXT = false, class LEV, bool MODES = EXT>
+// FIELDS: the run may have a gridded K_h or the drift correction (uniform run-time tests).
+template <bool GRIDS, bool EXT = false, class LEV, bool MODES = EXT, bool FIELDS = true>
 __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV &LV,
                                                   const StepTime &T, const ScenDev &sc,
                                                   const ScenDev *scg, unsigned long long gid,
@@ -372,17 +383,17 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
     const int k = T.k;
     // 1. weather at the old position and t_k (with the scenario's perturbation modes: msc);
     // 2. diffusivities
-    const Met m = sample_met_pair<EXT, LEV, MODES>(P, LV, T.pair, T.khp, T.blp, T.ts.f, x, y, z,
-                                                  T.tk, msc);
-    const float sig_h = T.khp ? sqrtf(2.0f * P.k_scale * m.kh * P.dt) : sig_h_uniform;
-    const float sig_z = sqrtf(2.0f * P.k_scale * m.kz * P.dt);
+    const Met m = sample_met_pair<EXT, LEV, MODES, FIELDS>(P, LV, T, x, y, z, msc);
+    const float sig_h = FIELDS && P.khpair ? sqrtf(P.k2 * m.kh * P.dt) : sig_h_uniform;
+    const float sig_z = sqrtf(P.k2 * m.kz * P.dt);
     // 3. N(0,1) draws
     const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
     float n0, n1, n2;
     normals3(w, n0, n1, n2);
     // 4. Eq. (1)-(2): wind then turbulent displacement
-    const float xn = x + (m.u + du) * P.dt + n0 * sig_h;
-    const float yn = y + (m.v + dv) * P.dt + n1 * sig_h;
+    // (fused multiply-adds, written out: every instantiation rounds alike)
+    const float xn = __fmaf_rn(n0, sig_h, __fmaf_rn(m.u + du, P.dt, x));
+    const float yn = __fmaf_rn(n1, sig_h, __fmaf_rn(m.v + dv, P.dt, y));
     float zn;
     if (EXT && wv) {
         // vertical Langevin variant (well-mixed for Gaussian turbulence of variance
@@ -406,8 +417,8 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
         *wv = wp;
         zn = z + (m.w + wp) * P.dt;
     } else {
-        zn = z + m.w * P.dt + n2 * sig_z;
-        if (P.drift) zn += P.k_scale * m.dkz * P.dt;
+        zn = __fmaf_rn(n2, sig_z, __fmaf_rn(m.w, P.dt, z));
+        if (FIELDS && P.drift) zn = __fmaf_rn(P.k_scale * m.dkz, P.dt, zn);
     }
     // 5. reflection, at most 4 folds, then clamp: the first fold by selects (near the ground
     // most warps hold a lane that folds once), the rest of the loop only where that leaves a
@@ -455,7 +466,7 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
         int jr = (int)floorf((yn - P.y0) * P.inv_dy + 0.5f);
         ir = min(max(ir, 0), P.nx - 1);
         jr = min(max(jr, 0), P.ny - 1);
-        int hr = (int)floorf(__fdiv_rn(T.tk - P.met_t0, P.met_dt));
+        int hr = (int)floorf(__fdiv_rn((float)k * P.dt - P.met_t0, P.met_dt));
         hr = min(max(hr, 0), P.n_t - 1);
         if (__ldg(P.rain + ((long long)hr * P.ny + jr) * P.nx + ir)) kind = 1;
     }
@@ -502,7 +513,7 @@ struct MinBlocks {
 // release step and ends with the particle: no status is tested inside it, and the lanes of a
 // tile of late releases all work from the loop's first turn. (The dosage samples gather a
 // warp's lanes at the same step, so with them the loop runs over common steps.)
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
 __global__ void __launch_bounds__(BLOCK, (MinBlocks<BLOCK, OCC>::value))
 advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *queue, int k0,
                int k1, int do_bin, int ppt)
@@ -518,8 +529,8 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
     const float sig_h_uniform = sqrtf(2.0f * P.k_scale * fmaxf(P.kh_uniform, 0.0f) * P.dt);
     // the launch's step times (the first barrier of the tile loop publishes them)
     __shared__ StepTable s_tab;
-    const int n_tab = min(k1 - k0, STEP_TAB);
-    for (int i = threadIdx.x; i < n_tab; i += BLOCK)
+    const uint32_t tab = shared_addr(&s_tab);
+    for (int i = threadIdx.x; i < k1 - k0; i += BLOCK)
         step_table_set(s_tab, i, step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k0 + i));
 
     int iter = 0;
@@ -589,46 +600,51 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
             unsigned int steps = 0u;                        // active steps of this particle
             float2 o0 = make_float2(0.f, 0.f), o1 = o0;     // wind offsets at h0, h1 (MIXED)
             int cur_h = -1;
-            DepCache dc;                                    // odd-step deposition words
-            dc.pair = -1;
             int k = k0;
             if (st == ST_UNRELEASED && sp >= k0 && sp < k1) {
                 x = __ldg(&sc.src_x); y = __ldg(&sc.src_y); z = __ldg(&sc.src_z);
                 st = ST_ACTIVE;
                 k = sp;
             }
+            const int k_own = k;                            // this lane's first step
+            DepCache dc;                                    // odd-step deposition words
+            if (st == ST_ACTIVE) dep_begin(P, gid, k, dc);
             auto advance = [&](int k) {
-                const StepTime T = k - k0 < n_tab
-                                       ? step_time_tab(P, s_tab, k - k0, k)
-                                       : step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k);
+                const StepTime T = step_time_tab<FIELDS || EXT || MIXED>(tab, k - k0, k);
                 float du = T.du, dv = T.dv;
                 if (MIXED && P.woff) {
-                    if (T.ts.h0 != cur_h) {
-                        cur_h = T.ts.h0;
+                    if (T.h0 != cur_h) {
+                        cur_h = T.h0;
                         const float2 *w = P.woff + (long long)sj * P.n_t;
-                        o0 = __ldg(w + T.ts.h0);
-                        o1 = __ldg(w + T.ts.h1);
+                        o0 = __ldg(w + T.h0);
+                        o1 = __ldg(w + min(T.h0 + 1, P.n_t - 1));
                     }
-                    // the same expression as step_time's, so sorting changes no bit
-                    du = P.bias_u + fmaf(T.ts.f, o1.x - o0.x, o0.x);
-                    dv = P.bias_v + fmaf(T.ts.f, o1.y - o0.y, o0.y);
+                    // the same expression as step_offset's, so sorting changes no bit
+                    du = P.bias_u + fmaf(T.f, o1.x - o0.x, o0.x);
+                    dv = P.bias_v + fmaf(T.f, o1.y - o0.y, o0.y);
                 }
-                ++steps;
-                st = particle_step<true, EXT, Levels, MODES>(P, LV, T, sc, &sc, gid, sp,
-                                                             sig_h_uniform, du, dv, x, y, z,
-                                                             nullptr, lang ? &wv : nullptr, msc,
-                                                             &dc);
+                return particle_step<true, EXT, Levels, MODES, FIELDS>(
+                    P, LV, T, sc, &sc, gid, sp, sig_h_uniform, du, dv, x, y, z, nullptr,
+                    lang ? &wv : nullptr, msc, &dc);
             };
             if (!EXT || !P.dose_every) {
+                if (st == ST_ACTIVE) {
 #pragma unroll 1
-                for (; st == ST_ACTIVE && k < k1; ++k) advance(k);
+                    do {
+                        st = advance(k);
+                        ++k;
+                    } while (st == ST_ACTIVE && k < k1);
+                    steps = (unsigned int)(k - k_own);
+                }
             } else {
-                const int k_own = k;                        // this lane's first step
 #pragma unroll 1
                 for (k = k0; k < k1; ++k) {
                     // the samples are warp-collective: the warp stays together
                     if (!__any_sync(0xffffffffu, st == ST_ACTIVE)) break;
-                    if (st == ST_ACTIVE && k >= k_own) advance(k);
+                    if (st == ST_ACTIVE && k >= k_own) {
+                        st = advance(k);
+                        ++steps;
+                    }
                     // every dose_every-th step, the decayed masses at t_{k+1}
                     if ((k + 1) % P.dose_every == 0) {
                         const bool on = st == ST_ACTIVE && k >= k_own;
@@ -672,8 +688,8 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
                 if (on) {
                     int ix, jy, kz;
                     float fa, fb, fc;
-                    axis(x, P.x0, P.inv_dx, P.nx, ix, fa);
-                    axis(y, P.y0, P.inv_dy, P.ny, jy, fb);
+                    axis(x, P.x0, P.inv_dx, P.nx2, ix, fa);
+                    axis(y, P.y0, P.inv_dy, P.ny2, jy, fb);
                     level(P, LV, z, kz, fc);
                     key = cell_key(P, ix, jy, kz);
                 } else if (local < count) {
@@ -738,54 +754,56 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
     }
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
 void adv_prefer_l1()
 {
     // the kernel needs a few KB of shared memory per block: ask for a small carve-out so the
     // rest of the SM's unified L1 serves the weather gathers (measured +0.7 to +1.7 %)
-    cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES>,
+    cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>,
                          cudaFuncAttributePreferredSharedMemoryCarveout, 10);
     (void)cudaGetLastError();
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
 cudaError_t launch_adv(const AdvanceLaunch &L)
 {
     static std::once_flag once;          // per instantiation; contexts may use several threads
-    std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES>);
+    std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>);
     const size_t smem = adv_dyn_smem(L.params->n_lut);
-    advance_kernel<BLOCK, OCC, MIXED, EXT, MODES><<<L.grid, BLOCK, smem, L.stream>>>(
+    advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS><<<L.grid, BLOCK, smem, L.stream>>>(
         *L.params, L.ranges, L.n_tiles(), L.queue, L.k0, L.k1, L.do_bin, L.ppt);
     return cudaGetLastError();
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
 int occ_adv(size_t smem)
 {
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, advance_kernel<BLOCK, OCC, MIXED, EXT, MODES>, BLOCK, smem);
+        &n, advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>, BLOCK, smem);
     return n;
 }
 
-// (occupancy variant, mixed scenarios, options: 0 none, 1 extended, 2 perturbation modes
-// alone) -> instantiation, for one block size
-#define LPM_ADV_CASE(FN, BLOCK, OCC, MIX, EX, ...)                                     \
-    case OCC * 100 + MIX * 10 + EX:                                                    \
-        return FN<BLOCK, OCC, (MIX != 0), (EX == 1), (EX != 0)>(__VA_ARGS__);
-#define LPM_ADV_CASES2(FN, BLOCK, OCC, EX, ...)                                        \
-    LPM_ADV_CASE(FN, BLOCK, OCC, 0, EX, __VA_ARGS__)                                   \
-    LPM_ADV_CASE(FN, BLOCK, OCC, 1, EX, __VA_ARGS__)
+// (occupancy variant, mixed scenarios, options: AdvanceLaunch::variant) -> instantiation, for
+// one block size
+#define LPM_ADV_CASE(FN, BLOCK, OCC, MIX, VAR, ...)                                    \
+    case OCC * 100 + MIX * 10 + VAR:                                                   \
+        return FN<BLOCK, OCC, (MIX != 0), (VAR == ADV_EXT),                            \
+                  (VAR == ADV_EXT || VAR == ADV_MODES || VAR == ADV_MODES_FIELDS),     \
+                  (VAR == ADV_EXT || VAR == ADV_FIELDS || VAR == ADV_MODES_FIELDS)>(__VA_ARGS__);
+#define LPM_ADV_CASES2(FN, BLOCK, VAR, ...)                                            \
+    LPM_ADV_CASE(FN, BLOCK, 0, 0, VAR, __VA_ARGS__)                                    \
+    LPM_ADV_CASE(FN, BLOCK, 0, 1, VAR, __VA_ARGS__)                                    \
+    LPM_ADV_CASE(FN, BLOCK, 1, 0, VAR, __VA_ARGS__)                                    \
+    LPM_ADV_CASE(FN, BLOCK, 1, 1, VAR, __VA_ARGS__)                                    \
+    LPM_ADV_CASE(FN, BLOCK, 2, 0, VAR, __VA_ARGS__)                                    \
+    LPM_ADV_CASE(FN, BLOCK, 2, 1, VAR, __VA_ARGS__)
 #define LPM_ADV_CASES(FN, BLOCK, ...)                                                  \
-    LPM_ADV_CASES2(FN, BLOCK, 0, 0, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 0, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 0, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 0, 1, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 1, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 1, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 0, 2, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 1, 2, __VA_ARGS__)                                       \
-    LPM_ADV_CASES2(FN, BLOCK, 2, 2, __VA_ARGS__)
+    LPM_ADV_CASES2(FN, BLOCK, 0, __VA_ARGS__)                                          \
+    LPM_ADV_CASES2(FN, BLOCK, 1, __VA_ARGS__)                                          \
+    LPM_ADV_CASES2(FN, BLOCK, 2, __VA_ARGS__)                                          \
+    LPM_ADV_CASES2(FN, BLOCK, 3, __VA_ARGS__)                                          \
+    LPM_ADV_CASES2(FN, BLOCK, 4, __VA_ARGS__)
 
 #define LPM_ADVANCE_TU(BLOCK)                                                          \
     cudaError_t launch_advance_b##BLOCK(const AdvanceLaunch &L)                         \

@@ -55,8 +55,8 @@ struct lpm_ctx {
     // weather
     float4 *d_uvwk = nullptr;               // slabs as given [n_t][nodes]
     float *d_kh = nullptr;
-    float4 *d_pair = nullptr;               // time-paired slabs [n_pair][nodes][2]
-    float2 *d_khpair = nullptr;             // [n_pair][nodes]
+    float4 *d_pair = nullptr;               // time-paired slabs [n_pair][slab_records][2]
+    float2 *d_khpair = nullptr;             // [n_pair][slab_records]
     uint8_t *d_rain = nullptr;
     std::vector<char> met_set;
     bool any_rain = false;
@@ -317,7 +317,10 @@ void fill_params(const lpm_ctx *c, StepParams &P)
     P.khpair = c->d_khpair;
     P.rain = c->any_rain ? c->d_rain : nullptr;
     P.nx = g.nx; P.ny = g.ny; P.nz = g.nz; P.n_t = g.n_met_t;
-    P.slab = (long long)g.nx * g.ny * g.nz;
+    P.nx2 = g.nx - 2; P.ny2 = g.ny - 2;
+    P.slab = slab_records(g.nx, g.ny, g.nz);
+    P.rec_y = 4u * (unsigned int)g.nx;
+    P.rec_z = P.rec_y * (unsigned int)((g.ny + 1) >> 1);
     P.x0 = (float)g.x0; P.y0 = (float)g.y0;
     P.dx = (float)g.dx; P.dy = (float)g.dy;
     P.inv_dx = (float)(1.0 / g.dx); P.inv_dy = (float)(1.0 / g.dy);
@@ -329,10 +332,12 @@ void fill_params(const lpm_ctx *c, StepParams &P)
         const float z0 = (float)c->zlev[k];
         const float inv = k + 1 < g.nz ? 1.0f / ((float)c->zlev[k + 1] - z0) : 0.0f;
         P.zi[k] = make_float2(z0, inv);
+        P.znext[k] = k < g.nz - 2 ? (float)c->zlev[k + 1] : std::numeric_limits<float>::infinity();
     }
     P.dt = (float)g.dt;
     P.kh_uniform = (float)g.kh_uniform;
     P.k_scale = (float)c->k_scale;
+    P.k2 = 2.0f * P.k_scale;
     P.bias_u = (float)c->bias_u;
     P.bias_v = (float)c->bias_v;
     P.lambda = g.half_life_s > 0 ? (float)(std::log(2.0) / g.half_life_s) : 0.0f;
@@ -364,6 +369,7 @@ void fill_params(const lpm_ctx *c, StepParams &P)
     P.ginv_dx = 1.0 / g.cdx; P.ginv_dy = 1.0 / g.cdy; P.ginv_dz = 1.0 / g.cdz;
     P.zlut = c->n_lut > 0 ? c->d_zlut : nullptr;
     P.n_lut = c->n_lut;
+    P.lut_last = c->n_lut - 1;
     P.lut_z0 = c->lut_z0;
     P.lut_inv_h = c->lut_inv_h;
     P.m0 = c->d_m0;
@@ -790,10 +796,11 @@ lpm_status lpm_create(const lpm_config *cfg, void *cuda_stream, lpm_ctx **out)
     const size_t ns = (size_t)cfg->n_scenarios;
     const size_t n_pair = (size_t)std::max(1, cfg->n_met_t - 1);
     CREATE_CUDA(cudaMalloc(&c->d_uvwk, nodes * cfg->n_met_t * sizeof(float4)));
-    CREATE_CUDA(cudaMalloc(&c->d_pair, nodes * n_pair * 2 * sizeof(float4)));
+    const size_t recs = (size_t)slab_records(cfg->nx, cfg->ny, cfg->nz);
+    CREATE_CUDA(cudaMalloc(&c->d_pair, recs * n_pair * 2 * sizeof(float4)));
     if (cfg->kh_uniform < 0) {
         CREATE_CUDA(cudaMalloc(&c->d_kh, nodes * cfg->n_met_t * sizeof(float)));
-        CREATE_CUDA(cudaMalloc(&c->d_khpair, nodes * n_pair * sizeof(float2)));
+        CREATE_CUDA(cudaMalloc(&c->d_khpair, recs * n_pair * sizeof(float2)));
     }
     CREATE_CUDA(cudaMalloc(&c->d_rain, (size_t)cfg->nx * cfg->ny * cfg->n_met_t));
     CREATE_CUDA(cudaMemsetAsync(c->d_rain, 0, (size_t)cfg->nx * cfg->ny * cfg->n_met_t, c->stream));
@@ -912,6 +919,7 @@ lpm_status lpm_set_met(lpm_ctx *c, int t_index, const float *uvwk, const float *
         return fail(c, LPM_E_INVALID, "kh must be given iff kh_uniform < 0");
     const size_t nodes = (size_t)g.nx * g.ny * g.nz;
     const size_t cols = (size_t)g.nx * g.ny;
+    const size_t recs = (size_t)slab_records(g.nx, g.ny, g.nz);
     const bool async = !on_device && is_pinned_host(uvwk) && is_pinned_host(kh) &&
                        is_pinned_host(rain);
     cudaStream_t s = c->stream;
@@ -950,7 +958,7 @@ lpm_status lpm_set_met(lpm_ctx *c, int t_index, const float *uvwk, const float *
         LPM_CUDA(c, launch_pack(s, c->d_uvwk + nodes * h, c->d_uvwk + nodes * h1,
                                 c->d_kh ? c->d_kh + nodes * h : nullptr,
                                 c->d_kh ? c->d_kh + nodes * h1 : nullptr,
-                                c->d_pair + nodes * 2 * h, c->d_khpair ? c->d_khpair + nodes * h : nullptr,
+                                c->d_pair + recs * 2 * h, c->d_khpair ? c->d_khpair + recs * h : nullptr,
                                 g.nx, g.ny, g.nz));
         c->n_launches++;
         if (async) {
@@ -1271,8 +1279,6 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
         L.ppt = c->ppt;
         L.occ = c->occ;
         L.mixed = batched;
-        L.ext = P.dose_every > 0 || P.blpair != nullptr || P.n_species > 1 || P.langevin;
-        L.modes = P.n_modes > 0;
         const int n_tiles = L.n_tiles();
         keys_ready = false;
         if (n_tiles <= 0) continue;
@@ -1375,6 +1381,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
         const long long next_bin = (k / g.bin_every + 1) * (long long)g.bin_every;
         long long e = std::min(k_end, std::min(next_bin, (long long)g.n_steps));
         if (E > 0) e = std::min(e, (k / E + 1) * E);
+        e = std::min(e, k + STEP_TAB);
         sg.k = k;
         sg.e = e;
         sg.do_bin = (e % g.bin_every == 0) || e == g.n_steps;
@@ -1402,10 +1409,8 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
     // ---- run ------------------------------------------------------------------------------
     if (!batched) {
         long long kernels = 0;
-        const bool ext_opts = P.dose_every > 0 || P.blpair != nullptr || P.n_species > 1 ||
-                              P.langevin;
         const int occ_blocks = std::max(1, advance_occupancy(
-            c->block, c->occ, false, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
+            c->block, c->occ, false, adv_variant(P),
             adv_dyn_smem(P.n_lut)));
         st = run_segments(c, P, plan, c->stream, c->sorted_upto, c->cur, kernels, true,
                           occ_blocks);
@@ -1423,10 +1428,8 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
             if (!c->cap_stream)
                 LPM_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
             const cudaStream_t cs = c->cap_stream;
-            const bool ext_opts = P.dose_every > 0 || P.blpair != nullptr || P.n_species > 1 ||
-                                  P.langevin;
             const int occ_blocks = std::max(1, advance_occupancy(
-                c->block, c->occ, true, ext_opts ? 1 : P.n_modes > 0 ? 2 : 0,
+                c->block, c->occ, true, adv_variant(P),
                 adv_dyn_smem(P.n_lut)));
             lpm_ctx::Graph ng{};
             ng.k0 = c->k;
@@ -1872,8 +1875,8 @@ lpm_status lpm_set_boundary_layer(lpm_ctx *c, int t_index, const float *bl, int 
         const int h1 = g.n_met_t > 1 ? h + 1 : h;
         if (h < 0 || h1 > g.n_met_t - 1 || (g.n_met_t > 1 && h > g.n_met_t - 2)) continue;
         if (!c->bl_set[(size_t)h] || !c->bl_set[(size_t)h1]) continue;
-        LPM_CUDA(c, launch_pack(c->stream, c->d_bl + cols * h, c->d_bl + cols * h1, nullptr,
-                                nullptr, c->d_blpair + cols * 2 * h, nullptr, g.nx, g.ny, 1));
+        LPM_CUDA(c, launch_pack_columns(c->stream, c->d_bl + cols * h, c->d_bl + cols * h1,
+                                        c->d_blpair + cols * 2 * h, g.nx, g.ny));
         c->n_launches++;
     }
     if (!on_device) LPM_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -45,20 +45,53 @@ __global__ void release_all_kernel(const StepParams P, float4 *__restrict__ stat
 }
 
 // ---------------------------------------------------------------------------------
-// Time pairing of the weather: pair[node] = (slab h, slab h+1 - slab h), so that one
-// 32-byte load brings both time levels of a corner and the time blend is one FMA (the
-// difference is the FP32 subtraction the blend would otherwise do at every step).
+// Time pairing of the weather: record = (slab h, slab h+1 - slab h), so that one 32-byte
+// load brings both time levels of a corner and the time blend is one FMA (the difference is
+// the FP32 subtraction the blend would otherwise do at every step). One thread a line of four
+// records (node_record), along x: rows of the slabs are read whole and lines written whole
+// (memory-bound: 32 B read and 32 B written a node). Nodes that an odd grid lacks are padded
+// with zeros, which no step reads.
 // ---------------------------------------------------------------------------------
 __global__ void pack_kernel(const float4 *__restrict__ a, const float4 *__restrict__ b,
                             const float *__restrict__ ka, const float *__restrict__ kb,
-                            float4 *__restrict__ pair, float2 *__restrict__ khpair, long long nodes)
+                            float4 *__restrict__ pair, float2 *__restrict__ khpair, int nx, int ny,
+                            int nz)
+{
+    const long long lines = slab_records(nx, ny, nz) / 4;
+    const int nby = (ny + 1) >> 1;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < lines; t += stride) {
+        const int i = (int)(t % nx);
+        const long long m = t / nx;
+        const int j0 = 2 * (int)(m % nby), k0 = 2 * (int)(m / nby);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int j = j0 + (r & 1), k = k0 + (r >> 1);
+            float4 u = make_float4(0.f, 0.f, 0.f, 0.f), d = u;
+            float2 kh = make_float2(0.f, 0.f);
+            if (j < ny && k < nz) {
+                const long long n = ((long long)k * ny + j) * nx + i;
+                const float4 v = b[n];
+                u = a[n];
+                d = make_float4(v.x - u.x, v.y - u.y, v.z - u.z, v.w - u.w);
+                if (khpair) kh = make_float2(ka[n], kb[n] - ka[n]);
+            }
+            pair[8 * t + 2 * r] = u;
+            pair[8 * t + 2 * r + 1] = d;
+            if (khpair) khpair[4 * t + r] = kh;
+        }
+    }
+}
+
+// The same for 2D columns, row-major.
+__global__ void pack_columns_kernel(const float4 *__restrict__ a, const float4 *__restrict__ b,
+                                    float4 *__restrict__ pair, long long n_cols)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < nodes; n += stride) {
+    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < n_cols; n += stride) {
         const float4 u = a[n], v = b[n];
         pair[2 * n] = u;
         pair[2 * n + 1] = make_float4(v.x - u.x, v.y - u.y, v.z - u.z, v.w - u.w);
-        if (khpair) khpair[n] = make_float2(ka[n], kb[n] - ka[n]);
     }
 }
 
@@ -210,12 +243,22 @@ cudaError_t launch_fixed_to_double(cudaStream_t s, const unsigned long long *in,
 cudaError_t launch_pack(cudaStream_t s, const float4 *a, const float4 *b, const float *ka,
                         const float *kb, float4 *pair, float2 *khpair, int nx, int ny, int nz)
 {
-    const long long nodes = (long long)nx * ny * nz;
+    const long long lines = slab_records(nx, ny, nz) / 4;
+    const int block = 128;
+    long long blocks = (lines + block - 1) / block;
+    if (blocks > 152 * 32) blocks = 152 * 32;
+    pack_kernel<<<(unsigned)blocks, block, 0, s>>>(a, b, ka, kb, pair, khpair, nx, ny, nz);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_columns(cudaStream_t s, const float4 *a, const float4 *b, float4 *pair,
+                                int nx, int ny)
+{
+    const long long n = (long long)nx * ny;
     const int block = 256;
-    long long blocks = (nodes + block - 1) / block;
+    long long blocks = (n + block - 1) / block;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    if (blocks < 1) blocks = 1;
-    pack_kernel<<<(unsigned)blocks, block, 0, s>>>(a, b, ka, kb, pair, khpair, nodes);
+    pack_columns_kernel<<<(unsigned)blocks, block, 0, s>>>(a, b, pair, n);
     return cudaGetLastError();
 }
 

@@ -38,6 +38,22 @@ struct Ranges {
     unsigned int *keys, *hist;
 };
 
+// Longest launch in steps: its step times sit in a table in shared memory.
+constexpr int STEP_TAB = 128;
+
+// Options of an advance launch, by the instantiation that carries their code: none; the
+// extended step (dosage, Eq. 3 K_z, a decay chain, the Langevin variant, with anything else);
+// perturbation modes; a gridded K_h or the drift correction; both of these.
+enum { ADV_PLAIN = 0, ADV_EXT = 1, ADV_MODES = 2, ADV_FIELDS = 3, ADV_MODES_FIELDS = 4 };
+
+inline int adv_variant(const StepParams &P)
+{
+    if (P.dose_every > 0 || P.blpair || P.n_species > 1 || P.langevin) return ADV_EXT;
+    const bool fields = P.khpair || P.drift;
+    if (P.n_modes > 0) return fields ? ADV_MODES_FIELDS : ADV_MODES;
+    return fields ? ADV_FIELDS : ADV_PLAIN;
+}
+
 struct AdvanceLaunch {
     cudaStream_t stream;
     const StepParams *params;
@@ -47,11 +63,9 @@ struct AdvanceLaunch {
     int k0, k1, do_bin;
     int block, ppt, occ;
     bool mixed;               // lanes of one tile may belong to different scenarios
-    bool ext;                 // dosage, Eq. 3 K_z, a decay chain or the Langevin variant is on
-    bool modes;               // perturbation modes are on (both: 1 particle per thread)
     unsigned int grid;
     int n_tiles() const { return ranges.tiles_a + ranges.n_b; }
-    int variant() const { return ext ? 1 : modes ? 2 : 0; }   // kernel options, see LPM_ADV_CASES
+    int variant() const { return adv_variant(*params); }
 };
 
 // Inputs of a sort: the live sorted particles of state_a (when has_a) followed by the B
@@ -149,6 +163,8 @@ int occupancy_b256(int occ, bool mixed, int variant, size_t smem);
 int occupancy_b512(int occ, bool mixed, int variant, size_t smem);
 cudaError_t launch_pack(cudaStream_t s, const float4 *a, const float4 *b, const float *ka,
                         const float *kb, float4 *pair, float2 *khpair, int nx, int ny, int nz);
+cudaError_t launch_pack_columns(cudaStream_t s, const float4 *a, const float4 *b, float4 *pair,
+                                int nx, int ny);
 cudaError_t launch_sort(cudaStream_t s, const StepParams &P, const SortSource &in,
                         const SortBuffers &out);
 cudaError_t launch_gather(cudaStream_t s, const float4 *home, const float4 *sorted,

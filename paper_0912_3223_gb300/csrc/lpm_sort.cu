@@ -76,8 +76,8 @@ __global__ void sort_keys_kernel(const StepParams P, const SortSource S,
                 if ((__float_as_uint(s.w) >> TAG_SHIFT) == ST_ACTIVE) {
                     int ix, jy, kz;
                     float a, b, c;
-                    axis(s.x, P.x0, P.inv_dx, P.nx, ix, a);
-                    axis(s.y, P.y0, P.inv_dy, P.ny, jy, b);
+                    axis(s.x, P.x0, P.inv_dx, P.nx2, ix, a);
+                    axis(s.y, P.y0, P.inv_dy, P.ny2, jy, b);
                     level(P, LV, s.z, kz, c);
                     key = cell_key(P, ix, jy, kz);
                     if (S.key_scen > 0) {
