@@ -371,7 +371,11 @@ __device__ __forceinline__ Met sample_met_pair(const StepParams &P, const LEV &L
 // particle's scenario plus the bias at t_k. With GRIDS, deposition and exit add their mass
 // to the scenario's grids and counters; *fold receives dz/dz_pre (+-1, 0 when clamped).
 // FIELDS: the run may have a gridded K_h or the drift correction (uniform run-time tests).
-template <bool GRIDS, bool EXT = false, class LEV, bool MODES = EXT, bool FIELDS = true>
+// DRAWS_FIRST: the draws stand before the gathers, so that the two overlap where registers
+// allow it (measured at 128 registers a thread: 2e4 particles over a day 4.55 -> 4.38 ms; at
+// 64 it costs spills: 1e7 particles 40.8 -> 41.9 ms).
+template <bool GRIDS, bool EXT = false, class LEV, bool MODES = EXT, bool FIELDS = true,
+          bool DRAWS_FIRST = false>
 __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV &LV,
                                                   const StepTime &T, const ScenDev &sc,
                                                   const ScenDev *scg, unsigned long long gid,
@@ -381,15 +385,19 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
                                                   DepCache *dc = nullptr)
 {
     const int k = T.k;
+    float n0, n1, n2;
+    auto draw = [&]() {
+        const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
+        normals3(w, n0, n1, n2);
+    };
+    if (DRAWS_FIRST) draw();
     // 1. weather at the old position and t_k (with the scenario's perturbation modes: msc);
     // 2. diffusivities
     const Met m = sample_met_pair<EXT, LEV, MODES, FIELDS>(P, LV, T, x, y, z, msc);
     const float sig_h = FIELDS && P.khpair ? sqrtf(P.k2 * m.kh * P.dt) : sig_h_uniform;
     const float sig_z = sqrtf(P.k2 * m.kz * P.dt);
     // 3. N(0,1) draws
-    const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
-    float n0, n1, n2;
-    normals3(w, n0, n1, n2);
+    if (!DRAWS_FIRST) draw();
     // 4. Eq. (1)-(2): wind then turbulent displacement
     // (fused multiply-adds, written out: every instantiation rounds alike)
     const float xn = __fmaf_rn(n0, sig_h, __fmaf_rn(m.u + du, P.dt, x));
@@ -497,16 +505,18 @@ struct MinBlocks {
 };
 
 // Advance: each thread keeps a particle in registers and runs steps [k0, k1) over the
-// launch's tiles (Ranges): sorted tiles of A and release-ordered tiles of B, handed out by
-// block index (grid over all tiles) or by an atomic queue (persistent grid); a tile holds ppt
-// particles per thread, one after the other. With MIXED the lanes of a tile may belong to
-// different scenarios (the sorted particles of a batched context): each lane finds its
-// scenario from its home slot and carries its own wind offset; the results are bit-identical
-// to the per-scenario path. EXT adds, as uniform run-time options, the dosage samples (every
-// P.dose_every steps) inside the time loop, K_z from Eq. 3 (P.blpair), the daughters of a
-// decay chain (P.n_species > 1), the Langevin variant and the scenarios' perturbation modes
-// (P.n_modes > 0); MODES without EXT carries the modes alone. The default instantiations
-// carry none of that code.
+// launch's particles (Ranges): sorted ones of A, release-ordered tiles of B. The persistent
+// grid takes tiles of a block's size from an atomic queue: neighbours in the sorted order
+// share weather records, so they run on one SM and, held by the block's barrier, at nearly
+// the same step (handing single warps out instead cost 10 %, without the barrier 14 %). A
+// launch that fits the grid at once is spread evenly over its blocks. With MIXED the lanes of
+// a warp may belong to different scenarios (the sorted particles of a batched context): each
+// lane finds its scenario from its home slot and carries its own wind offset; the results are
+// bit-identical to the per-scenario path. EXT adds, as uniform run-time options, the dosage
+// samples (every P.dose_every steps) inside the time loop, K_z from Eq. 3 (P.blpair), the
+// daughters of a decay chain (P.n_species > 1), the Langevin variant and the scenarios'
+// perturbation modes (P.n_modes > 0); MODES carries the modes alone, FIELDS a gridded K_h and
+// the drift correction. The plain instantiations carry none of that code.
 //
 // Bound by issued instructions (32 warps an SM keep the schedulers 75 % busy, DRAM idle), so
 // the step is kept short of branches and constant loads. A lane's time loop starts at its own
@@ -515,63 +525,66 @@ struct MinBlocks {
 // warp's lanes at the same step, so with them the loop runs over common steps.)
 template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
 __global__ void __launch_bounds__(BLOCK, (MinBlocks<BLOCK, OCC>::value))
-advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *queue, int k0,
-               int k1, int do_bin, int ppt)
+advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, int k1, int do_bin)
 {
     extern __shared__ float4 s_adv_dyn[];            // the level table, sized by the launch
     __shared__ unsigned long long s_acc[BLOCK];
-    __shared__ int s_tile;
     __shared__ unsigned long long s_steps;
+    __shared__ unsigned int s_tile;
+    __shared__ StepTable s_tab;                      // the launch's step times
+    // Units of a warp's 32 particles: those of A, then those of the B tiles. (A launch of the
+    // pair that has another number of units for its shape has nothing to do.)
+    constexpr unsigned int WARPS = BLOCK / 32;
+    const long long live = R.a_live ? (long long)*R.a_live : 0;
+    const unsigned int units_a = (unsigned int)((live + 31) >> 5);
+    const unsigned int n_units = units_a + ((unsigned int)R.n_b << R.unit_shift);
+    if (n_units < R.unit_min || n_units > R.unit_max) return;
     const Levels LV = load_levels(P, reinterpret_cast<unsigned char *>(s_adv_dyn));
     unsigned long long *s_warp = s_acc + (threadIdx.x & ~31);
+    const int lane = threadIdx.x & 31;
+    const unsigned int warp = threadIdx.x >> 5;
     const long long n_cells = (long long)P.cx * P.cy * P.cz;
     // the uniform horizontal diffusivity gives one displacement scale for the run
-    const float sig_h_uniform = sqrtf(2.0f * P.k_scale * fmaxf(P.kh_uniform, 0.0f) * P.dt);
-    // the launch's step times (the first barrier of the tile loop publishes them)
-    __shared__ StepTable s_tab;
+    const float sig_h_uniform = sqrtf(P.k2 * fmaxf(P.kh_uniform, 0.0f) * P.dt);
     const uint32_t tab = shared_addr(&s_tab);
     for (int i = threadIdx.x; i < k1 - k0; i += BLOCK)
         step_table_set(s_tab, i, step_time(P, MIXED ? nullptr : P.scen[0].wind_offset, k0 + i));
+    if (threadIdx.x == 0) s_steps = 0ull;
+    __syncthreads();
 
-    int iter = 0;
-    for (;;) {
-        // ---- fetch a tile -----------------------------------------------------------
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_tile = queue ? (int)atomicAdd(queue, 1u) : (int)blockIdx.x + iter * (int)gridDim.x;
-            s_steps = 0ull;
-        }
-        __syncthreads();
-        const int t = s_tile;
-        ++iter;
-        if (t >= n_tiles) break;
-        const bool in_a = t < R.tiles_a;
-        float4 *state;
-        long long first;
-        int count, tscen;
-        if (in_a) {
-            state = R.state_a;
-            first = (long long)t * BLOCK * ppt;
-            count = (int)max(0LL, min((long long)BLOCK * ppt, (long long)*R.a_live - first));
-            tscen = 0;
-        } else {
-            const Tile tl = R.b_tiles[R.b_first + (t - R.tiles_a)];
-            state = R.state_b;
-            first = tl.first;
-            count = tl.count;
-            tscen = tl.scen;
-            if (!LPM_IN_BOUNDS(P.err, first >= 0 && first + count <= P.slot_cap && tscen >= 0 &&
-                                          tscen < P.n_scen))
-                count = 0;
-        }
-        if (count <= 0) continue;                       // the whole block skips
-        const ScenDev &scg = P.scen[tscen];
+    // A block's tile is a run of neighbouring units: as many as it has warps, or, when all
+    // units fit the grid at once, the same share for every block.
+    const bool one_round = n_units <= WARPS * gridDim.x;
+    const unsigned int tile_units =
+        one_round ? max(1u, (n_units + gridDim.x - 1u) / gridDim.x) : WARPS;
+    for (unsigned int tile = blockIdx.x; tile * tile_units < n_units;) {
+        const unsigned int unit = tile * tile_units + warp;
+        if (warp < tile_units && unit < n_units) {
+            const bool in_a = unit < units_a;
+            float4 *state;
+            long long first;                         // slot of lane 0
+            int count, tscen;
+            if (in_a) {
+                state = R.state_a;
+                first = (long long)unit * 32;
+                count = (int)min(32LL, live - first);
+                tscen = 0;
+            } else {
+                const unsigned int u = unit - units_a;
+                const Tile tl = R.b_tiles[R.b_first + (u >> R.unit_shift)];
+                const int off = (int)(u & ((1u << R.unit_shift) - 1u)) * 32;
+                state = R.state_b;
+                first = tl.first + off;
+                count = max(0, min(32, tl.count - off));
+                tscen = tl.scen;
+                if (!LPM_IN_BOUNDS(P.err, first >= 0 && first + count <= P.slot_cap && tscen >= 0 &&
+                                              tscen < P.n_scen))
+                    count = 0;
+            }
+            const ScenDev &scg = P.scen[tscen];
 
-#pragma unroll 1
-        for (int j = 0; j < ppt; ++j) {
             // ---- load the particle ------------------------------------------------------
-            const int local = j * BLOCK + threadIdx.x;
-            const long long slot = first + local;
+            const long long slot = first + lane;
             float *wsrc = in_a ? R.w_a : R.w_b;
             const bool lang = EXT && P.langevin && wsrc;
             const bool modes = MODES && P.n_modes > 0 && P.mode_sc;
@@ -579,7 +592,7 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
             uint32_t st = ST_EXITED;
             int sp = 0, sj = tscen;                          // sj: scenario of the particle
             unsigned long long gid = 0ull;
-            if (local < count) {
+            if (lane < count) {
                 long long home = in_a ? (long long)__ldg(R.pidx + slot) : slot;
                 if (!LPM_IN_BOUNDS(P.err, home >= 0 && home < P.slot_cap)) home = 0;
                 if (MIXED && in_a) sj = scen_of(P, home);
@@ -623,7 +636,7 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
                     du = P.bias_u + fmaf(T.f, o1.x - o0.x, o0.x);
                     dv = P.bias_v + fmaf(T.f, o1.y - o0.y, o0.y);
                 }
-                return particle_step<true, EXT, Levels, MODES, FIELDS>(
+                return particle_step<true, EXT, Levels, MODES, FIELDS, OCC != 2>(
                     P, LV, T, sc, &sc, gid, sp, sig_h_uniform, du, dv, x, y, z, nullptr,
                     lang ? &wv : nullptr, msc, &dc);
             };
@@ -665,25 +678,24 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
             }
 
             // ---- store ------------------------------------------------------------------
-            const bool on = local < count && st == ST_ACTIVE;
-            if (local < count) {
-                state[first + local] = make_float4(x, y, z, __uint_as_float((st << TAG_SHIFT) |
+            const bool on = lane < count && st == ST_ACTIVE;
+            if (lane < count) {
+                state[slot] = make_float4(x, y, z, __uint_as_float((st << TAG_SHIFT) |
                                                                             (uint32_t)sp));
                 // only a moving particle has a turbulent velocity (0 once deposited or
                 // exited, and before its release)
-                if (lang) wsrc[first + local] = on ? wv : 0.0f;
+                if (lang) wsrc[slot] = on ? wv : 0.0f;
             }
 
             // ---- sort keys for the sort that follows (its inputs: A slots, then B lanes) ----
             if (R.keys) {
                 const unsigned int dead_key = (unsigned int)sort_key_range(P.nx, P.ny, P.nz);
-                const int lane = threadIdx.x & 31;
                 long long idx = -1;
                 unsigned int key = KEY_NONE_U;
                 if (in_a) {
-                    if (local < count) idx = first + local;
+                    if (lane < count) idx = slot;
                 } else {
-                    idx = (long long)*R.a_live + (long long)(t - R.tiles_a) * BLOCK * ppt + local;
+                    idx = live + (long long)(unit - units_a) * 32 + lane;
                 }
                 if (on) {
                     int ix, jy, kz;
@@ -692,7 +704,7 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
                     axis(y, P.y0, P.inv_dy, P.ny2, jy, fb);
                     level(P, LV, z, kz, fc);
                     key = cell_key(P, ix, jy, kz);
-                } else if (local < count) {
+                } else if (lane < count) {
                     key = dead_key;
                 }
                 if (idx >= 0) R.keys[idx] = key;
@@ -740,17 +752,22 @@ advance_kernel(const StepParams P, const Ranges R, int n_tiles, unsigned int *qu
 
             // ---- active particle-steps --------------------------------------------------
             if (MIXED) {
-                warp_count_scen(local < count ? sj : -1, steps, C_ACTIVE_STEPS, P, s_warp);
+                warp_count_scen(lane < count ? sj : -1, steps, C_ACTIVE_STEPS, P, s_warp);
             } else {
                 const unsigned int sum = __reduce_add_sync(0xffffffffu, steps);
                 if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&s_steps, (unsigned long long)sum);
             }
         }
-        if (!MIXED) {
-            __syncthreads();
-            if (threadIdx.x == 0 && s_steps)
-                atomicAdd(scg.ctr + C_ACTIVE_STEPS * P.ctr_stride, s_steps);
-        }
+        if (one_round) break;
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = gridDim.x + atomicAdd(queue, 1u);
+        __syncthreads();
+        tile = s_tile;
+    }
+    if (!MIXED) {
+        __syncthreads();
+        if (threadIdx.x == 0 && s_steps)
+            atomicAdd(P.scen[0].ctr + C_ACTIVE_STEPS * P.ctr_stride, s_steps);
     }
 }
 
@@ -771,7 +788,7 @@ cudaError_t launch_adv(const AdvanceLaunch &L)
     std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>);
     const size_t smem = adv_dyn_smem(L.params->n_lut);
     advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS><<<L.grid, BLOCK, smem, L.stream>>>(
-        *L.params, L.ranges, L.n_tiles(), L.queue, L.k0, L.k1, L.do_bin, L.ppt);
+        *L.params, L.ranges, L.queue, L.k0, L.k1, L.do_bin);
     return cudaGetLastError();
 }
 

@@ -83,7 +83,8 @@ struct lpm_ctx {
     unsigned long long *d_dep = nullptr;    // [n_scen][2*cy*cx]
     unsigned long long *d_ctr = nullptr;    // [N_COUNTERS][n_scen]
     unsigned int *d_err = nullptr;
-    unsigned int *d_queue = nullptr;
+    unsigned int *d_queue = nullptr;        // tile-queue counters of a call's launches
+    size_t queue_cap = 0;
     float *d_m0 = nullptr;
     size_t d_m0_cap = 0;
     unsigned char *d_zlut = nullptr;        // vertical level lookup table
@@ -108,6 +109,7 @@ struct lpm_ctx {
     bool tables_dirty = true;
     long long k = 0;                        // steps taken
     long long n_bins = 0;                   // snapshots taken
+    bool launch_set = false;                // lpm_set_launch was called; else by size
     int block = 512, ppt = 1, occ = 2;
 
     // sorting by weather cell (both forms) at the multiples of sort_every: d_state is the
@@ -551,13 +553,22 @@ long long released_before(const ScenHost &h, long long k1)
     return std::max(0LL, std::min(upto - h.part_first, h.n));
 }
 
+// Particles of a tile of the tile table: what a block of the chosen launch shape holds, and by
+// default 512, or a warp's 32 in runs small enough to be spread warp by warp (a scenario's or
+// an interval's last tile is then at most 31 lanes short).
+int tile_particles(const lpm_ctx *c)
+{
+    if (c->launch_set) return c->block * c->ppt;
+    return c->n_slots_used <= (1 << 17) ? 32 : 512;
+}
+
 // Tile table (see lpm_ctx::tiles). A segment [k, e) after the sort at sorted_upto runs
 // the tiles from the interval of sorted_upto up to the last tile whose first particle
 // leaves before e; a sort at a multiple of E takes the tiles of the intervals since the
 // previous sort. Tiles never straddle an interval, so no particle is in both sets.
 lpm_status build_tiles(lpm_ctx *c)
 {
-    const int T = c->block * c->ppt;
+    const int T = tile_particles(c);
     const long long NS = std::max<long long>(1, c->cfg.n_steps);
     const long long E = c->sort_every > 0 ? c->sort_every : NS;
     const long long n_int = (NS + E - 1) / E;
@@ -809,7 +820,8 @@ lpm_status lpm_create(const lpm_config *cfg, void *cuda_stream, lpm_ctx **out)
     CREATE_CUDA(cudaMalloc(&c->d_dep, ns * c->ndep() * sizeof(unsigned long long)));
     CREATE_CUDA(cudaMalloc(&c->d_ctr, ns * N_COUNTERS * sizeof(unsigned long long)));
     CREATE_CUDA(cudaMalloc(&c->d_err, sizeof(unsigned int)));
-    CREATE_CUDA(cudaMalloc(&c->d_queue, sizeof(unsigned int)));
+    c->queue_cap = 64;
+    CREATE_CUDA(cudaMalloc(&c->d_queue, c->queue_cap * sizeof(unsigned int)));
     CREATE_CUDA(cudaMalloc(&c->d_scen, ns * sizeof(ScenDev)));
     CREATE_CUDA(cudaMalloc(&c->d_woff, ns * cfg->n_met_t * sizeof(float2)));
     CREATE_CUDA(cudaMemsetAsync(c->d_conc, 0, ns * c->ncell() * sizeof(unsigned long long), c->stream));
@@ -1159,6 +1171,7 @@ lpm_status lpm_set_launch(lpm_ctx *c, int block, int ppt, int occupancy)
         occupancy < 0 || occupancy > 2)
         return fail(c, LPM_E_INVALID, "launch shape %d x %d (occupancy %d) not supported", block, ppt,
                     occupancy);
+    c->launch_set = true;
     c->block = block;
     c->ppt = ppt;
     c->occ = occupancy;
@@ -1195,18 +1208,63 @@ struct Segment {
     int b_lo, b_hi;                    // tiles run from their home slots
 };
 
+// Launch shapes of an advance segment of at most `units` warps of particles (unless
+// lpm_set_launch chose one):
+//  - up to 20 warps an SM, 128 registers a thread (16 at a time): a step's latency is all that counts, and
+//    its eight gathers fly together. Advance of 2e4 particles over a day: 4.2 ms against 7.2 at
+//    64 registers. From 16 warps an SM on it takes a second round, still the faster one at 20
+//    (2e5 particles x 720 steps 1.70 ms against 1.84 at 80 registers) and no longer at 24.
+//    Blocks of 256 except where there are fewer warps than schedulers;
+//  - up to 1e6 particles, and the extended step at any size, 80 registers (24 warps): 3e5
+//    particles x 720 steps 2.08 ms against 2.22 at 64 registers, dose assessment 3.9 against 4.3
+//    (the extended step spills at 64);
+//  - above, and with mixed scenarios, 64 registers (32 warps): 1e7 particles 40.8 ms against
+//    42.5, 64 scenarios 59 against 66.
+// `units` counts every particle released so far; where the bound leaves open which of the
+// first two is the better one, both are launched and the device's live count lets one of them
+// return at once (2 us).
+struct Shape {
+    int block, occ, blocks;            // blocks: the persistent grid's limit
+    unsigned int unit_min, unit_max;
+};
+
+int launch_shapes(const lpm_ctx *c, const StepParams &P, long long units, Shape h[2])
+{
+    constexpr unsigned int ANY = 0xffffffffu;
+    const unsigned int few = 20u * (unsigned int)c->sm_count;
+    const int variant = adv_variant(P);
+    const bool mixed = P.n_scen > 1;
+    int n = 0;
+    if (c->launch_set) {
+        h[n++] = {c->block, c->occ, 0, 0u, ANY};
+    } else {
+        const bool small = units <= few, large = units > 8LL * few;
+        if (!large)
+            h[n++] = {units <= 4LL * c->sm_count ? 512 : 256, 0, 0, 0u, small ? ANY : few};
+        if (!small) {
+            const bool wide = variant != ADV_EXT && (mixed || units > 32768);
+            h[n++] = {wide ? 512 : 256, wide ? 2 : 1, 0, large ? 0u : few + 1u, ANY};
+        }
+    }
+    for (int i = 0; i < n; ++i)
+        h[i].blocks = c->sm_count * std::max(1, advance_occupancy(h[i].block, h[i].occ, mixed,
+                                                                  variant, adv_dyn_smem(P.n_lut)));
+    return n;
+}
+
 // Issues the segments on stream s, starting from sort state (upto, cur); returns the
 // kernels launched and leaves the final sort state in (upto, cur). `direct`: launched now
 // (not captured), so advance launches are counted and, with profiling, timed.
 lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segment> &plan,
                         cudaStream_t s, long long &upto, int &cur, long long &kernels,
-                        bool direct, int occ_blocks)
+                        bool direct)
 {
     const lpm_config &g = c->cfg;
     const bool batched = g.n_scenarios > 1;
-    const int T = c->block * c->ppt;
+    const int T = tile_particles(c);
     const size_t ns = (size_t)g.n_scenarios;
     bool keys_ready = false;                 // the previous launch wrote the sort's keys
+    LPM_CUDA(c, cudaMemsetAsync(c->d_queue, 0, plan.size() * sizeof(unsigned int), s));
     for (size_t gi = 0; gi < plan.size(); ++gi) {
         const Segment &sg = plan[gi];
         if (direct) {
@@ -1263,25 +1321,24 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
         L.stream = s;
         L.params = &P;
         L.ranges.state_a = c->d_sorted[cur];
-        L.ranges.a_live = c->d_live;
+        L.ranges.a_live = upto > 0 ? c->d_live : nullptr;
         L.ranges.pidx = c->d_pidx[cur];
-        L.ranges.tiles_a = (int)((sg.a_bound + T - 1) / T);
         L.ranges.state_b = c->d_state;
         L.ranges.b_tiles = c->d_tiles;
         L.ranges.b_first = sg.b_lo;
         L.ranges.n_b = sg.b_hi - sg.b_lo;
+        while ((32 << L.ranges.unit_shift) < T) ++L.ranges.unit_shift;
         L.ranges.w_a = c->langevin ? c->d_w_sorted[cur] : nullptr;
         L.ranges.w_b = c->langevin ? c->d_w_home : nullptr;
         L.k0 = (int)sg.k;
         L.k1 = (int)sg.e;
         L.do_bin = sg.do_bin ? 1 : 0;
-        L.block = c->block;
-        L.ppt = c->ppt;
-        L.occ = c->occ;
         L.mixed = batched;
-        const int n_tiles = L.n_tiles();
+        // an upper bound of the launch's warp units (the kernel counts the live particles)
+        const long long units =
+            (sg.a_bound + 31) / 32 + ((long long)L.ranges.n_b << L.ranges.unit_shift);
         keys_ready = false;
-        if (n_tiles <= 0) continue;
+        if (units <= 0) continue;
         // the next segment starts with a sort of exactly these particles: write its keys here
         // (one scenario: measured +0.9 %; the 256-scenario ensemble sorted every 30 steps:
         // +0.3 %)
@@ -1294,11 +1351,10 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
             L.ranges.hist = c->d_hist;
             keys_ready = true;
         }
-        // persistent grid over an atomic tile queue (the plain run: measured +0.8 % against
-        // a grid of all tiles, each block loading the level table once for many tiles)
-        LPM_CUDA(c, cudaMemsetAsync(c->d_queue, 0, sizeof(unsigned int), s));
-        L.queue = c->d_queue;
-        L.grid = (unsigned)std::max(1, std::min(n_tiles, occ_blocks * c->sm_count));
+        // persistent grid over an atomic tile queue, one counter per launch of the call
+        L.queue = c->d_queue + gi;
+        Shape shapes[2];
+        const int n_shapes = launch_shapes(c, P, units, shapes);
         const bool timed = direct && c->profiling;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (timed) {
@@ -1309,11 +1365,18 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
         }
         {
             NvtxRange nr("lpm advance");
-            LPM_CUDA(c, launch_advance(L));
+            for (int i = 0; i < n_shapes; ++i) {
+                L.block = shapes[i].block;
+                L.occ = shapes[i].occ;
+                L.grid = (unsigned)std::min<long long>(units, shapes[i].blocks);
+                L.ranges.unit_min = shapes[i].unit_min;
+                L.ranges.unit_max = shapes[i].unit_max;
+                LPM_CUDA(c, launch_advance(L));
+            }
         }
         if (timed) LPM_CUDA(c, cudaEventRecord(e1, s));
         if (direct) c->n_adv_launches++;
-        kernels++;
+        kernels += n_shapes;
     }
     return LPM_OK;
 }
@@ -1368,7 +1431,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
     StepParams P;
     fill_params(c, P);
     const bool batched = g.n_scenarios > 1;
-    const int T = c->block * c->ppt;
+    const int T = tile_particles(c);
     const long long E = c->sort_every, Et = c->tiles_E;
     const long long k_end = c->k + n;
 
@@ -1401,6 +1464,15 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
         plan.push_back(sg);
         k = e;
     }
+    if (plan.size() > c->queue_cap) {
+        drop_graphs(c);                      // graphs hold the counters' address
+        LPM_CUDA(c, cudaStreamSynchronize(c->stream));
+        cudaFree(c->d_queue);
+        c->d_queue = nullptr;
+        c->queue_cap = 0;
+        LPM_CUDA(c, cudaMalloc(&c->d_queue, plan.size() * sizeof(unsigned int)));
+        c->queue_cap = plan.size();
+    }
     if (upto > 0) {
         st = ensure_sort_buffers(c, std::max<size_t>(keys_need, 1));
         if (st != LPM_OK) return st;
@@ -1409,11 +1481,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
     // ---- run ------------------------------------------------------------------------------
     if (!batched) {
         long long kernels = 0;
-        const int occ_blocks = std::max(1, advance_occupancy(
-            c->block, c->occ, false, adv_variant(P),
-            adv_dyn_smem(P.n_lut)));
-        st = run_segments(c, P, plan, c->stream, c->sorted_upto, c->cur, kernels, true,
-                          occ_blocks);
+        st = run_segments(c, P, plan, c->stream, c->sorted_upto, c->cur, kernels, true);
         c->n_launches += kernels;
         if (st != LPM_OK) return st;
     } else {
@@ -1428,17 +1496,13 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
             if (!c->cap_stream)
                 LPM_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
             const cudaStream_t cs = c->cap_stream;
-            const int occ_blocks = std::max(1, advance_occupancy(
-                c->block, c->occ, true, adv_variant(P),
-                adv_dyn_smem(P.n_lut)));
             lpm_ctx::Graph ng{};
             ng.k0 = c->k;
             ng.k1 = k_end;
             ng.upto0 = ng.upto1 = c->sorted_upto;
             ng.cur0 = ng.cur1 = c->cur;
             LPM_CUDA(c, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-            lpm_status rs = run_segments(c, P, plan, cs, ng.upto1, ng.cur1, ng.kernels, false,
-                                         occ_blocks);
+            lpm_status rs = run_segments(c, P, plan, cs, ng.upto1, ng.cur1, ng.kernels, false);
             cudaGraph_t graph = nullptr;
             const cudaError_t ce = cudaStreamEndCapture(cs, &graph);
             if (rs != LPM_OK || ce != cudaSuccess) {

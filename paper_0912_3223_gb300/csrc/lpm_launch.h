@@ -20,21 +20,20 @@ struct NvtxRange {
 // The particles of an advance launch. A = the sorted live particles [0, live) of state_a
 // (live count on the device; home slot of sorted slot i in pidx[i]; any scenario);
 // B = tiles [b_first, b_first + n_b) of the tile table, each a run of one scenario's
-// particles at their home slots in state_b. Launch tile t < tiles_a is slots
-// [t*T, t*T + T) of A, tile tiles_a + u is B tile b_first + u.
+// particles at their home slots in state_b.
 struct Ranges {
     float4 *state_a;
-    const unsigned int *a_live;
+    const unsigned int *a_live;   // nullptr: no particle has been sorted yet
     const unsigned int *pidx;
-    int tiles_a;                  // tiles covering an upper bound of the live count
     float4 *state_b;
     const Tile *b_tiles;
     int b_first, n_b;
+    int unit_shift;               // a B tile holds up to 32 << unit_shift particles
+    unsigned int unit_min, unit_max;   // the launch runs if it has that many warps of particles
     float *w_a, *w_b;             // Langevin w' of A (sorted) and B (home) slots, or nullptr
     // when the next sort takes exactly this launch's particles as its inputs (A slots, then
     // the B tiles lane by lane): their sort keys and histogram (zeroed before the launch),
-    // written at the segment's end so that the sort skips its key pass; else nullptr (one
-    // scenario only: the mixed-scenario instantiations carry no key code)
+    // written at the segment's end so that the sort skips its key pass; else nullptr
     unsigned int *keys, *hist;
 };
 
@@ -58,13 +57,11 @@ struct AdvanceLaunch {
     cudaStream_t stream;
     const StepParams *params;
     Ranges ranges;
-    unsigned int *queue;      // work-queue counter (zeroed before the launch), or nullptr:
-                              // then block b takes tiles b, b + grid, ...
+    unsigned int *queue;      // work-queue counter (zeroed before the launch)
     int k0, k1, do_bin;
-    int block, ppt, occ;
+    int block, occ;
     bool mixed;               // lanes of one tile may belong to different scenarios
     unsigned int grid;
-    int n_tiles() const { return ranges.tiles_a + ranges.n_b; }
     int variant() const { return adv_variant(*params); }
 };
 
