@@ -689,7 +689,8 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
 
             // ---- sort keys for the sort that follows (its inputs: A slots, then B lanes) ----
             if (R.keys) {
-                const unsigned int dead_key = (unsigned int)sort_key_range(P.nx, P.ny, P.nz);
+                const unsigned int dead_key =
+                    (unsigned int)sort_dead_key(P.nx, P.ny, P.nz, R.key_shift, 0);
                 long long idx = -1;
                 unsigned int key = KEY_NONE_U;
                 if (in_a) {
@@ -703,14 +704,12 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                     axis(x, P.x0, P.inv_dx, P.nx2, ix, fa);
                     axis(y, P.y0, P.inv_dy, P.ny2, jy, fb);
                     level(P, LV, z, kz, fc);
-                    key = cell_key(P, ix, jy, kz);
+                    key = cell_key(P, ix, jy, kz) >> R.key_shift;
                 } else if (lane < count) {
                     key = dead_key;
                 }
                 if (idx >= 0) R.keys[idx] = key;
-                const unsigned int peers = __match_any_sync(0xffffffffu, key);
-                if (key != KEY_NONE_U && lane == __ffs(peers) - 1)
-                    atomicAdd(R.hist + key, (unsigned int)__popc(peers));
+                sort_count(R.counts, key);
             }
 
             // ---- end-of-segment concentration snapshot (every n-th step, Sec. 3.2) --------

@@ -123,7 +123,9 @@ struct lpm_ctx {
     unsigned int *d_slot_of = nullptr;      // per home slot: sorted slot, grave index or home
     unsigned int *d_keys = nullptr;
     size_t keys_cap = 0;
-    unsigned int *d_hist = nullptr, *d_bsums = nullptr, *d_live = nullptr;   // d_live = meta[4]
+    SortCounts counts{nullptr, nullptr};    // zero between sorts; counts_dirty: a failed call
+    bool counts_dirty = false;              // may have left some
+    unsigned int *d_offsets = nullptr, *d_live = nullptr;   // d_live = meta[4]
     float4 *d_grave = nullptr;              // particles found dead at a sort (read-back only)
     unsigned int *d_grave_n = nullptr;
     unsigned int *d_grave_home = nullptr;   // home slot of each entry of d_grave
@@ -183,8 +185,9 @@ struct lpm_ctx {
         std::vector<long long> ckoff;           // [n_seg + 1] checkpoint offsets (sorted entries)
         long long max_width = 0;
         Tile *d_tiles = nullptr;
-        unsigned int *ord = nullptr, *live = nullptr, *keys = nullptr, *hist = nullptr,
-                     *bsums = nullptr, *meta = nullptr, *slot_of = nullptr, *grave_n = nullptr;
+        unsigned int *ord = nullptr, *live = nullptr, *keys = nullptr, *offsets = nullptr,
+                     *meta = nullptr, *grave_n = nullptr;
+        SortCounts counts{nullptr, nullptr};
         float4 *st[2] = {nullptr, nullptr};
         float4 *home = nullptr, *mu = nullptr, *grave = nullptr;
     } as;
@@ -639,8 +642,8 @@ lpm_status ensure_sort_buffers(lpm_ctx *c, size_t keys_need)
 {
     // allocate whatever is still missing (an earlier call may have stopped at a failure)
     const size_t n = (size_t)c->cfg.max_particles;
-    const size_t nb = (size_t)sort_key_range(c->cfg.nx, c->cfg.ny, c->cfg.nz) + 1;
-    const size_t ntiles = (nb + 1023) / 1024;
+    const size_t ntiles = (size_t)scan_tiles(sort_key_range(c->cfg.nx, c->cfg.ny, c->cfg.nz) + 1);
+    const size_t nb = ntiles * SCAN_TILE;
     auto need = [&](auto *&p, size_t bytes) -> cudaError_t {
         if (p) return cudaSuccess;
         drop_graphs(c);                      // graphs hold the buffers' addresses
@@ -654,8 +657,15 @@ lpm_status ensure_sort_buffers(lpm_ctx *c, size_t keys_need)
         LPM_CUDA(c, need(c->d_slot_of, n * sizeof(unsigned int)));
         LPM_CUDA(c, cudaMemsetAsync(c->d_slot_of, 0xff, n * sizeof(unsigned int), c->stream));
     }
-    LPM_CUDA(c, need(c->d_hist, nb * sizeof(unsigned int)));
-    LPM_CUDA(c, need(c->d_bsums, ntiles * sizeof(unsigned int)));
+    LPM_CUDA(c, need(c->d_offsets, nb * sizeof(unsigned int)));
+    if (!c->counts.keys || !c->counts.tiles) c->counts_dirty = true;
+    LPM_CUDA(c, need(c->counts.keys, nb * sizeof(unsigned int)));
+    LPM_CUDA(c, need(c->counts.tiles, ntiles * sizeof(unsigned int)));
+    if (c->counts_dirty) {
+        LPM_CUDA(c, cudaMemsetAsync(c->counts.keys, 0, nb * sizeof(unsigned int), c->stream));
+        LPM_CUDA(c, cudaMemsetAsync(c->counts.tiles, 0, ntiles * sizeof(unsigned int), c->stream));
+        c->counts_dirty = false;
+    }
     if (!c->d_live) {
         LPM_CUDA(c, need(c->d_live, 4 * sizeof(unsigned int)));
         LPM_CUDA(c, cudaMemsetAsync(c->d_live, 0, 4 * sizeof(unsigned int), c->stream));
@@ -870,7 +880,7 @@ void lpm_destroy(lpm_ctx *c)
                     c->d_err, c->d_queue, c->d_m0, c->d_scen, c->d_woff, c->d_tiles,
                     c->d_zlut, c->d_mq, c->d_qi, c->d_ckpt, c->d_rec, c->d_rC, c->d_rw,
                     c->d_rgrad, c->d_adj_tiles, c->d_sorted[0], c->d_sorted[1], c->d_pidx[0],
-                    c->d_pidx[1], c->d_slot_of, c->d_keys, c->d_hist, c->d_bsums, c->d_live,
+                    c->d_pidx[1], c->d_slot_of, c->d_keys, c->counts.keys, c->counts.tiles, c->d_offsets, c->d_live,
                     c->d_grave, c->d_grave_n, c->d_grave_home, c->d_dose, c->d_bl, c->d_blpair,
                     c->d_sp_conc, c->d_sp_dep, c->d_w_home, c->d_w_sorted[0],
                     c->d_w_sorted[1], c->d_traj, c->d_fin, c->d_traj_tile, c->d_conv,
@@ -879,8 +889,8 @@ void lpm_destroy(lpm_ctx *c)
         if (p) cudaFree(p);
     {
         lpm_ctx::AdjSorted &S = c->as;
-        void *aps[] = {S.d_tiles, S.ord, S.live, S.keys, S.hist, S.bsums, S.meta, S.slot_of,
-                       S.grave_n, S.st[0], S.st[1], S.home, S.mu, S.grave};
+        void *aps[] = {S.d_tiles, S.ord, S.live, S.keys, S.counts.keys, S.counts.tiles, S.offsets,
+                       S.meta, S.grave_n, S.st[0], S.st[1], S.home, S.mu, S.grave};
         for (void *p : aps)
             if (p) cudaFree(p);
     }
@@ -1263,6 +1273,7 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
     const bool batched = g.n_scenarios > 1;
     const int T = tile_particles(c);
     const size_t ns = (size_t)g.n_scenarios;
+    const int key_shift = sort_key_shift(c->n_slots_used);
     bool keys_ready = false;                 // the previous launch wrote the sort's keys
     LPM_CUDA(c, cudaMemsetAsync(c->d_queue, 0, plan.size() * sizeof(unsigned int), s));
     for (size_t gi = 0; gi < plan.size(); ++gi) {
@@ -1293,7 +1304,8 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
             in.tiles = c->d_tiles;
             in.b_first = sg.sort_b_lo;
             in.n_b = sg.sort_b_hi - sg.sort_b_lo;
-            in.T = T;
+            while ((1 << in.t_shift) < T) ++in.t_shift;
+            in.key_shift = key_shift;
             in.w_a = c->langevin ? c->d_w_sorted[cur] : nullptr;
             in.w_b = c->langevin ? c->d_w_home : nullptr;
             in.keys_ready = keys_ready;
@@ -1303,8 +1315,8 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
             out.slot_of = nullptr;               // rebuilt on request (ensure_slot_map)
             out.grave_home = c->d_grave_home;
             out.keys = c->d_keys;
-            out.hist = c->d_hist;
-            out.block_sums = c->d_bsums;
+            out.offsets = c->d_offsets;
+            out.counts = c->counts;
             out.meta = c->d_live;
             out.grave = c->d_grave;
             out.grave_count = c->d_grave_n;
@@ -1315,7 +1327,7 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
             c->slot_map_stale = true;
             cur = 1 - cur;
             upto = sg.k;
-            kernels += keys_ready ? 6 : 7;
+            kernels += keys_ready ? 2 : 3;
         }
         AdvanceLaunch L{};
         L.stream = s;
@@ -1345,10 +1357,9 @@ lpm_status run_segments(lpm_ctx *c, const StepParams &P, const std::vector<Segme
         const Segment *nx = gi + 1 < plan.size() ? &plan[gi + 1] : nullptr;
         if (nx && nx->sort && nx->sort_b_lo == sg.b_lo && nx->sort_b_hi == sg.b_hi &&
             nx->sort_a_bound == (upto > 0 ? sg.a_bound : 0)) {
-            const size_t nb = (size_t)sort_key_range(g.nx, g.ny, g.nz) + 1;
-            LPM_CUDA(c, cudaMemsetAsync(c->d_hist, 0, nb * sizeof(unsigned int), s));
             L.ranges.keys = c->d_keys;
-            L.ranges.hist = c->d_hist;
+            L.ranges.counts = c->counts;
+            L.ranges.key_shift = key_shift;
             keys_ready = true;
         }
         // persistent grid over an atomic tile queue, one counter per launch of the call
@@ -1483,7 +1494,10 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
         long long kernels = 0;
         st = run_segments(c, P, plan, c->stream, c->sorted_upto, c->cur, kernels, true);
         c->n_launches += kernels;
-        if (st != LPM_OK) return st;
+        if (st != LPM_OK) {
+            c->counts_dirty = true;
+            return st;
+        }
     } else {
         // the whole call as one graph, captured once per (steps, starting sort state) on a
         // private stream (the caller's may be the legacy stream, which cannot be captured)
@@ -2112,15 +2126,20 @@ lpm_status adj_sorted_buffers(lpm_ctx *c)
     lpm_ctx::AdjSorted &S = c->as;
     const size_t ns = std::max<size_t>(1, (size_t)c->n_slots_used);
     const size_t nseg = S.tiles_a.size();
-    const size_t nb = (size_t)sort_dead_key(c->cfg.nx, c->cfg.ny, c->cfg.nz, adj_key_scen(c)) + 1;
+    const size_t ntiles = (size_t)scan_tiles(
+        sort_dead_key(c->cfg.nx, c->cfg.ny, c->cfg.nz, 0, adj_key_scen(c)) + 1);
+    const size_t nb = ntiles * SCAN_TILE;
     auto need = [&](auto *&p, size_t bytes) -> cudaError_t {
         return p ? cudaSuccess : cudaMalloc(&p, bytes);
     };
     LPM_CUDA(c, need(S.ord, std::max<size_t>(1, nseg) * ns * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.live, std::max<size_t>(1, nseg) * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.keys, (size_t)std::max<long long>(1, S.max_width) * sizeof(unsigned int)));
-    LPM_CUDA(c, need(S.hist, nb * sizeof(unsigned int)));
-    LPM_CUDA(c, need(S.bsums, ((nb + 1023) / 1024) * sizeof(unsigned int)));
+    LPM_CUDA(c, need(S.offsets, nb * sizeof(unsigned int)));
+    LPM_CUDA(c, need(S.counts.keys, nb * sizeof(unsigned int)));
+    LPM_CUDA(c, need(S.counts.tiles, ntiles * sizeof(unsigned int)));
+    LPM_CUDA(c, cudaMemsetAsync(S.counts.keys, 0, nb * sizeof(unsigned int), c->stream));
+    LPM_CUDA(c, cudaMemsetAsync(S.counts.tiles, 0, ntiles * sizeof(unsigned int), c->stream));
     LPM_CUDA(c, need(S.meta, 4 * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.grave_n, sizeof(unsigned int)));
     for (float4 **p : {&S.st[0], &S.st[1], &S.home, &S.mu, &S.grave})
@@ -2181,9 +2200,11 @@ lpm_status adj_forward_sorted(lpm_ctx *c, const StepParams &P, const AdjParams &
             in.tiles = S.d_tiles;
             in.b_first = G.b_first;
             in.n_b = S.seg_tile[(size_t)s + 1] - G.b_first;
-            in.T = ADJ_BLOCK;
+            in.t_shift = 0;
+            while ((1 << in.t_shift) < ADJ_BLOCK) ++in.t_shift;
+            in.key_shift = sort_key_shift(c->n_slots_used);
             in.w_a = in.w_b = nullptr;
-            in.keys_ready = false;
+            in.keys_ready = false;       // (writing them in the forward cost it 1 to 2 %)
             in.key_scen = adj_key_scen(c);
             SortBuffers out;
             out.state_out = S.st[cur ^ 1];
@@ -2191,8 +2212,8 @@ lpm_status adj_forward_sorted(lpm_ctx *c, const StepParams &P, const AdjParams &
             out.slot_of = nullptr;                // the adjoint reads no slot map
             out.grave_home = nullptr;
             out.keys = S.keys;
-            out.hist = S.hist;
-            out.block_sums = S.bsums;
+            out.offsets = S.offsets;
+            out.counts = S.counts;
             out.meta = S.meta;
             out.grave = S.grave;
             out.grave_count = S.grave_n;
@@ -2200,7 +2221,7 @@ lpm_status adj_forward_sorted(lpm_ctx *c, const StepParams &P, const AdjParams &
             out.cap = std::max<long long>(1, c->n_slots_used);
             out.err = c->d_err;
             LPM_CUDA(c, launch_sort(c->stream, P, in, out));
-            c->n_launches += 7;
+            c->n_launches += 3;
             cur ^= 1;
         }
     }

@@ -17,6 +17,17 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// Counts of a sort: particles per key, and per tile of SCAN_TILE keys. Zero except between
+// the pass that writes the keys and the sort that uses them up. Both padded to whole tiles.
+constexpr int SCAN_TILE_BITS = 12;
+constexpr int SCAN_TILE = 1 << SCAN_TILE_BITS;
+
+struct SortCounts {
+    unsigned int *keys, *tiles;
+};
+
+inline long long scan_tiles(long long n_keys) { return (n_keys + SCAN_TILE - 1) / SCAN_TILE; }
+
 // The particles of an advance launch. A = the sorted live particles [0, live) of state_a
 // (live count on the device; home slot of sorted slot i in pidx[i]; any scenario);
 // B = tiles [b_first, b_first + n_b) of the tile table, each a run of one scenario's
@@ -32,9 +43,11 @@ struct Ranges {
     unsigned int unit_min, unit_max;   // the launch runs if it has that many warps of particles
     float *w_a, *w_b;             // Langevin w' of A (sorted) and B (home) slots, or nullptr
     // when the next sort takes exactly this launch's particles as its inputs (A slots, then
-    // the B tiles lane by lane): their sort keys and histogram (zeroed before the launch),
-    // written at the segment's end so that the sort skips its key pass; else nullptr
-    unsigned int *keys, *hist;
+    // the B tiles lane by lane): their sort keys and counts, written at the segment's end so
+    // that the sort skips its key pass; else nullptr
+    unsigned int *keys;
+    SortCounts counts;
+    int key_shift;
 };
 
 // Longest launch in steps: its step times sit in a table in shared memory.
@@ -74,9 +87,10 @@ struct SortSource {
     long long a_bound;            // upper bound of the live count
     const float4 *state_b;
     const Tile *tiles;
-    int b_first, n_b, T;
+    int b_first, n_b, t_shift;    // T = 1 << t_shift
     const float *w_a, *w_b;       // Langevin w' (moved with the particles), or nullptr
-    bool keys_ready;              // keys and histogram already written (fused key pass)
+    bool keys_ready;              // keys and counts already written (fused key pass)
+    int key_shift;                // cell keys are cell_key >> key_shift
     int key_scen;                 // 0: cell keys; n > 0: keys (scenario, cell tile) over n
                                   // scenarios, scenario-major (sort_dead_key)
 };
@@ -87,7 +101,8 @@ struct SortBuffers {
     unsigned int *slot_of;        // per home slot: sorted slot, GRAVE | index, or SLOT_HOME;
                                   // nullptr: not kept (launch_slot_map rebuilds it)
     unsigned int *grave_home;     // home slot of each dead-particle entry, or nullptr
-    unsigned int *keys, *hist, *block_sums, *meta;
+    unsigned int *keys, *offsets, *meta;   // offsets: first place of each key
+    SortCounts counts;
     float4 *grave;
     unsigned int *grave_count;
     float *w_out;                 // Langevin w' of the sorted particles, or nullptr
@@ -112,10 +127,32 @@ constexpr unsigned int KEY_NONE_U = 0xffffffffu;     // sort input that is no pa
 // Key of the particles that left the working set (the last key of a sort): after the cell
 // keys, or after key_scen scenarios' tile keys (scenario s, tile t: s * tiles + t, one
 // key per tile of 2^(2 SORT_TILE_BITS + SORT_TILE_ZBITS) cells).
-__host__ __device__ inline long long sort_dead_key(int nx, int ny, int nz, int key_scen)
+constexpr int SORT_CELL_BITS = 2 * SORT_TILE_BITS + SORT_TILE_ZBITS;   // cells of a tile, log2
+
+__host__ __device__ inline long long sort_dead_key(int nx, int ny, int nz, int key_shift,
+                                                   int key_scen)
 {
     const long long r = sort_key_range(nx, ny, nz);
-    return key_scen > 0 ? (long long)key_scen * (r >> (2 * SORT_TILE_BITS + SORT_TILE_ZBITS)) : r;
+    return key_scen > 0 ? (long long)key_scen * (r >> SORT_CELL_BITS) : r >> key_shift;
+}
+
+// Cell keys of a sort of at most n particles: whole cells, or cell tiles where there are few
+// particles a tile anyway (their order within it is of no use, and 64 times fewer keys are
+// counted and scanned).
+inline int sort_key_shift(long long n) { return n <= (1 << 17) ? SORT_CELL_BITS : 0; }
+
+// Counts a key (KEY_NONE_U: none), one atomic per key and per tile of keys present in the
+// warp. Every lane of the warp must call it.
+__device__ __forceinline__ void sort_count(const SortCounts &C, unsigned int key)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned int peers = __match_any_sync(0xffffffffu, key);
+    if (key != KEY_NONE_U && lane == __ffs(peers) - 1)
+        atomicAdd(C.keys + key, (unsigned int)__popc(peers));
+    const unsigned int tile = key != KEY_NONE_U ? key >> SCAN_TILE_BITS : KEY_NONE_U;
+    const unsigned int near = __match_any_sync(0xffffffffu, tile);
+    if (tile != KEY_NONE_U && lane == __ffs(near) - 1)
+        atomicAdd(C.tiles + tile, (unsigned int)__popc(near));
 }
 
 // Key of cell (ix, jy, kz): its tile, then its place in the tile.
