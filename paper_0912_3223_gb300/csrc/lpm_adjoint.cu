@@ -153,6 +153,24 @@ __device__ __forceinline__ void receptors_near(const AdjParams &A, float x, floa
     hi = __ldg(A.rbin_off + b + 1);
 }
 
+// Adds mass m at (x, y, z) to the receptor sums C[r] (shared or global).
+__device__ __forceinline__ void sample_receptors(const AdjParams &A, const float4 *s_rec, float x,
+                                                 float y, float z, float m, double *C)
+{
+    int lo, hi;
+    receptors_near(A, x, y, lo, hi);
+    for (int t = lo; t < hi; ++t) {
+        const int r = __ldg(A.rbin_idx + t);
+        const float4 q = s_rec[r];
+        const float dx = x - q.x, dy = y - q.y, dz = z - q.z, dzi = z + q.z;
+        const float h2 = dx * dx + dy * dy;
+        const float d1 = h2 + dz * dz, d2 = h2 + dzi * dzi;
+        if (d1 > A.cut2 && d2 > A.cut2) continue;
+        const float G = A.norm * (expf(-d1 * A.inv2s2) + expf(-d2 * A.inv2s2));
+        atomicAdd(C + r, (double)(m * G));
+    }
+}
+
 // ---------------------------------------------------------------------------------
 // Forward: receptor concentrations, and checkpoints or the whole trajectory.
 // ---------------------------------------------------------------------------------
@@ -214,18 +232,7 @@ adj_forward_kernel(const StepParams P, const AdjParams A)
             }
             if ((k + 1) % A.every == 0) {
                 const float m = m0 * expf(-P.lambda * (float)(k + 1 - sp) * P.dt) * A.inv_ns;
-                int lo, hi;
-                receptors_near(A, x, y, lo, hi);
-                for (int t = lo; t < hi; ++t) {
-                    const int r = __ldg(A.rbin_idx + t);
-                    const float4 q = s_rec[r];
-                    const float dx = x - q.x, dy = y - q.y, dz = z - q.z, dzi = z + q.z;
-                    const float h2 = dx * dx + dy * dy;
-                    const float d1 = h2 + dz * dz, d2 = h2 + dzi * dzi;
-                    if (d1 > A.cut2 && d2 > A.cut2) continue;
-                    const float G = A.norm * (expf(-d1 * A.inv2s2) + expf(-d2 * A.inv2s2));
-                    atomicAdd(&s_C[r], (double)(m * G));
-                }
+                sample_receptors(A, s_rec, x, y, z, m, s_C);
             }
         }
         if (TRAJ)
@@ -252,14 +259,14 @@ struct Adjoint {
 // A.w) for a particle whose scenario is not its block's.
 template <bool KHG, class LEV>
 __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParams &A,
-                                             const LEV &LV, const ScenDev &sc,
+                                             const LEV &LV, const StepTime &T,
                                              const float4 *s_rec, const float *s_w,
                                              unsigned long long gid, int sp, float m0, float mq,
-                                             float sig_h_uniform, float sq2dt, int k, float4 X,
+                                             float sig_h_uniform, float sq2dt, float4 X,
                                              float fold, float4 Xa, bool sample, Adjoint &J,
-                                             const double *wg = nullptr,
-                                             const float4 *ta = nullptr, int ta_k0 = 0)
+                                             const double *wg = nullptr)
 {
+    const int k = T.k;
     if (sample) {
         const float decay = expf(-P.lambda * (float)(k + 1 - sp) * P.dt);
         const float m = m0 * decay;
@@ -282,21 +289,23 @@ __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParam
             J.gq += wr * mq * decay * (e1 + e2);
         }
     }
-    const StepTime T = ta ? step_time_from(P, sc.wind_offset, ta[k - ta_k0], k)
-                          : step_time(P, sc.wind_offset, k);
     float val[5], g[5][3];
     sample_met_grad<KHG>(P, LV, T, sig_h_uniform, X.x, X.y, X.z, val, g);
-    const U4 w = philox4x32_10((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u,
-                               P.seed_lo, P.seed_hi);
+    const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
     float n0, n1, n2;
     normals3(w, n0, n1, n2);
-    const float kh = P.k_scale * val[4], kz = P.k_scale * val[3];
-    const float sig_h = sqrtf(2.0f * kh * P.dt), sig_z = sqrtf(2.0f * kz * P.dt);
-    const float ch = val[4] > 0.0f ? sq2dt / (2.0f * sqrtf(val[4])) : 0.0f;
+    const float kz = P.k_scale * val[3];
+    const float sig_z = sqrtf(2.0f * kz * P.dt);
     const float cz = val[3] > 0.0f ? sq2dt / (2.0f * sqrtf(val[3])) : 0.0f;
+    // a uniform K_h has one scale for the run and no gradient
+    float sig_h = sig_h_uniform, ch = 0.0f;
+    if (KHG) {
+        const float kh = P.k_scale * val[4];
+        sig_h = sqrtf(2.0f * kh * P.dt);
+        ch = val[4] > 0.0f ? sq2dt / (2.0f * sqrtf(val[4])) : 0.0f;
+    }
     // parameter partials: s_K, b_u, b_v
-    const float inv2sk = 0.5f / P.k_scale;
-    J.gsk += (J.mu0 * n0 * sig_h + J.mu1 * n1 * sig_h + J.mu2 * fold * n2 * sig_z) * inv2sk;
+    J.gsk += (J.mu0 * n0 * sig_h + J.mu1 * n1 * sig_h + J.mu2 * fold * n2 * sig_z) * A.inv2sk;
     J.gbu += J.mu0 * P.dt;
     J.gbv += J.mu1 * P.dt;
     // mu <- J^T mu
@@ -304,8 +313,8 @@ __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParam
     float nm[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const float jx = P.dt * g[0][d] + n0 * ch * g[4][d];
-        const float jy = P.dt * g[1][d] + n1 * ch * g[4][d];
+        const float jx = KHG ? P.dt * g[0][d] + n0 * ch * g[4][d] : P.dt * g[0][d];
+        const float jy = KHG ? P.dt * g[1][d] + n1 * ch * g[4][d] : P.dt * g[1][d];
         const float jz = P.dt * g[2][d] + n2 * cz * g[3][d];
         nm[d] = J.mu0 * jx + J.mu1 * jy + mz * jz;
     }
@@ -314,7 +323,7 @@ __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParam
     J.mu2 = mz + nm[2];
 }
 
-// Sums of the block's particles (FP64) and one atomic per parameter per block: the source
+// Sums of a group's particles (FP64) and one atomic per parameter and group: the source
 // partials are the sum of mu at release.
 __device__ __forceinline__ void reduce_gradient(const AdjParams &A, const Tile &tile, Adjoint J,
                                                 bool valid, int qidx, double *s_g, double *s_gq)
@@ -331,22 +340,24 @@ __device__ __forceinline__ void reduce_gradient(const AdjParams &A, const Tile &
     if (J.gq != 0.f) atomicAdd(&s_gq[qidx], (double)J.gq);
     __syncthreads();
     double *G = A.grad + (long long)tile.scen * A.ng;
-    if (threadIdx.x < 3) atomicAdd(G + threadIdx.x, s_g[threadIdx.x]);
-    else if (threadIdx.x < 6) atomicAdd(G + 3 + A.nq + (threadIdx.x - 3), s_g[threadIdx.x]);
-    for (int i = threadIdx.x; i < A.nq; i += ADJ_BLOCK)
+    const int lane = threadIdx.x % ADJ_BLOCK;
+    if (lane < 6 && s_g[lane] != 0.0)
+        atomicAdd(G + (lane < 3 ? lane : A.nq + lane), s_g[lane]);
+    for (int i = lane; i < A.nq; i += ADJ_BLOCK)
         if (s_gq[i] != 0.0) atomicAdd(G + 3 + i, s_gq[i]);
 }
 
-// Receptors and per-scenario dL/dC (scaled by 1 / samples) into shared memory.
+// Receptors and the group's scenario's dL/dC (scaled by 1 / samples) into shared memory.
 __device__ __forceinline__ void load_receptors(const AdjParams &A, const Tile &tile, float4 *s_rec,
                                                float *s_w, double *s_g, double *s_gq)
 {
-    for (int r = threadIdx.x; r < A.R; r += ADJ_BLOCK) {
-        s_rec[r] = A.rec[r];
+    const int lane = threadIdx.x % ADJ_BLOCK;
+    for (int r = lane; r < A.R; r += ADJ_BLOCK) {
+        if (threadIdx.x < ADJ_BLOCK) s_rec[r] = A.rec[r];
         s_w[r] = (float)(A.w[(long long)tile.scen * A.R + r] * (double)A.inv_ns);
     }
-    for (int i = threadIdx.x; i < A.nq; i += ADJ_BLOCK) s_gq[i] = 0.0;
-    if (threadIdx.x < 6) s_g[threadIdx.x] = 0.0;
+    for (int i = lane; i < A.nq; i += ADJ_BLOCK) s_gq[i] = 0.0;
+    if (lane < 6) s_g[lane] = 0.0;
     __syncthreads();
 }
 
@@ -421,8 +432,9 @@ adj_backward_kernel(const StepParams P, const AdjParams A)
             if (!(run && k >= kstart && k <= klast)) continue;
             const int i = k - k_lo;
             const bool sample = (k + 1) % A.every == 0 && !(ev && k == klast);
-            reverse_step<KHG>(P, A, LV, sc, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt, k,
-                         seg[i], (float)sfold[i], seg[i + 1], sample, J);
+            reverse_step<KHG>(P, A, LV, step_time(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0,
+                              mq, sig_h_uniform, sq2dt, seg[i], (float)sfold[i], seg[i + 1],
+                              sample, J);
         }
         __syncwarp();
     }
@@ -482,8 +494,8 @@ adj_backward_traj_kernel(const StepParams P, const AdjParams A)
             Xn = __ldcs(row + (long long)(k - 1 - k0) * ADJ_BLOCK);
         if (!act) continue;
         const bool sample = (k + 1) % A.every == 0 && !(ev && k == kn - 1);
-        reverse_step<KHG>(P, A, LV, sc, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt, k, X,
-                     X.w, Xa, sample, J);
+        reverse_step<KHG>(P, A, LV, step_time(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0, mq,
+                          sig_h_uniform, sq2dt, X, X.w, Xa, sample, J);
         Xa = X;
     }
     reduce_gradient(A, tile, J, valid, qidx, s_g, s_gq);
@@ -493,15 +505,15 @@ adj_backward_traj_kernel(const StepParams P, const AdjParams A)
 // level table
 // (small arrays keep the shared-memory carve-out small and leave the rest of the SM's
 // unified L1 to the weather gathers).
-static size_t adj_smem_forward(const StepParams &P, const AdjParams &A)
+static size_t adj_smem_forward(const StepParams &P, const AdjParams &A, int groups = 1)
 {
-    return (size_t)A.R * (sizeof(float4) + sizeof(double)) + (size_t)P.n_lut;
+    return (size_t)A.R * (sizeof(float4) + groups * sizeof(double)) + (size_t)P.n_lut;
 }
 
-static size_t adj_smem_backward(const StepParams &P, const AdjParams &A)
+static size_t adj_smem_backward(const StepParams &P, const AdjParams &A, int groups = 1)
 {
-    return (size_t)A.R * (sizeof(float4) + sizeof(float)) + (size_t)(6 + A.nq) * sizeof(double) +
-           (size_t)P.n_lut;
+    return (size_t)A.R * (sizeof(float4) + groups * sizeof(float)) +
+           (size_t)groups * (6 + A.nq) * sizeof(double) + (size_t)P.n_lut;
 }
 
 // ---------------------------------------------------------------------------------
@@ -510,16 +522,29 @@ static size_t adj_smem_backward(const StepParams &P, const AdjParams &A)
 // releases; between segments the survivors are re-sorted (lpm_sort.cu). The states of a
 // segment are stored row by row in that order; the backward sweeps the segments in
 // reverse and hands dL/dX from one segment to the previous one through G.mu, indexed by
-// home slot. A block keeps the receptor sums and gradients of one scenario (its first
-// entry's) in shared memory; entries of another scenario, at a scenario boundary of the
-// sorted order, add theirs to the global sums directly.
+// home slot. A group of ADJ_BLOCK entries keeps the receptor sums and gradients of one
+// scenario (its first entry's) in shared memory; entries of another scenario, at a scenario
+// boundary of the sorted order, add theirs to the global sums directly.
 // ---------------------------------------------------------------------------------
+
+// Threads of the segment kernels' blocks, in groups of ADJ_BLOCK entries with receptor sums of
+// their own. The forwards take two groups a block: neighbours in the sorted order then share
+// the SM's L1 at nearly the same step (hits 86 -> 92 %) and one copy of the tables, of which
+// more would cost blocks; 4 a SM (64 registers) with the trajectory, 3 (80) without, where
+// the row stores do not hold it up (1e6 x 1080 and 2e5 x 720 with checkpoints, whole gradients:
+// 15.8 and 5.3 ms; 4 and 4: 15.8 and 5.7; 3 and 3: 16.0 and 5.4; blocks of 512: 15.9 and 5.7).
+// The reverse sweep at 5 blocks of 128 a SM (96 registers): blocks of 256 at 2 or 3 a SM 16.1 and
+// 16.7 ms, of 384 16.4, of 640 16.6.
+constexpr int SEG_FWD_BLOCK = 256, SEG_BWD_BLOCK = 128;
+
 template <bool MULTI>
-__device__ __forceinline__ bool seg_entry(const StepParams &P, const AdjSeg &G, long long e,
+__device__ __forceinline__ bool seg_entry(const StepParams &P, const AdjSeg &G, int group,
                                           bool from_a, unsigned int live, long long &home,
                                           int &scen)
 {
+    const int lane = threadIdx.x % ADJ_BLOCK;
     if (from_a) {
+        const long long e = (long long)group * ADJ_BLOCK + lane;
         if (e >= (long long)live) {
             scen = 0;
             home = P.scen[0].first_slot;
@@ -529,56 +554,77 @@ __device__ __forceinline__ bool seg_entry(const StepParams &P, const AdjSeg &G, 
         scen = MULTI ? scen_of(P, home) : 0;
         return true;
     }
-    const Tile t = G.tiles[G.b_first + (blockIdx.x - G.tiles_a)];
-    const bool ok = (int)threadIdx.x < t.count;
+    const Tile t = G.tiles[G.b_first + (group - G.tiles_a)];
+    const bool ok = lane < t.count;
     scen = MULTI ? t.scen : 0;
-    home = t.first + (ok ? threadIdx.x : 0);
+    home = t.first + (ok ? lane : 0);
     return ok;
 }
 
-// The block's scenario: that of its first entry (a sorted block starts below the live
-// count, or the launch returned before).
+// The scenario of a group that has entries: that of its first one.
 template <bool MULTI>
-__device__ __forceinline__ int seg_block_scen(const StepParams &P, const AdjSeg &G, bool from_a)
+__device__ __forceinline__ int seg_group_scen(const StepParams &P, const AdjSeg &G, int group,
+                                              bool from_a)
 {
     if (!MULTI) return 0;
-    if (from_a) return scen_of(P, G.ord[(long long)blockIdx.x * ADJ_BLOCK]);
-    return G.tiles[G.b_first + (blockIdx.x - G.tiles_a)].scen;
+    if (from_a) return scen_of(P, G.ord[(long long)group * ADJ_BLOCK]);
+    return G.tiles[G.b_first + (group - G.tiles_a)].scen;
 }
 
-// 8 blocks per SM (64 registers) for the trajectory form; 7 (72 registers, no spills) for
-// the checkpoint form's forward and recomputation, measured 2 % faster there. MULTI:
-// entries of several scenarios (else all of scenario 0).
-template <int MODE, bool MULTI>
-__global__ void __launch_bounds__(ADJ_BLOCK, MODE == SEG_STORE ? 8 : 7)
-adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
+// True when no group of the block starting at `group0` has entries: groups of A at or beyond
+// the live count, groups beyond the segment's.
+__device__ __forceinline__ bool seg_block_empty(const AdjSeg &G, int group0, int n, int n_groups,
+                                                unsigned int live)
+{
+    for (int g = group0; g < min(group0 + n, n_groups); ++g)
+        if (g >= G.tiles_a || (long long)g * ADJ_BLOCK < (long long)live) return false;
+    return true;
+}
+
+// Receptor forward of a segment (MODE: SegMode). MULTI: entries of several scenarios (else
+// all of scenario 0); FIELDS: a gridded K_h. Instructions bound it as they do the advance
+// kernel: the step times come from a table, the deposition words from one block for two
+// steps, the samples by a countdown.
+template <int MODE, bool MULTI, bool FIELDS>
+__global__ void __launch_bounds__(SEG_FWD_BLOCK, MODE == SEG_STORE ? 4 : 3)
+adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
 {
     constexpr bool SAMPLE = MODE != SEG_RECOMPUTE;          // receptor sums, sort inputs
     constexpr bool ROWS = MODE != SEG_CKPT;                 // every state into traj / fin
-    const bool from_a = (int)blockIdx.x < G.tiles_a;
-    const unsigned int live = from_a ? *G.live : 0u;
-    if (from_a && (long long)blockIdx.x * ADJ_BLOCK >= (long long)live) return;
+    constexpr int GROUPS = SEG_FWD_BLOCK / ADJ_BLOCK;
+    const int group0 = blockIdx.x * GROUPS;
+    const unsigned int live = group0 < G.tiles_a ? *G.live : 0u;
+    if (seg_block_empty(G, group0, GROUPS, n_groups, live)) return;
     extern __shared__ float4 s_dyn[];             // sized by the launch: adj_smem_forward
     float4 *s_rec = s_dyn;                        // [R]
-    double *s_C = reinterpret_cast<double *>(s_rec + A.R);    // [R]
-    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_C + A.R);   // [n_lut]
+    double *s_C = reinterpret_cast<double *>(s_rec + A.R);    // [GROUPS][R]
+    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_C + GROUPS * A.R);   // [n_lut]
+    __shared__ float4 s_ta[CK];                   // the segment's step times
     const Levels LV = load_levels(P, s_lut);
-    if (SAMPLE)
-        for (int r = threadIdx.x; r < A.R; r += ADJ_BLOCK) {
-            s_rec[r] = A.rec[r];
-            s_C[r] = 0.0;
-        }
+    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_FWD_BLOCK)
+        s_ta[i] = step_time_parts(P, G.k_lo + i);
+    if (SAMPLE) {
+        for (int r = threadIdx.x; r < A.R; r += SEG_FWD_BLOCK) s_rec[r] = A.rec[r];
+        for (int r = threadIdx.x; r < GROUPS * A.R; r += SEG_FWD_BLOCK) s_C[r] = 0.0;
+    }
     __syncthreads();
-    const int bs = SAMPLE ? seg_block_scen<MULTI>(P, G, from_a) : 0;
-    const float sig_h_uniform = sqrtf(2.0f * P.k_scale * fmaxf(P.kh_uniform, 0.0f) * P.dt);
-    const long long e = (long long)blockIdx.x * ADJ_BLOCK + threadIdx.x;
+    const int group = group0 + threadIdx.x / ADJ_BLOCK;
+    const bool from_a = group < G.tiles_a;
+    const bool used = group < n_groups && (!from_a || (long long)group * ADJ_BLOCK < (long long)live);
+    double *C = s_C + (threadIdx.x / ADJ_BLOCK) * A.R;      // the group's sums
+    const int bs = SAMPLE && used ? seg_group_scen<MULTI>(P, G, group, from_a) : 0;
+    const float sig_h_uniform = sqrtf(P.k2 * fmaxf(P.kh_uniform, 0.0f) * P.dt);
+    const uint32_t tab = shared_addr(s_ta);
+    const long long e = (long long)group * ADJ_BLOCK + threadIdx.x % ADJ_BLOCK;
     long long home;
     int scen;
-    if (seg_entry<MULTI>(P, G, e, from_a, live, home, scen)) {
-        const ScenDev sc = P.scen[scen];
-        const unsigned long long gid = (unsigned long long)(sc.id0 + (home - sc.first_slot));
+    if (used && seg_entry<MULTI>(P, G, group, from_a, live, home, scen)) {
+        const ScenDev &sc = P.scen[scen];
+        const unsigned long long gid =
+            (unsigned long long)(__ldg(&sc.id0) + (home - __ldg(&sc.first_slot)));
         const int sp = (int)release_step_of(sc, home);
         const float m0 = __ldg(P.m0 + sc.m0_off + (sp - sc.rel_first));
+        const float2 *wind = sc.wind_offset;
         float x = sc.src_x, y = sc.src_y, z = sc.src_z;
         if (from_a) {
             const float4 s0 = MODE == SEG_RECOMPUTE ? G.ck[e] : G.sorted[e];
@@ -586,37 +632,35 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
             x = s0.x; y = s0.y; z = s0.z;
         }
         uint32_t st = ST_ACTIVE;
-        const int k_first = max(sp, G.k_lo);
-        int kn = k_first;                          // one past the last step taken
-        for (int k = k_first; k < G.k_hi; ++k) {
-            const StepTime T = step_time(P, sc.wind_offset, k);
+        int k = max(sp, G.k_lo);
+        float4 *row = ROWS ? G.traj + (long long)(k - G.k_lo) * G.width + e : nullptr;
+        int until = A.every - 1 - k % A.every;     // steps before the next sample step
+        DepCache dc;
+        dep_begin(P, gid, k, dc);
+#pragma unroll 1
+        do {
+            const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
             const float xb = x, yb = y, zb = z;
             float fs = 1.0f;
-            st = particle_step<false>(P, LV, T, sc, nullptr, gid, sp, sig_h_uniform, T.du, T.dv,
-                                      x, y, z, &fs);
-            if (ROWS)
-                __stcs(G.traj + (long long)(k - G.k_lo) * G.width + e, make_float4(xb, yb, zb, fs));
-            kn = k + 1;
-            if (st != ST_ACTIVE) break;
-            if (SAMPLE && (k + 1) % A.every == 0) {
-                const float m = m0 * expf(-P.lambda * (float)(k + 1 - sp) * P.dt) * A.inv_ns;
-                int lo, hi;
-                receptors_near(A, x, y, lo, hi);
-                for (int t = lo; t < hi; ++t) {
-                    const int r = __ldg(A.rbin_idx + t);
-                    const float4 q = s_rec[r];
-                    const float dx = x - q.x, dy = y - q.y, dz = z - q.z, dzi = z + q.z;
-                    const float h2 = dx * dx + dy * dy;
-                    const float d1 = h2 + dz * dz, d2 = h2 + dzi * dzi;
-                    if (d1 > A.cut2 && d2 > A.cut2) continue;
-                    const float Gk = A.norm * (expf(-d1 * A.inv2s2) + expf(-d2 * A.inv2s2));
-                    if (scen == bs) atomicAdd(&s_C[r], (double)(m * Gk));
-                    else atomicAdd(A.C + (long long)scen * A.R + r, (double)(m * Gk));
+            st = particle_step<false, false, Levels, false, FIELDS>(
+                P, LV, T, sc, nullptr, gid, sp, sig_h_uniform, T.du, T.dv, x, y, z,
+                ROWS ? &fs : nullptr, nullptr, nullptr, &dc);
+            if (ROWS) {
+                __stcs(row, make_float4(xb, yb, zb, fs));
+                row += G.width;
+            }
+            ++k;
+            if (SAMPLE && --until < 0) {
+                until = A.every - 1;
+                if (st == ST_ACTIVE) {
+                    const float m = m0 * expf(-P.lambda * (float)(k - sp) * P.dt) * A.inv_ns;
+                    sample_receptors(A, s_rec, x, y, z, m,
+                                     scen == bs ? C : A.C + (long long)scen * A.R);
                 }
             }
-        }
+        } while (st == ST_ACTIVE && k < G.k_hi);
         if (ROWS)
-            G.fin[e] = make_float4(x, y, z, __uint_as_float((uint32_t)kn |
+            G.fin[e] = make_float4(x, y, z, __uint_as_float((uint32_t)k |
                                                             (st != ST_ACTIVE ? 0x80000000u : 0u)));
         if (SAMPLE) {
             const float4 out = pack_state(x, y, z, st, sp);      // what the sort reads
@@ -626,41 +670,55 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
     }
     if (SAMPLE) {
         __syncthreads();
-        for (int r = threadIdx.x; r < A.R; r += ADJ_BLOCK)
-            if (s_C[r] != 0.0) atomicAdd(A.C + (long long)bs * A.R + r, s_C[r]);
+        if (used)
+            for (int r = threadIdx.x % ADJ_BLOCK; r < A.R; r += ADJ_BLOCK)
+                if (C[r] != 0.0) atomicAdd(A.C + (long long)bs * A.R + r, C[r]);
     }
 }
 
+// Reverse sweep of a segment (KHG: gridded K_h). Bound by the latency of its gathers at 19
+// warps an SM (96 registers hold the record differences; issue 56 % busy); a uniform K_h's
+// scale is taken out of the loop, its vanishing derivative dropped (571 -> 480 instructions
+// a step with that, the tabled times and the shared round keys).
 template <bool KHG, bool MULTI>
-__global__ void __launch_bounds__(ADJ_BLOCK, 5)
-adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
+__global__ void __launch_bounds__(SEG_BWD_BLOCK, 5)
+adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
 {
-    const bool from_a = (int)blockIdx.x < G.tiles_a;
-    const unsigned int live = from_a ? *G.live : 0u;
-    if (from_a && (long long)blockIdx.x * ADJ_BLOCK >= (long long)live) return;
+    constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
+    const int group0 = blockIdx.x * GROUPS;
+    const unsigned int live = group0 < G.tiles_a ? *G.live : 0u;
+    if (seg_block_empty(G, group0, GROUPS, n_groups, live)) return;
     extern __shared__ float4 s_dyn[];             // sized by the launch: adj_smem_backward
+    const int gi = threadIdx.x / ADJ_BLOCK;
     float4 *s_rec = s_dyn;                        // [R]
-    double *s_g = reinterpret_cast<double *>(s_rec + A.R);    // [6]
-    double *s_gq = s_g + 6;                       // [nq]
-    float *s_w = reinterpret_cast<float *>(s_gq + A.nq);      // [R]
-    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + A.R);   // [n_lut]
+    double *s_g = reinterpret_cast<double *>(s_rec + A.R);    // [GROUPS][6]
+    double *s_gq = s_g + 6 * GROUPS;              // [GROUPS][nq]
+    float *s_w = reinterpret_cast<float *>(s_gq + GROUPS * A.nq);      // [GROUPS][R]
+    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + GROUPS * A.R);   // [n_lut]
+    s_g += 6 * gi;
+    s_gq += A.nq * gi;
+    s_w += A.R * gi;
     const Levels LV = load_levels(P, s_lut);
-    // the segment's step times, once per block (measured: backward 1 % faster; the forward
-    // kernels, at more blocks per SM, lost more to the extra shared memory than they gained)
+    // the segment's step times, once per block
     __shared__ float4 s_ta[CK];
-    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += ADJ_BLOCK)
+    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_BWD_BLOCK)
         s_ta[i] = step_time_parts(P, G.k_lo + i);
+    const int group = group0 + gi;
+    const bool from_a = group < G.tiles_a;
+    const bool used = group < n_groups && (!from_a || (long long)group * ADJ_BLOCK < (long long)live);
     Tile tb{0, 0, 0};
-    tb.scen = seg_block_scen<MULTI>(P, G, from_a);
+    if (used) tb.scen = seg_group_scen<MULTI>(P, G, group, from_a);
     load_receptors(A, tb, s_rec, s_w, s_g, s_gq);     // (ends with a barrier)
-    const float sig_h_uniform = sqrtf(2.0f * P.k_scale * fmaxf(P.kh_uniform, 0.0f) * P.dt);
+    const float sig_h_uniform = sqrtf(P.k2 * fmaxf(P.kh_uniform, 0.0f) * P.dt);
     const float sq2dt = sqrtf(2.0f * P.k_scale * P.dt);
-    const long long e = (long long)blockIdx.x * ADJ_BLOCK + threadIdx.x;
-    long long home;
-    int scen;
-    const bool valid = seg_entry<MULTI>(P, G, e, from_a, live, home, scen);
-    const ScenDev sc = P.scen[scen];
-    // receptor weights of another scenario than the block's come from global memory
+    const uint32_t tab = shared_addr(s_ta);
+    const long long e = (long long)group * ADJ_BLOCK + threadIdx.x % ADJ_BLOCK;
+    long long home = P.scen[0].first_slot;
+    int scen = 0;
+    const bool valid = used && seg_entry<MULTI>(P, G, group, from_a, live, home, scen);
+    const ScenDev &sc = P.scen[scen];
+    const float2 *wind = sc.wind_offset;
+    // receptor weights of another scenario than the group's come from global memory
     const double *wg = MULTI && scen != tb.scen ? A.w + (long long)scen * A.R : nullptr;
     const unsigned long long gid = (unsigned long long)(sc.id0 + (home - sc.first_slot));
     const int sp = (int)release_step_of(sc, home);
@@ -679,20 +737,26 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
         const float4 m = G.mu[home];
         J.mu0 = m.x; J.mu1 = m.y; J.mu2 = m.z;
     }
-    const int k_top = __reduce_max_sync(0xffffffffu, kn) - 1;
-    const int k_bot = __reduce_min_sync(0xffffffffu, kb < kn ? kb : 0x7fffffff);
-    const float4 *row = G.traj + e;
-    float4 Xn = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k_top >= kb && k_top < kn) Xn = __ldcs(row + (long long)(k_top - G.k_lo) * G.width);
-    for (int k = k_top; k >= k_bot; --k) {
-        const bool act = k >= kb && k < kn;
-        const float4 X = Xn;
-        if (k - 1 >= kb && k - 1 < kn) Xn = __ldcs(row + (long long)(k - 1 - G.k_lo) * G.width);
-        if (!act) continue;
-        const bool sample = (k + 1) % A.every == 0 && !(ev && k == kn - 1);
-        reverse_step<KHG>(P, A, LV, sc, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt, k, X,
-                     X.w, Xa, sample, J, wg, s_ta, G.k_lo);
-        Xa = X;
+    // each lane sweeps its own steps, last first; a row is read one step ahead
+    if (kb < kn) {
+        int k = kn - 1;
+        const float4 *row = G.traj + (long long)(k - G.k_lo) * G.width + e;
+        float4 Xn = __ldcs(row);
+        int since = (k + 1) % A.every;             // 0: step k is a sample step
+        bool first = ev;                           // the step that ended the run has no sample
+#pragma unroll 1
+        do {
+            const float4 X = Xn;
+            row -= G.width;
+            if (k > kb) Xn = __ldcs(row);
+            const bool sample = since == 0 && !first;
+            first = false;
+            since = since == 0 ? A.every - 1 : since - 1;
+            const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
+            reverse_step<KHG>(P, A, LV, T, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt, X,
+                              X.w, Xa, sample, J, wg);
+            Xa = X;
+        } while (--k >= kb);
     }
     // released earlier: hand mu to the previous segment; released here: mu is the
     // particle's share of the source partials
@@ -701,7 +765,7 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
         J.mu0 = J.mu1 = J.mu2 = 0.f;
     }
     if (MULTI && valid && scen != tb.scen) {
-        // another scenario than the block's: its partials straight into its gradient
+        // another scenario than the group's: its partials straight into its gradient
         double *Gs = A.grad + (long long)scen * A.ng;
         atomicAdd(Gs + 0, (double)J.mu0);
         atomicAdd(Gs + 1, (double)J.mu1);
@@ -726,12 +790,12 @@ static void adj_set_carveout()
     cudaFuncSetAttribute(adj_backward_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     cudaFuncSetAttribute(adj_backward_traj_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     const void *seg[] = {
-        (const void *)adj_forward_seg_kernel<SEG_STORE, false>,
-        (const void *)adj_forward_seg_kernel<SEG_CKPT, false>,
-        (const void *)adj_forward_seg_kernel<SEG_RECOMPUTE, false>,
-        (const void *)adj_forward_seg_kernel<SEG_STORE, true>,
-        (const void *)adj_forward_seg_kernel<SEG_CKPT, true>,
-        (const void *)adj_forward_seg_kernel<SEG_RECOMPUTE, true>,
+#define LPM_SEG_FWD_ALL(M) (const void *)adj_forward_seg_kernel<M, false, false>,          \
+                           (const void *)adj_forward_seg_kernel<M, false, true>,            \
+                           (const void *)adj_forward_seg_kernel<M, true, false>,            \
+                           (const void *)adj_forward_seg_kernel<M, true, true>
+        LPM_SEG_FWD_ALL(SEG_STORE), LPM_SEG_FWD_ALL(SEG_CKPT), LPM_SEG_FWD_ALL(SEG_RECOMPUTE),
+#undef LPM_SEG_FWD_ALL
         (const void *)adj_backward_seg_kernel<false, false>,
         (const void *)adj_backward_seg_kernel<true, false>,
         (const void *)adj_backward_seg_kernel<false, true>,
@@ -747,40 +811,46 @@ static void adj_prefer_l1()
 }
 
 cudaError_t launch_adj_forward_seg(cudaStream_t s, const StepParams &P, const AdjParams &A,
-                                   const AdjSeg &G, int n_blocks, int mode)
+                                   const AdjSeg &G, int n_groups, int mode)
 {
-    if (n_blocks <= 0) return cudaSuccess;
+    if (n_groups <= 0) return cudaSuccess;
     adj_prefer_l1();
-    const size_t sm = adj_smem_forward(P, A);
-    const bool multi = P.n_scen > 1;
-#define LPM_SEG_FWD(M)                                                                   \
-    (multi ? adj_forward_seg_kernel<M, true><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G)     \
-           : adj_forward_seg_kernel<M, false><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G))
+    constexpr int GROUPS = SEG_FWD_BLOCK / ADJ_BLOCK;
+    const int n = (n_groups + GROUPS - 1) / GROUPS;
+    const size_t sm = adj_smem_forward(P, A, GROUPS);
+    const bool multi = P.n_scen > 1, fields = P.khpair != nullptr;
+#define LPM_SEG_FWD(M, U, F) adj_forward_seg_kernel<M, U, F><<<n, SEG_FWD_BLOCK, sm, s>>>(P, A, G, n_groups)
+#define LPM_SEG_FWD_MODE(M)                                                              \
+    (multi ? (fields ? LPM_SEG_FWD(M, true, true) : LPM_SEG_FWD(M, true, false))          \
+           : (fields ? LPM_SEG_FWD(M, false, true) : LPM_SEG_FWD(M, false, false)))
     switch (mode) {
-    case SEG_STORE: LPM_SEG_FWD(SEG_STORE); break;
-    case SEG_CKPT: LPM_SEG_FWD(SEG_CKPT); break;
-    case SEG_RECOMPUTE: LPM_SEG_FWD(SEG_RECOMPUTE); break;
+    case SEG_STORE: LPM_SEG_FWD_MODE(SEG_STORE); break;
+    case SEG_CKPT: LPM_SEG_FWD_MODE(SEG_CKPT); break;
+    case SEG_RECOMPUTE: LPM_SEG_FWD_MODE(SEG_RECOMPUTE); break;
     default: return cudaErrorInvalidValue;
     }
+#undef LPM_SEG_FWD_MODE
 #undef LPM_SEG_FWD
     return cudaGetLastError();
 }
 
 cudaError_t launch_adj_backward_seg(cudaStream_t s, const StepParams &P, const AdjParams &A,
-                                    const AdjSeg &G, int n_blocks)
+                                    const AdjSeg &G, int n_groups)
 {
-    if (n_blocks <= 0) return cudaSuccess;
+    if (n_groups <= 0) return cudaSuccess;
     adj_prefer_l1();
-    const size_t sm = adj_smem_backward(P, A);
+    constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
+    const int n = (n_groups + GROUPS - 1) / GROUPS;
+    const size_t sm = adj_smem_backward(P, A, GROUPS);
     const bool multi = P.n_scen > 1;
     if (P.khpair && multi)
-        adj_backward_seg_kernel<true, true><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G);
+        adj_backward_seg_kernel<true, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
     else if (P.khpair)
-        adj_backward_seg_kernel<true, false><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G);
+        adj_backward_seg_kernel<true, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
     else if (multi)
-        adj_backward_seg_kernel<false, true><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G);
+        adj_backward_seg_kernel<false, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
     else
-        adj_backward_seg_kernel<false, false><<<n_blocks, ADJ_BLOCK, sm, s>>>(P, A, G);
+        adj_backward_seg_kernel<false, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
     return cudaGetLastError();
 }
 

@@ -23,6 +23,7 @@ struct AdjParams {
     float inv2s2;                     // 1 / (2 sigma^2)
     float norm;                       // (2 pi sigma^2)^(-3/2)
     float inv_s2;                     // 1 / sigma^2
+    float inv2sk;                     // 0.5 / k_scale
     float cut2;                       // squared distance beyond which a kernel term is dropped
     int every;
     float inv_ns;                     // 1 / number of samples

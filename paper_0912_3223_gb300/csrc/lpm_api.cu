@@ -2543,6 +2543,7 @@ lpm_status adj_prepare(lpm_ctx *c, const double *rec, int R, double bandwidth, i
     A.inv2s2 = (float)(1.0 / (2.0 * s2));
     A.norm = (float)std::pow(2.0 * 3.14159265358979323846 * s2, -1.5);
     A.inv_s2 = (float)(1.0 / s2);
+    A.inv2sk = 0.5f / P.k_scale;
     A.cut2 = (float)(36.0 * s2);
     A.every = every;
     A.inv_ns = (float)(1.0 / n_samp);
