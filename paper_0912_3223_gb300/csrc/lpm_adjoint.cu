@@ -257,7 +257,7 @@ struct Adjoint {
 // Jacobian of step k at the state X before it (fold = the step's reflection sign). The
 // receptor weights dL/dC / n_s come from s_w, or from wg (the particle's scenario's row of
 // A.w) for a particle whose scenario is not its block's.
-template <bool KHG, class LEV>
+template <bool KHG, bool DRAWS_FIRST = false, class LEV>
 __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParams &A,
                                              const LEV &LV, const StepTime &T,
                                              const float4 *s_rec, const float *s_w,
@@ -289,11 +289,14 @@ __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParam
             J.gq += wr * mq * decay * (e1 + e2);
         }
     }
-    float val[5], g[5][3];
+    float val[5], g[5][3], n0, n1, n2;
+    auto draw = [&]() {
+        const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
+        normals3(w, n0, n1, n2);
+    };
+    if (DRAWS_FIRST) draw();
     sample_met_grad<KHG>(P, LV, T, sig_h_uniform, X.x, X.y, X.z, val, g);
-    const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
-    float n0, n1, n2;
-    normals3(w, n0, n1, n2);
+    if (!DRAWS_FIRST) draw();
     const float kz = P.k_scale * val[3];
     const float sig_z = sqrtf(2.0f * kz * P.dt);
     const float cz = val[3] > 0.0f ? sq2dt / (2.0f * sqrtf(val[3])) : 0.0f;
@@ -535,7 +538,17 @@ static size_t adj_smem_backward(const StepParams &P, const AdjParams &A, int gro
 // 15.8 and 5.3 ms; 4 and 4: 15.8 and 5.7; 3 and 3: 16.0 and 5.4; blocks of 512: 15.9 and 5.7).
 // The reverse sweep at 5 blocks of 128 a SM (96 registers): blocks of 256 at 2 or 3 a SM 16.1 and
 // 16.7 ms, of 384 16.4, of 640 16.6.
-constexpr int SEG_FWD_BLOCK = 256, SEG_BWD_BLOCK = 128;
+//
+// FEW: segments of at most 4 groups an SM are bound by a step's latency: one group a block, 128
+// registers a thread, the draws before the gathers so that the two overlap.
+constexpr int SEG_BWD_BLOCK = 128;
+constexpr int seg_fwd_block(bool few) { return few ? 128 : 256; }
+constexpr int SEG_FEW = 4;
+
+constexpr int seg_fwd_blocks(int mode, bool few)
+{
+    return few ? 4 : mode == SEG_STORE ? 4 : 3;
+}
 
 template <bool MULTI>
 __device__ __forceinline__ bool seg_entry(const StepParams &P, const AdjSeg &G, int group,
@@ -585,13 +598,13 @@ __device__ __forceinline__ bool seg_block_empty(const AdjSeg &G, int group0, int
 // all of scenario 0); FIELDS: a gridded K_h. Instructions bound it as they do the advance
 // kernel: the step times come from a table, the deposition words from one block for two
 // steps, the samples by a countdown.
-template <int MODE, bool MULTI, bool FIELDS>
-__global__ void __launch_bounds__(SEG_FWD_BLOCK, MODE == SEG_STORE ? 4 : 3)
+template <int MODE, bool MULTI, bool FIELDS, bool FEW>
+__global__ void __launch_bounds__(seg_fwd_block(FEW), seg_fwd_blocks(MODE, FEW))
 adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
 {
     constexpr bool SAMPLE = MODE != SEG_RECOMPUTE;          // receptor sums, sort inputs
     constexpr bool ROWS = MODE != SEG_CKPT;                 // every state into traj / fin
-    constexpr int GROUPS = SEG_FWD_BLOCK / ADJ_BLOCK;
+    constexpr int BLOCK = seg_fwd_block(FEW), GROUPS = BLOCK / ADJ_BLOCK;
     const int group0 = blockIdx.x * GROUPS;
     const unsigned int live = group0 < G.tiles_a ? *G.live : 0u;
     if (seg_block_empty(G, group0, GROUPS, n_groups, live)) return;
@@ -601,11 +614,11 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
     unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_C + GROUPS * A.R);   // [n_lut]
     __shared__ float4 s_ta[CK];                   // the segment's step times
     const Levels LV = load_levels(P, s_lut);
-    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_FWD_BLOCK)
+    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += BLOCK)
         s_ta[i] = step_time_parts(P, G.k_lo + i);
     if (SAMPLE) {
-        for (int r = threadIdx.x; r < A.R; r += SEG_FWD_BLOCK) s_rec[r] = A.rec[r];
-        for (int r = threadIdx.x; r < GROUPS * A.R; r += SEG_FWD_BLOCK) s_C[r] = 0.0;
+        for (int r = threadIdx.x; r < A.R; r += BLOCK) s_rec[r] = A.rec[r];
+        for (int r = threadIdx.x; r < GROUPS * A.R; r += BLOCK) s_C[r] = 0.0;
     }
     __syncthreads();
     const int group = group0 + threadIdx.x / ADJ_BLOCK;
@@ -642,7 +655,7 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
             const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
             const float xb = x, yb = y, zb = z;
             float fs = 1.0f;
-            st = particle_step<false, false, Levels, false, FIELDS>(
+            st = particle_step<false, false, Levels, false, FIELDS, FEW>(
                 P, LV, T, sc, nullptr, gid, sp, sig_h_uniform, T.du, T.dv, x, y, z,
                 ROWS ? &fs : nullptr, nullptr, nullptr, &dc);
             if (ROWS) {
@@ -680,8 +693,8 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
 // warps an SM (96 registers hold the record differences; issue 56 % busy); a uniform K_h's
 // scale is taken out of the loop, its vanishing derivative dropped (571 -> 480 instructions
 // a step with that, the tabled times and the shared round keys).
-template <bool KHG, bool MULTI>
-__global__ void __launch_bounds__(SEG_BWD_BLOCK, 5)
+template <bool KHG, bool MULTI, bool FEW>
+__global__ void __launch_bounds__(SEG_BWD_BLOCK, FEW ? 4 : 5)
 adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
 {
     constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
@@ -753,8 +766,8 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, i
             first = false;
             since = since == 0 ? A.every - 1 : since - 1;
             const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
-            reverse_step<KHG>(P, A, LV, T, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt, X,
-                              X.w, Xa, sample, J, wg);
+            reverse_step<KHG, FEW>(P, A, LV, T, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt,
+                                   X, X.w, Xa, sample, J, wg);
             Xa = X;
         } while (--k >= kb);
     }
@@ -790,16 +803,24 @@ static void adj_set_carveout()
     cudaFuncSetAttribute(adj_backward_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     cudaFuncSetAttribute(adj_backward_traj_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     const void *seg[] = {
-#define LPM_SEG_FWD_ALL(M) (const void *)adj_forward_seg_kernel<M, false, false>,          \
-                           (const void *)adj_forward_seg_kernel<M, false, true>,            \
-                           (const void *)adj_forward_seg_kernel<M, true, false>,            \
-                           (const void *)adj_forward_seg_kernel<M, true, true>
+#define LPM_SEG_FWD_ALL(M) (const void *)adj_forward_seg_kernel<M, false, false, false>,   \
+                           (const void *)adj_forward_seg_kernel<M, false, true, false>,     \
+                           (const void *)adj_forward_seg_kernel<M, true, false, false>,     \
+                           (const void *)adj_forward_seg_kernel<M, true, true, false>,      \
+                           (const void *)adj_forward_seg_kernel<M, false, false, true>,     \
+                           (const void *)adj_forward_seg_kernel<M, false, true, true>,      \
+                           (const void *)adj_forward_seg_kernel<M, true, false, true>,      \
+                           (const void *)adj_forward_seg_kernel<M, true, true, true>
         LPM_SEG_FWD_ALL(SEG_STORE), LPM_SEG_FWD_ALL(SEG_CKPT), LPM_SEG_FWD_ALL(SEG_RECOMPUTE),
 #undef LPM_SEG_FWD_ALL
-        (const void *)adj_backward_seg_kernel<false, false>,
-        (const void *)adj_backward_seg_kernel<true, false>,
-        (const void *)adj_backward_seg_kernel<false, true>,
-        (const void *)adj_backward_seg_kernel<true, true>};
+        (const void *)adj_backward_seg_kernel<false, false, false>,
+        (const void *)adj_backward_seg_kernel<true, false, false>,
+        (const void *)adj_backward_seg_kernel<false, true, false>,
+        (const void *)adj_backward_seg_kernel<true, true, false>,
+        (const void *)adj_backward_seg_kernel<false, false, true>,
+        (const void *)adj_backward_seg_kernel<true, false, true>,
+        (const void *)adj_backward_seg_kernel<false, true, true>,
+        (const void *)adj_backward_seg_kernel<true, true, true>};
     for (const void *f : seg) cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     (void)cudaGetLastError();
 }
@@ -811,15 +832,20 @@ static void adj_prefer_l1()
 }
 
 cudaError_t launch_adj_forward_seg(cudaStream_t s, const StepParams &P, const AdjParams &A,
-                                   const AdjSeg &G, int n_groups, int mode)
+                                   const AdjSeg &G, int n_groups, int mode, int n_sm)
 {
     if (n_groups <= 0) return cudaSuccess;
     adj_prefer_l1();
-    constexpr int GROUPS = SEG_FWD_BLOCK / ADJ_BLOCK;
-    const int n = (n_groups + GROUPS - 1) / GROUPS;
-    const size_t sm = adj_smem_forward(P, A, GROUPS);
+    const bool few = n_groups <= SEG_FEW * n_sm;
+    const int groups = seg_fwd_block(few) / ADJ_BLOCK;
+    const int n = (n_groups + groups - 1) / groups;
+    const size_t sm = adj_smem_forward(P, A, groups);
     const bool multi = P.n_scen > 1, fields = P.khpair != nullptr;
-#define LPM_SEG_FWD(M, U, F) adj_forward_seg_kernel<M, U, F><<<n, SEG_FWD_BLOCK, sm, s>>>(P, A, G, n_groups)
+#define LPM_SEG_FWD(M, U, F)                                                              \
+    (few ? adj_forward_seg_kernel<M, U, F, true>                                          \
+               <<<n, seg_fwd_block(true), sm, s>>>(P, A, G, n_groups)                     \
+         : adj_forward_seg_kernel<M, U, F, false>                                         \
+               <<<n, seg_fwd_block(false), sm, s>>>(P, A, G, n_groups))
 #define LPM_SEG_FWD_MODE(M)                                                              \
     (multi ? (fields ? LPM_SEG_FWD(M, true, true) : LPM_SEG_FWD(M, true, false))          \
            : (fields ? LPM_SEG_FWD(M, false, true) : LPM_SEG_FWD(M, false, false)))
@@ -835,22 +861,27 @@ cudaError_t launch_adj_forward_seg(cudaStream_t s, const StepParams &P, const Ad
 }
 
 cudaError_t launch_adj_backward_seg(cudaStream_t s, const StepParams &P, const AdjParams &A,
-                                    const AdjSeg &G, int n_groups)
+                                    const AdjSeg &G, int n_groups, int n_sm)
 {
     if (n_groups <= 0) return cudaSuccess;
     adj_prefer_l1();
+    const bool few = n_groups <= SEG_FEW * n_sm;
     constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
     const int n = (n_groups + GROUPS - 1) / GROUPS;
     const size_t sm = adj_smem_backward(P, A, GROUPS);
     const bool multi = P.n_scen > 1;
+#define LPM_SEG_BWD(K, U)                                                                 \
+    (few ? adj_backward_seg_kernel<K, U, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups) \
+         : adj_backward_seg_kernel<K, U, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups))
     if (P.khpair && multi)
-        adj_backward_seg_kernel<true, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
+        LPM_SEG_BWD(true, true);
     else if (P.khpair)
-        adj_backward_seg_kernel<true, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
+        LPM_SEG_BWD(true, false);
     else if (multi)
-        adj_backward_seg_kernel<false, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
+        LPM_SEG_BWD(false, true);
     else
-        adj_backward_seg_kernel<false, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups);
+        LPM_SEG_BWD(false, false);
+#undef LPM_SEG_BWD
     return cudaGetLastError();
 }
 

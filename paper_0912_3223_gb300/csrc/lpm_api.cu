@@ -188,6 +188,7 @@ struct lpm_ctx {
         unsigned int *ord = nullptr, *live = nullptr, *keys = nullptr, *offsets = nullptr,
                      *meta = nullptr, *grave_n = nullptr;
         SortCounts counts{nullptr, nullptr};
+        bool counts_dirty = true;               // not zeroed yet, or left by a failed forward
         float4 *st[2] = {nullptr, nullptr};
         float4 *home = nullptr, *mu = nullptr, *grave = nullptr;
     } as;
@@ -2138,8 +2139,11 @@ lpm_status adj_sorted_buffers(lpm_ctx *c)
     LPM_CUDA(c, need(S.offsets, nb * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.counts.keys, nb * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.counts.tiles, ntiles * sizeof(unsigned int)));
-    LPM_CUDA(c, cudaMemsetAsync(S.counts.keys, 0, nb * sizeof(unsigned int), c->stream));
-    LPM_CUDA(c, cudaMemsetAsync(S.counts.tiles, 0, ntiles * sizeof(unsigned int), c->stream));
+    if (S.counts_dirty) {                        // (a sort leaves them zeroed)
+        LPM_CUDA(c, cudaMemsetAsync(S.counts.keys, 0, nb * sizeof(unsigned int), c->stream));
+        LPM_CUDA(c, cudaMemsetAsync(S.counts.tiles, 0, ntiles * sizeof(unsigned int), c->stream));
+        S.counts_dirty = false;
+    }
     LPM_CUDA(c, need(S.meta, 4 * sizeof(unsigned int)));
     LPM_CUDA(c, need(S.grave_n, sizeof(unsigned int)));
     for (float4 **p : {&S.st[0], &S.st[1], &S.home, &S.mu, &S.grave})
@@ -2188,7 +2192,7 @@ lpm_status adj_forward_sorted(lpm_ctx *c, const StepParams &P, const AdjParams &
             LPM_CUDA(c, cudaMemcpyAsync(S.live + s, S.meta, sizeof(unsigned int),
                                         cudaMemcpyDeviceToDevice, c->stream));
         LPM_CUDA(c, launch_adj_forward_seg(c->stream, P, A, G, (int)(G.width / ADJ_BLOCK),
-                                           c->adj_traj ? SEG_STORE : SEG_CKPT));
+                                           c->adj_traj ? SEG_STORE : SEG_CKPT, c->sm_count));
         c->n_launches++;
         if (s + 1 < n_seg) {
             SortSource in;
@@ -2247,7 +2251,7 @@ lpm_status adj_backward_ckpt(lpm_ctx *c, const StepParams &P, const AdjParams &A
     auto recompute = [&](int s) -> lpm_status {
         const AdjSeg G = adj_segment(c, s, 0);
         LPM_CUDA(c, launch_adj_forward_seg(c->adj_stream, P, A, G, (int)(G.width / ADJ_BLOCK),
-                                           SEG_RECOMPUTE));
+                                           SEG_RECOMPUTE, c->sm_count));
         LPM_CUDA(c, cudaEventRecord(recomputed[s & 1], c->adj_stream));
         c->n_launches++;
         return LPM_OK;
@@ -2265,7 +2269,8 @@ lpm_status adj_backward_ckpt(lpm_ctx *c, const StepParams &P, const AdjParams &A
         }
         const AdjSeg G = adj_segment(c, s, 0);
         LPM_CUDA(c, cudaStreamWaitEvent(c->stream, recomputed[s & 1], 0));
-        LPM_CUDA(c, launch_adj_backward_seg(c->stream, P, A, G, (int)(G.width / ADJ_BLOCK)));
+        LPM_CUDA(c, launch_adj_backward_seg(c->stream, P, A, G, (int)(G.width / ADJ_BLOCK),
+                                            c->sm_count));
         LPM_CUDA(c, cudaEventRecord(swept[s & 1], c->stream));
         c->n_launches++;
     }
@@ -2287,7 +2292,8 @@ lpm_status adj_backward_sorted(lpm_ctx *c, const StepParams &P, const AdjParams 
     }
     for (int s = (int)c->as.tiles_a.size() - 1; s >= 0; --s) {
         const AdjSeg G = adj_segment(c, s, 0);
-        LPM_CUDA(c, launch_adj_backward_seg(c->stream, P, A, G, (int)(G.width / ADJ_BLOCK)));
+        LPM_CUDA(c, launch_adj_backward_seg(c->stream, P, A, G, (int)(G.width / ADJ_BLOCK),
+                                            c->sm_count));
         c->n_launches++;
     }
     return LPM_OK;
@@ -2586,7 +2592,10 @@ lpm_status adj_forward(lpm_ctx *c, const double *rec, int R, double bandwidth, i
     LPM_CUDA(c, cudaMemsetAsync(c->d_rC, 0, (size_t)c->cfg.n_scenarios * R * sizeof(double), c->stream));
     if (c->adj_sorted) {
         st = adj_forward_sorted(c, P, A);
-        if (st != LPM_OK) return st;
+        if (st != LPM_OK) {
+            c->as.counts_dirty = true;
+            return st;
+        }
     } else {
         LPM_CUDA(c, launch_adj_forward(c->stream, P, A, (int)c->adj_tiles.size()));
         c->n_launches++;
