@@ -83,6 +83,8 @@ struct lpm_ctx {
     unsigned long long *d_dep = nullptr;    // [n_scen][2*cy*cx]
     unsigned long long *d_ctr = nullptr;    // [N_COUNTERS][n_scen]
     unsigned int *d_err = nullptr;
+    unsigned long long *h_words = nullptr;  // page-locked copies of it and of a scenario's
+                                            // counters (read-backs)
     unsigned int *d_queue = nullptr;        // tile-queue counters of a call's launches
     size_t queue_cap = 0;
     float *d_m0 = nullptr;
@@ -164,8 +166,8 @@ struct lpm_ctx {
     short *d_qi = nullptr;                  // emission-series index per release step
     float4 *d_ckpt = nullptr;
     size_t d_ckpt_cap = 0;
-    double *d_conv = nullptr;               // read-back of a grid converted on the device
-    size_t d_conv_cap = 0;
+    char *d_conv = nullptr;                 // read-back scratch: what the device converts
+    size_t d_conv_cap = 0;                  // (bytes)
     // trajectory storage (the default when it fits): rows of every tile from its first
     // release step on, and the state after each particle's last step (float4 elements)
     float4 *d_traj = nullptr, *d_fin = nullptr;
@@ -513,12 +515,16 @@ lpm_status upload_tables(lpm_ctx *c)
     return LPM_OK;
 }
 
+// Synchronises the context's streams and reports device-side errors: the last call of every
+// read-back, after the copies that it enqueued, so that one wait serves both.
 lpm_status check_device_error(lpm_ctx *c)
 {
-    unsigned int e = 0;
+    LPM_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_err, sizeof(unsigned int), cudaMemcpyDeviceToHost,
+                                c->stream));
     LPM_CUDA(c, cudaStreamSynchronize(c->stream));
     if (c->copy_stream) LPM_CUDA(c, cudaStreamSynchronize(c->copy_stream));
-    LPM_CUDA(c, cudaMemcpy(&e, c->d_err, sizeof e, cudaMemcpyDeviceToHost));
+    unsigned int e;
+    std::memcpy(&e, c->h_words, sizeof e);
     if (e & ERR_NAN) return fail(c, LPM_E_NUMERIC, "a particle position became non-finite");
     if (e & ERR_INDEX) return fail(c, LPM_E_CUDA, "a grid index fell outside its array");
     if (e & ERR_TIMEOUT) return fail(c, LPM_E_TIMEOUT, "a bounded device loop hit its limit");
@@ -753,12 +759,12 @@ lpm_status collect_events(lpm_ctx *c)
     return LPM_OK;
 }
 
-lpm_status read_counters(lpm_ctx *c, int scenario, unsigned long long v[N_COUNTERS])
+// Enqueues the copy of a scenario's counters to h_words[1 ...]; check_device_error waits for it.
+lpm_status read_counters(lpm_ctx *c, int scenario)
 {
-    const size_t ns = (size_t)c->cfg.n_scenarios;
-    for (int i = 0; i < N_COUNTERS; ++i)
-        LPM_CUDA(c, cudaMemcpy(v + i, c->d_ctr + i * ns + scenario, sizeof(unsigned long long),
-                               cudaMemcpyDeviceToHost));
+    constexpr size_t w = sizeof(unsigned long long);
+    LPM_CUDA(c, cudaMemcpy2DAsync(c->h_words + 1, w, c->d_ctr + scenario, w * (size_t)c->cfg.n_scenarios, w,
+                                  N_COUNTERS, cudaMemcpyDeviceToHost, c->stream));
     return LPM_OK;
 }
 
@@ -831,6 +837,7 @@ lpm_status lpm_create(const lpm_config *cfg, void *cuda_stream, lpm_ctx **out)
     CREATE_CUDA(cudaMalloc(&c->d_dep, ns * c->ndep() * sizeof(unsigned long long)));
     CREATE_CUDA(cudaMalloc(&c->d_ctr, ns * N_COUNTERS * sizeof(unsigned long long)));
     CREATE_CUDA(cudaMalloc(&c->d_err, sizeof(unsigned int)));
+    CREATE_CUDA(cudaMallocHost(&c->h_words, (1 + N_COUNTERS) * sizeof(unsigned long long)));
     c->queue_cap = 64;
     CREATE_CUDA(cudaMalloc(&c->d_queue, c->queue_cap * sizeof(unsigned int)));
     CREATE_CUDA(cudaMalloc(&c->d_scen, ns * sizeof(ScenDev)));
@@ -895,6 +902,7 @@ void lpm_destroy(lpm_ctx *c)
         for (void *p : aps)
             if (p) cudaFree(p);
     }
+    if (c->h_words) cudaFreeHost(c->h_words);
     if (c->copy_stream) cudaStreamSynchronize(c->copy_stream);
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : c->ev_pair)
@@ -1572,23 +1580,34 @@ lpm_status lpm_sync(lpm_ctx *c)
 }
 
 namespace {
-// Converts n 64-bit fixed-point sums to doubles (x f) on the device and copies them to the
-// host; the conversion and the copy run on the context stream, then it is synchronised.
-lpm_status read_fixed(lpm_ctx *c, const unsigned long long *src, size_t n, double f, double *out)
+// Room for `bytes` of converted read-back data.
+lpm_status conv_room(lpm_ctx *c, size_t bytes)
 {
-    if (n > c->d_conv_cap) {
-        LPM_CUDA(c, cudaStreamSynchronize(c->stream));
-        if (c->d_conv) cudaFree(c->d_conv);
-        c->d_conv = nullptr;
-        c->d_conv_cap = 0;
-        LPM_CUDA(c, cudaMalloc(&c->d_conv, n * sizeof(double)));
-        c->d_conv_cap = n;
-    }
-    LPM_CUDA(c, launch_fixed_to_double(c->stream, src, c->d_conv, (long long)n, f));
-    c->n_launches++;
-    LPM_CUDA(c, cudaMemcpyAsync(out, c->d_conv, n * sizeof(double), cudaMemcpyDeviceToHost,
-                                c->stream));
+    if (bytes <= c->d_conv_cap) return LPM_OK;
     LPM_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (c->d_conv) cudaFree(c->d_conv);
+    c->d_conv = nullptr;
+    c->d_conv_cap = 0;
+    LPM_CUDA(c, cudaMalloc(&c->d_conv, bytes));
+    c->d_conv_cap = bytes;
+    return LPM_OK;
+}
+
+// Enqueues the conversion of n 64-bit fixed-point sums to doubles (x f, / d) at element `at`
+// of the scratch, and the copy of the first n0 of them to out0 and the rest to out1 (either
+// may be nullptr).
+lpm_status read_fixed(lpm_ctx *c, const unsigned long long *src, size_t n, double f, double d,
+                      size_t at, double *out0, size_t n0, double *out1)
+{
+    double *conv = reinterpret_cast<double *>(c->d_conv) + at;
+    LPM_CUDA(c, launch_fixed_to_double(c->stream, src, conv, (long long)n, f, d));
+    c->n_launches++;
+    if (out0)
+        LPM_CUDA(c, cudaMemcpyAsync(out0, conv, n0 * sizeof(double), cudaMemcpyDeviceToHost,
+                                    c->stream));
+    if (out1)
+        LPM_CUDA(c, cudaMemcpyAsync(out1, conv + n0, (n - n0) * sizeof(double),
+                                    cudaMemcpyDeviceToHost, c->stream));
     return LPM_OK;
 }
 }  // namespace
@@ -1599,11 +1618,12 @@ lpm_status lpm_concentration(lpm_ctx *c, int scenario, double *out, size_t n_out
     if (scenario < 0 || scenario >= c->cfg.n_scenarios) return fail(c, LPM_E_INVALID, "bad scenario");
     if (!out || n_out != c->ncell())
         return fail(c, LPM_E_INVALID, "out must hold cz*cy*cx = %zu doubles", c->ncell());
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
     const lpm_config &g = c->cfg;
     const double f = std::ldexp(1.0, -c->scen[(size_t)scenario].shift) / (g.cdx * g.cdy * g.cdz);
-    return read_fixed(c, c->d_conc + (size_t)scenario * c->ncell(), c->ncell(), f, out);
+    lpm_status st = conv_room(c, n_out * sizeof(double));
+    if (st != LPM_OK) return st;
+    st = read_fixed(c, c->d_conc + (size_t)scenario * n_out, n_out, f, 1.0, 0, out, n_out, nullptr);
+    return st != LPM_OK ? st : check_device_error(c);
 }
 
 lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, size_t n_out)
@@ -1612,13 +1632,15 @@ lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, si
     if (scenario < 0 || scenario >= c->cfg.n_scenarios) return fail(c, LPM_E_INVALID, "bad scenario");
     const size_t plane = (size_t)c->cfg.cx * c->cfg.cy;
     if (n_out != plane) return fail(c, LPM_E_INVALID, "n_out must be cy*cx = %zu", plane);
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
     const double f = std::ldexp(1.0, -c->scen[(size_t)scenario].shift) / (c->cfg.cdx * c->cfg.cdy);
-    const unsigned long long *src = c->d_dep + (size_t)scenario * c->ndep();
-    if (dry && (st = read_fixed(c, src, plane, f, dry)) != LPM_OK) return st;
-    if (wet && (st = read_fixed(c, src + plane, plane, f, wet)) != LPM_OK) return st;
-    return LPM_OK;
+    lpm_status st = conv_room(c, 2 * plane * sizeof(double));
+    if (st != LPM_OK) return st;
+    if (dry || wet) {
+        st = read_fixed(c, c->d_dep + (size_t)scenario * c->ndep(), 2 * plane, f, 1.0, 0, dry, plane,
+                        wet);
+        if (st != LPM_OK) return st;
+    }
+    return check_device_error(c);
 }
 
 lpm_status lpm_budget(lpm_ctx *c, int scenario, double out[8])
@@ -1644,11 +1666,11 @@ lpm_status lpm_budget(lpm_ctx *c, int scenario, double out[8])
                               c->d_sorted[c->cur], c->d_pidx[c->cur], sorted ? c->d_live : nullptr,
                               sorted ? released_total(c, c->sorted_upto) : 0, (int)c->k));
     c->n_launches++;
+    st = read_counters(c, scenario);
+    if (st != LPM_OK) return st;
     st = check_device_error(c);
     if (st != LPM_OK) return st;
-    unsigned long long v[N_COUNTERS];
-    st = read_counters(c, scenario, v);
-    if (st != LPM_OK) return st;
+    const unsigned long long *v = c->h_words + 1;
     const double f = std::ldexp(1.0, -h.shift);
     // initial mass of the held particles released before the current step
     double released = 0.0;
@@ -1676,41 +1698,29 @@ lpm_status lpm_particles(lpm_ctx *c, int64_t first, int64_t count, float *xyz, u
     if (first < 0 || count < 0 || first + count > c->n_slots_used)
         return fail(c, LPM_E_INVALID, "slots [%lld, %lld) outside the %lld released",
                     (long long)first, (long long)(first + count), c->n_slots_used);
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
-    if (count == 0) return LPM_OK;
-    std::vector<float4> h((size_t)count);
-    if (c->d_sorted[0]) {
-        // slot order: gather from the home slots, the sorted set and the dead array into
-        // the spare sorted buffer (free until the next sort)
-        float4 *tmp = c->d_sorted[1 - c->cur];
-        {
-            const lpm_status sm = ensure_slot_map(c);
-            if (sm != LPM_OK) return sm;
-        }
-        LPM_CUDA(c, launch_gather(c->stream, c->d_state, c->d_sorted[c->cur], c->d_slot_of,
-                                  c->d_grave, first, count, tmp));
-        LPM_CUDA(c, cudaMemcpyAsync(h.data(), tmp, h.size() * sizeof(float4),
-                                    cudaMemcpyDeviceToHost, c->stream));
-        LPM_CUDA(c, cudaStreamSynchronize(c->stream));
+    lpm_status st = LPM_OK;
+    const bool sorted = c->d_sorted[0] != nullptr;
+    if (sorted && count > 0 && (st = ensure_slot_map(c)) != LPM_OK) return st;
+    // slot order, from the home slots, the sorted set and the dead array, as the caller's two
+    // arrays, a bounded piece at a time
+    const int64_t most = (int64_t)1 << 22;
+    if ((st = conv_room(c, (size_t)std::min(count, most) * 4 * sizeof(float))) != LPM_OK) return st;
+    for (int64_t at = 0; at < count && (xyz || tag); at += most) {
+        const int64_t n = std::min(most, count - at);
+        float *d_xyz = reinterpret_cast<float *>(c->d_conv);
+        unsigned int *d_tag = reinterpret_cast<unsigned int *>(d_xyz + 3 * n);
+        LPM_CUDA(c, launch_gather_xyz(c->stream, c->d_state, sorted ? c->d_sorted[c->cur] : nullptr,
+                                      sorted ? c->d_slot_of : nullptr, c->d_grave, first + at, n,
+                                      xyz ? d_xyz : nullptr, tag ? d_tag : nullptr));
         c->n_launches++;
-    } else {
-        LPM_CUDA(c, cudaMemcpy(h.data(), c->d_state + first, h.size() * sizeof(float4),
-                               cudaMemcpyDeviceToHost));
+        if (xyz)
+            LPM_CUDA(c, cudaMemcpyAsync(xyz + 3 * at, d_xyz, (size_t)n * 3 * sizeof(float),
+                                        cudaMemcpyDeviceToHost, c->stream));
+        if (tag)
+            LPM_CUDA(c, cudaMemcpyAsync(tag + at, d_tag, (size_t)n * sizeof(uint32_t),
+                                        cudaMemcpyDeviceToHost, c->stream));
     }
-    for (size_t i = 0; i < h.size(); ++i) {
-        if (xyz) {
-            xyz[3 * i] = h[i].x;
-            xyz[3 * i + 1] = h[i].y;
-            xyz[3 * i + 2] = h[i].z;
-        }
-        if (tag) {
-            uint32_t t;
-            std::memcpy(&t, &h[i].w, sizeof t);
-            tag[i] = t;
-        }
-    }
-    return LPM_OK;
+    return check_device_error(c);
 }
 
 lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_conc, uint64_t *dep,
@@ -1720,19 +1730,17 @@ lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_co
     if (scenario < 0 || scenario >= c->cfg.n_scenarios) return fail(c, LPM_E_INVALID, "bad scenario");
     if (conc && n_conc != c->ncell()) return fail(c, LPM_E_INVALID, "n_conc must be %zu", c->ncell());
     if (dep && n_dep != c->ndep()) return fail(c, LPM_E_INVALID, "n_dep must be %zu", c->ndep());
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
+    lpm_status st = LPM_OK;
     if (conc)
-        LPM_CUDA(c, cudaMemcpy(conc, c->d_conc + (size_t)scenario * c->ncell(),
-                               n_conc * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+        LPM_CUDA(c, cudaMemcpyAsync(conc, c->d_conc + (size_t)scenario * c->ncell(),
+                                    n_conc * sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
     if (dep)
-        LPM_CUDA(c, cudaMemcpy(dep, c->d_dep + (size_t)scenario * c->ndep(),
-                               n_dep * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+        LPM_CUDA(c, cudaMemcpyAsync(dep, c->d_dep + (size_t)scenario * c->ndep(),
+                                    n_dep * sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
+    if (counters && (st = read_counters(c, scenario)) != LPM_OK) return st;
+    if ((st = check_device_error(c)) != LPM_OK) return st;
     if (counters) {
-        unsigned long long v[N_COUNTERS];
-        st = read_counters(c, scenario, v);
-        if (st != LPM_OK) return st;
-        for (int i = 0; i < 16; ++i) counters[i] = (int64_t)v[i];
+        for (int i = 0; i < 16; ++i) counters[i] = (int64_t)c->h_words[1 + i];
         counters[C_N_BINS] = c->n_bins;
     }
     if (shift) *shift = c->scen[(size_t)scenario].shift;
@@ -1877,8 +1885,6 @@ lpm_status lpm_species(lpm_ctx *c, int scenario, int species, double *conc, doub
     if (scenario < 0 || scenario >= c->cfg.n_scenarios) return fail(c, LPM_E_INVALID, "bad scenario");
     if (species < 0 || species >= c->n_species)
         return fail(c, LPM_E_INVALID, "species %d outside the chain of %d", species, c->n_species);
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
     const size_t ns = (size_t)c->cfg.n_scenarios, plane = (size_t)c->cfg.cx * c->cfg.cy;
     const unsigned long long *dc, *dd;
     if (species == 0) {
@@ -1888,22 +1894,21 @@ lpm_status lpm_species(lpm_ctx *c, int scenario, int species, double *conc, doub
         dc = c->d_sp_conc + ((size_t)(species - 1) * ns + scenario) * c->ncell();
         dd = c->d_sp_dep + ((size_t)(species - 1) * ns + scenario) * c->ndep();
     }
-    std::vector<unsigned long long> hc(c->ncell()), hd(c->ndep());
-    LPM_CUDA(c, cudaMemcpy(hc.data(), dc, hc.size() * 8, cudaMemcpyDeviceToHost));
-    LPM_CUDA(c, cudaMemcpy(hd.data(), dd, hd.size() * 8, cudaMemcpyDeviceToHost));
-    if (conc_fixed) std::memcpy(conc_fixed, hc.data(), hc.size() * 8);
-    if (dep_fixed) std::memcpy(dep_fixed, hd.data(), hd.size() * 8);
     const lpm_config &g = c->cfg;
     const double unit = std::ldexp(1.0, -c->scen[(size_t)scenario].shift);
-    if (conc)
-        for (size_t i = 0; i < hc.size(); ++i) conc[i] = (double)hc[i] * unit / (g.cdx * g.cdy * g.cdz);
-    for (int kind = 0; kind < 2; ++kind) {
-        double *out = kind ? wet : dry;
-        if (!out) continue;
-        for (size_t i = 0; i < plane; ++i)
-            out[i] = (double)hd[kind * plane + i] * unit / (g.cdx * g.cdy);
-    }
-    return LPM_OK;
+    const double vol = g.cdx * g.cdy * g.cdz, area = g.cdx * g.cdy;
+    lpm_status st = conv_room(c, (c->ncell() + c->ndep()) * sizeof(double));
+    if (st != LPM_OK) return st;
+    if (conc && (st = read_fixed(c, dc, c->ncell(), unit, vol, 0, conc, c->ncell(), nullptr)) != LPM_OK)
+        return st;
+    if ((dry || wet) &&
+        (st = read_fixed(c, dd, 2 * plane, unit, area, c->ncell(), dry, plane, wet)) != LPM_OK)
+        return st;
+    if (conc_fixed)
+        LPM_CUDA(c, cudaMemcpyAsync(conc_fixed, dc, c->ncell() * 8, cudaMemcpyDeviceToHost, c->stream));
+    if (dep_fixed)
+        LPM_CUDA(c, cudaMemcpyAsync(dep_fixed, dd, c->ndep() * 8, cudaMemcpyDeviceToHost, c->stream));
+    return check_device_error(c);
 }
 
 lpm_status lpm_set_kz_model(lpm_ctx *c, int model, double kz_min)
@@ -1997,20 +2002,20 @@ lpm_status lpm_dosage(lpm_ctx *c, int scenario, double *out, size_t n_out, uint6
     if (!c->d_dose) return fail(c, LPM_E_STATE, "dosage was never enabled (lpm_set_dosage)");
     if ((out || fixed) && n_out != c->ncell())
         return fail(c, LPM_E_INVALID, "n_out must be cz*cy*cx = %zu", c->ncell());
-    lpm_status st = check_device_error(c);
-    if (st != LPM_OK) return st;
-    if (n_samples) *n_samples = c->n_dose;
-    if (!out && !fixed) return LPM_OK;
-    std::vector<unsigned long long> h(c->ncell());
-    LPM_CUDA(c, cudaMemcpy(h.data(), c->d_dose + (size_t)scenario * c->ncell(),
-                           h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
-    if (fixed) std::memcpy(fixed, h.data(), h.size() * sizeof(uint64_t));
+    lpm_status st = LPM_OK;
+    const unsigned long long *src = c->d_dose + (size_t)scenario * c->ncell();
+    if (fixed)
+        LPM_CUDA(c, cudaMemcpyAsync(fixed, src, n_out * sizeof(uint64_t), cudaMemcpyDeviceToHost,
+                                    c->stream));
     if (out) {
         const lpm_config &g = c->cfg;
         const double f = std::ldexp(1.0, c->dose_bits - c->scen[(size_t)scenario].shift) *
                          ((double)c->dose_every * g.dt) / (g.cdx * g.cdy * g.cdz);
-        for (size_t i = 0; i < h.size(); ++i) out[i] = (double)h[i] * f;
+        if ((st = conv_room(c, n_out * sizeof(double))) != LPM_OK) return st;
+        if ((st = read_fixed(c, src, n_out, f, 1.0, 0, out, n_out, nullptr)) != LPM_OK) return st;
     }
+    if ((st = check_device_error(c)) != LPM_OK) return st;
+    if (n_samples) *n_samples = c->n_dose;
     return LPM_OK;
 }
 

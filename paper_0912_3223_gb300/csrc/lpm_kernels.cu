@@ -219,24 +219,30 @@ int advance_occupancy(int block, int occ, bool mixed, int variant, size_t smem)
     return 0;
 }
 
-// Read-back of a 64-bit fixed-point grid as physical values: out[i] = in[i] * f (the
-// conversion rounds to nearest, as on the host).
+// Read-back of a 64-bit fixed-point grid as physical values, in the host's arithmetic (the
+// conversion rounds to nearest): out[i] = in[i] * f, or with DIV in[i] * f / d.
+template <bool DIV>
 __global__ void fixed_to_double_kernel(const unsigned long long *__restrict__ in,
-                                       double *__restrict__ out, long long n, double f)
+                                       double *__restrict__ out, long long n, double f, double d)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        out[i] = __ull2double_rn(in[i]) * f;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const double v = __ull2double_rn(in[i]) * f;
+        out[i] = DIV ? __ddiv_rn(v, d) : v;
+    }
 }
 
 cudaError_t launch_fixed_to_double(cudaStream_t s, const unsigned long long *in, double *out,
-                                   long long n, double f)
+                                   long long n, double f, double d)
 {
     if (n <= 0) return cudaSuccess;
     const int block = 256;
     long long blocks = (n + block - 1) / block;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    fixed_to_double_kernel<<<(unsigned)blocks, block, 0, s>>>(in, out, n, f);
+    if (d == 1.0)
+        fixed_to_double_kernel<false><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d);
+    else
+        fixed_to_double_kernel<true><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d);
     return cudaGetLastError();
 }
 

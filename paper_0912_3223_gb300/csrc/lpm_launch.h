@@ -204,6 +204,9 @@ cudaError_t launch_sort(cudaStream_t s, const StepParams &P, const SortSource &i
 cudaError_t launch_gather(cudaStream_t s, const float4 *home, const float4 *sorted,
                           const unsigned int *slot_of, const float4 *grave, long long first,
                           long long count, float4 *out);
+cudaError_t launch_gather_xyz(cudaStream_t s, const float4 *home, const float4 *sorted,
+                              const unsigned int *slot_of, const float4 *grave, long long first,
+                              long long count, float *xyz, unsigned int *tag);
 cudaError_t launch_gather_w(cudaStream_t s, const float *home, const float *sorted,
                             const unsigned int *slot_of, long long first, long long count,
                             float *out);
@@ -219,7 +222,7 @@ cudaError_t launch_budget(cudaStream_t s, const StepParams &P, const float4 *hom
                           int k_now);
 
 cudaError_t launch_fixed_to_double(cudaStream_t s, const unsigned long long *in, double *out,
-                                   long long n, double f);
+                                   long long n, double f, double d = 1.0);
 void set_global_error(const char *msg);
 
 struct AdjParams;

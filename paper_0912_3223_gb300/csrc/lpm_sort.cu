@@ -279,6 +279,24 @@ __global__ void gather_kernel(const float4 *__restrict__ home, const float4 *__r
         out[i] = locate(home, sorted, slot_of, grave, first + i);
 }
 
+// The same as separate positions [count][3] and tags [count] (either may be nullptr).
+__global__ void gather_xyz_kernel(const float4 *__restrict__ home, const float4 *__restrict__ sorted,
+                                  const unsigned int *__restrict__ slot_of,
+                                  const float4 *__restrict__ grave, long long first, long long count,
+                                  float *__restrict__ xyz, unsigned int *__restrict__ tag)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
+        const float4 s = locate(home, sorted, slot_of, grave, first + i);
+        if (xyz) {
+            xyz[3 * i] = s.x;
+            xyz[3 * i + 1] = s.y;
+            xyz[3 * i + 2] = s.z;
+        }
+        if (tag) tag[i] = __float_as_uint(s.w);
+    }
+}
+
 // Langevin w' of particles [first, first + count) in home order (0 for dead ones).
 __global__ void gather_w_kernel(const float *__restrict__ home, const float *__restrict__ sorted,
                                 const unsigned int *__restrict__ slot_of, long long first,
@@ -356,6 +374,16 @@ cudaError_t launch_gather(cudaStream_t s, const float4 *home, const float4 *sort
     if (count <= 0) return cudaSuccess;
     gather_kernel<<<grid_for(count, 256), 256, 0, s>>>(home, sorted, slot_of, grave, first, count,
                                                        out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gather_xyz(cudaStream_t s, const float4 *home, const float4 *sorted,
+                              const unsigned int *slot_of, const float4 *grave, long long first,
+                              long long count, float *xyz, unsigned int *tag)
+{
+    if (count <= 0) return cudaSuccess;
+    gather_xyz_kernel<<<grid_for(count, 256), 256, 0, s>>>(home, sorted, slot_of, grave, first,
+                                                           count, xyz, tag);
     return cudaGetLastError();
 }
 
