@@ -22,7 +22,7 @@
 namespace lpm {
 
 // Weather and its spatial gradient: val = (u, v, w, K_z, K_h), g[q][d] = d val[q] / d x_d.
-// KHG: K_h is a gridded field (else uniform, gradient 0, and none of its code is compiled).
+// KHG: K_h may be a gridded field (else uniform, gradient 0, none of its code compiled).
 template <bool KHG, class LEV>
 __device__ __forceinline__ void sample_met_grad(const StepParams &P, const LEV &L,
                                                 const StepTime &T, float sig_h_uniform, float x,
@@ -184,8 +184,8 @@ adj_forward_kernel(const StepParams P, const AdjParams A)
     float4 *s_rec = s_dyn;                        // [R]
     double *s_C = reinterpret_cast<double *>(s_rec + A.R);    // [R]
     unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_C + A.R);   // [n_lut]
-    __shared__ float2 s_zi[MAX_LEVELS];            // warps span many levels here
-    const LevelsS LV = load_levels_smem(P, s_zi, s_lut);
+    __shared__ float4 s_ent[MAX_LEVELS];           // warps span many levels here
+    const auto LV = load_levels<Levels<true, false>>(P, s_lut, s_ent);
     for (int r = threadIdx.x; r < A.R; r += ADJ_BLOCK) {
         s_rec[r] = A.rec[r];
         s_C[r] = 0.0;
@@ -377,8 +377,8 @@ adj_backward_kernel(const StepParams P, const AdjParams A)
     double *s_gq = s_g + 6;                       // [nq]
     float *s_w = reinterpret_cast<float *>(s_gq + A.nq);      // [R]
     unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + A.R);   // [n_lut]
-    __shared__ float2 s_zi[MAX_LEVELS];            // warps span many levels here
-    const LevelsS LV = load_levels_smem(P, s_zi, s_lut);
+    __shared__ float4 s_ent[MAX_LEVELS];           // warps span many levels here
+    const auto LV = load_levels<Levels<true, false>>(P, s_lut, s_ent);
     const Tile tile = A.tiles[blockIdx.x];
     load_receptors(A, tile, s_rec, s_w, s_g, s_gq);
     const ScenDev sc = P.scen[tile.scen];
@@ -456,8 +456,8 @@ adj_backward_traj_kernel(const StepParams P, const AdjParams A)
     double *s_gq = s_g + 6;                       // [nq]
     float *s_w = reinterpret_cast<float *>(s_gq + A.nq);      // [R]
     unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + A.R);   // [n_lut]
-    __shared__ float2 s_zi[MAX_LEVELS];            // warps span many levels here
-    const LevelsS LV = load_levels_smem(P, s_zi, s_lut);
+    __shared__ float4 s_ent[MAX_LEVELS];           // warps span many levels here
+    const auto LV = load_levels<Levels<true, false>>(P, s_lut, s_ent);
     const Tile tile = A.tiles[blockIdx.x];
     load_receptors(A, tile, s_rec, s_w, s_g, s_gq);
     const ScenDev sc = P.scen[tile.scen];
@@ -595,7 +595,7 @@ __device__ __forceinline__ bool seg_block_empty(const AdjSeg &G, int group0, int
 }
 
 // Receptor forward of a segment (MODE: SegMode). MULTI: entries of several scenarios (else
-// all of scenario 0); FIELDS: a gridded K_h. Instructions bound it as they do the advance
+// all of scenario 0); FIELDS: a gridded K_h, or no level table. Instructions bound it as they do the advance
 // kernel: the step times come from a table, the deposition words from one block for two
 // steps, the samples by a countdown.
 template <int MODE, bool MULTI, bool FIELDS, bool FEW>
@@ -613,7 +613,9 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
     double *s_C = reinterpret_cast<double *>(s_rec + A.R);    // [GROUPS][R]
     unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_C + GROUPS * A.R);   // [n_lut]
     __shared__ float4 s_ta[CK];                   // the segment's step times
-    const Levels LV = load_levels(P, s_lut);
+    using Lev = Levels<MULTI, !FIELDS>;           // (the rule is at Levels)
+    __shared__ float4 s_ent[Lev::SMEM ? MAX_LEVELS : 1];
+    const Lev LV = load_levels<Lev>(P, s_lut, s_ent);
     for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += BLOCK)
         s_ta[i] = step_time_parts(P, G.k_lo + i);
     if (SAMPLE) {
@@ -655,7 +657,7 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
             const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
             const float xb = x, yb = y, zb = z;
             float fs = 1.0f;
-            st = particle_step<false, false, Levels, false, FIELDS, FEW>(
+            st = particle_step<false, false, Lev, false, FIELDS, FEW>(
                 P, LV, T, sc, nullptr, gid, sp, sig_h_uniform, T.du, T.dv, x, y, z,
                 ROWS ? &fs : nullptr, nullptr, nullptr, &dc);
             if (ROWS) {
@@ -689,7 +691,7 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
     }
 }
 
-// Reverse sweep of a segment (KHG: gridded K_h). Bound by the latency of its gathers at 19
+// Reverse sweep of a segment (KHG: gridded K_h, or no level table). Bound by the latency of its gathers at 19
 // warps an SM (96 registers hold the record differences; issue 56 % busy); a uniform K_h's
 // scale is taken out of the loop, its vanishing derivative dropped (571 -> 480 instructions
 // a step with that, the tabled times and the shared round keys).
@@ -711,7 +713,9 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, i
     s_g += 6 * gi;
     s_gq += A.nq * gi;
     s_w += A.R * gi;
-    const Levels LV = load_levels(P, s_lut);
+    using Lev = Levels<MULTI, !KHG>;              // (the rule is at Levels)
+    __shared__ float4 s_ent[Lev::SMEM ? MAX_LEVELS : 1];
+    const Lev LV = load_levels<Lev>(P, s_lut, s_ent);
     // the segment's step times, once per block
     __shared__ float4 s_ta[CK];
     for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_BWD_BLOCK)
@@ -840,7 +844,7 @@ cudaError_t launch_adj_forward_seg(cudaStream_t s, const StepParams &P, const Ad
     const int groups = seg_fwd_block(few) / ADJ_BLOCK;
     const int n = (n_groups + groups - 1) / groups;
     const size_t sm = adj_smem_forward(P, A, groups);
-    const bool multi = P.n_scen > 1, fields = P.khpair != nullptr;
+    const bool multi = P.n_scen > 1, fields = P.khpair || P.lut_last < 0;
 #define LPM_SEG_FWD(M, U, F)                                                              \
     (few ? adj_forward_seg_kernel<M, U, F, true>                                          \
                <<<n, seg_fwd_block(true), sm, s>>>(P, A, G, n_groups)                     \
@@ -869,13 +873,13 @@ cudaError_t launch_adj_backward_seg(cudaStream_t s, const StepParams &P, const A
     constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
     const int n = (n_groups + GROUPS - 1) / GROUPS;
     const size_t sm = adj_smem_backward(P, A, GROUPS);
-    const bool multi = P.n_scen > 1;
+    const bool multi = P.n_scen > 1, fields = P.khpair || P.lut_last < 0;
 #define LPM_SEG_BWD(K, U)                                                                 \
     (few ? adj_backward_seg_kernel<K, U, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups) \
          : adj_backward_seg_kernel<K, U, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups))
-    if (P.khpair && multi)
+    if (fields && multi)
         LPM_SEG_BWD(true, true);
-    else if (P.khpair)
+    else if (fields)
         LPM_SEG_BWD(true, false);
     else if (multi)
         LPM_SEG_BWD(false, true);

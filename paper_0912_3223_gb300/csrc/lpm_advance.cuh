@@ -516,18 +516,19 @@ struct MinBlocks {
 // samples (every P.dose_every steps) inside the time loop, K_z from Eq. 3 (P.blpair), the
 // daughters of a decay chain (P.n_species > 1), the Langevin variant and the scenarios'
 // perturbation modes (P.n_modes > 0); MODES carries the modes alone, FIELDS a gridded K_h and
-// the drift correction. The plain instantiations carry none of that code.
+// the drift correction. TABLE: the levels have a lookup table. The plain instantiations carry
+// none of that code.
 //
 // Bound by issued instructions (32 warps an SM keep the schedulers 75 % busy, DRAM idle), so
 // the step is kept short of branches and constant loads. A lane's time loop starts at its own
 // release step and ends with the particle: no status is tested inside it, and the lanes of a
 // tile of late releases all work from the loop's first turn. (The dosage samples gather a
 // warp's lanes at the same step, so with them the loop runs over common steps.)
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS, bool TABLE>
 __global__ void __launch_bounds__(BLOCK, (MinBlocks<BLOCK, OCC>::value))
 advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, int k1, int do_bin)
 {
-    extern __shared__ float4 s_adv_dyn[];            // the level table, sized by the launch
+    extern __shared__ float4 s_adv_dyn[];            // the level tables, sized by the launch
     __shared__ unsigned long long s_acc[BLOCK];
     __shared__ unsigned long long s_steps;
     __shared__ unsigned int s_tile;
@@ -539,7 +540,10 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
     const unsigned int units_a = (unsigned int)((live + 31) >> 5);
     const unsigned int n_units = units_a + ((unsigned int)R.n_b << R.unit_shift);
     if (n_units < R.unit_min || n_units > R.unit_max) return;
-    const Levels LV = load_levels(P, reinterpret_cast<unsigned char *>(s_adv_dyn));
+    // (the rule for the first is at Levels)
+    using Lev = Levels<OCC != 2 || EXT || MODES, TABLE>;
+    const Lev LV = load_levels<Lev>(P, reinterpret_cast<unsigned char *>(s_adv_dyn + P.nz),
+                                    s_adv_dyn);
     unsigned long long *s_warp = s_acc + (threadIdx.x & ~31);
     const int lane = threadIdx.x & 31;
     const unsigned int warp = threadIdx.x >> 5;
@@ -636,7 +640,7 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                     du = P.bias_u + fmaf(T.f, o1.x - o0.x, o0.x);
                     dv = P.bias_v + fmaf(T.f, o1.y - o0.y, o0.y);
                 }
-                return particle_step<true, EXT, Levels, MODES, FIELDS, OCC != 2>(
+                return particle_step<true, EXT, Lev, MODES, FIELDS, OCC != 2>(
                     P, LV, T, sc, &sc, gid, sp, sig_h_uniform, du, dv, x, y, z, nullptr,
                     lang ? &wv : nullptr, msc, &dc);
             };
@@ -770,33 +774,34 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
     }
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS, bool TABLE>
 void adv_prefer_l1()
 {
     // the kernel needs a few KB of shared memory per block: ask for a small carve-out so the
     // rest of the SM's unified L1 serves the weather gathers (measured +0.7 to +1.7 %)
-    cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>,
+    cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS, TABLE>,
                          cudaFuncAttributePreferredSharedMemoryCarveout, 10);
     (void)cudaGetLastError();
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS, bool TABLE>
 cudaError_t launch_adv(const AdvanceLaunch &L)
 {
     static std::once_flag once;          // per instantiation; contexts may use several threads
-    std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>);
-    const size_t smem = adv_dyn_smem(L.params->n_lut);
-    advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS><<<L.grid, BLOCK, smem, L.stream>>>(
+    std::call_once(once, adv_prefer_l1<BLOCK, OCC, MIXED, EXT, MODES, FIELDS, TABLE>);
+    const size_t smem = adv_dyn_smem(L.params->nz, L.params->n_lut);
+    advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS, TABLE><<<L.grid, BLOCK, smem,
+                                                                  L.stream>>>(
         *L.params, L.ranges, L.queue, L.k0, L.k1, L.do_bin);
     return cudaGetLastError();
 }
 
-template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS>
+template <int BLOCK, int OCC, bool MIXED, bool EXT, bool MODES, bool FIELDS, bool TABLE>
 int occ_adv(size_t smem)
 {
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS>, BLOCK, smem);
+        &n, advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS, TABLE>, BLOCK, smem);
     return n;
 }
 
@@ -804,9 +809,10 @@ int occ_adv(size_t smem)
 // one block size
 #define LPM_ADV_CASE(FN, BLOCK, OCC, MIX, VAR, ...)                                    \
     case OCC * 100 + MIX * 10 + VAR:                                                   \
-        return FN<BLOCK, OCC, (MIX != 0), (VAR == ADV_EXT),                            \
-                  (VAR == ADV_EXT || VAR == ADV_MODES || VAR == ADV_MODES_FIELDS),     \
-                  (VAR == ADV_EXT || VAR == ADV_FIELDS || VAR == ADV_MODES_FIELDS)>(__VA_ARGS__);
+        return FN<BLOCK, OCC, (MIX != 0), adv_is_ext(VAR),                          \
+                  (adv_is_ext(VAR) || VAR == ADV_MODES || VAR == ADV_MODES_FIELDS),        \
+                  (adv_is_ext(VAR) || VAR == ADV_FIELDS || VAR == ADV_MODES_FIELDS),       \
+                  (VAR == ADV_PLAIN || VAR == ADV_EXT || VAR == ADV_MODES)>(__VA_ARGS__);
 #define LPM_ADV_CASES2(FN, BLOCK, VAR, ...)                                            \
     LPM_ADV_CASE(FN, BLOCK, 0, 0, VAR, __VA_ARGS__)                                    \
     LPM_ADV_CASE(FN, BLOCK, 0, 1, VAR, __VA_ARGS__)                                    \
@@ -819,7 +825,8 @@ int occ_adv(size_t smem)
     LPM_ADV_CASES2(FN, BLOCK, 1, __VA_ARGS__)                                          \
     LPM_ADV_CASES2(FN, BLOCK, 2, __VA_ARGS__)                                          \
     LPM_ADV_CASES2(FN, BLOCK, 3, __VA_ARGS__)                                          \
-    LPM_ADV_CASES2(FN, BLOCK, 4, __VA_ARGS__)
+    LPM_ADV_CASES2(FN, BLOCK, 4, __VA_ARGS__)                                          \
+    LPM_ADV_CASES2(FN, BLOCK, 5, __VA_ARGS__)
 
 #define LPM_ADVANCE_TU(BLOCK)                                                          \
     cudaError_t launch_advance_b##BLOCK(const AdvanceLaunch &L)                         \

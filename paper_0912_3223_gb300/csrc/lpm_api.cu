@@ -1261,13 +1261,13 @@ int launch_shapes(const lpm_ctx *c, const StepParams &P, long long units, Shape 
         if (!large)
             h[n++] = {units <= 4LL * c->sm_count ? 512 : 256, 0, 0, 0u, small ? ANY : few};
         if (!small) {
-            const bool wide = variant != ADV_EXT && (mixed || units > 32768);
+            const bool wide = !adv_is_ext(variant) && (mixed || units > 32768);
             h[n++] = {wide ? 512 : 256, wide ? 2 : 1, 0, large ? 0u : few + 1u, ANY};
         }
     }
     for (int i = 0; i < n; ++i)
         h[i].blocks = c->sm_count * std::max(1, advance_occupancy(h[i].block, h[i].occ, mixed,
-                                                                  variant, adv_dyn_smem(P.n_lut)));
+                                                                  variant, adv_dyn_smem(P.nz, P.n_lut)));
     return n;
 }
 

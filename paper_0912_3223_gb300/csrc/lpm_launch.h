@@ -55,13 +55,24 @@ constexpr int STEP_TAB = 128;
 
 // Options of an advance launch, by the instantiation that carries their code: none; the
 // extended step (dosage, Eq. 3 K_z, a decay chain, the Langevin variant, with anything else);
-// perturbation modes; a gridded K_h or the drift correction; both of these.
-enum { ADV_PLAIN = 0, ADV_EXT = 1, ADV_MODES = 2, ADV_FIELDS = 3, ADV_MODES_FIELDS = 4 };
+// perturbation modes; a gridded K_h, the drift correction or levels without a lookup table;
+// modes and any of these; the extended step on levels without a lookup table.
+enum {
+    ADV_PLAIN = 0,
+    ADV_EXT = 1,
+    ADV_MODES = 2,
+    ADV_FIELDS = 3,
+    ADV_MODES_FIELDS = 4,
+    ADV_EXT_SEARCH = 5
+};
+
+constexpr bool adv_is_ext(int v) { return v == ADV_EXT || v == ADV_EXT_SEARCH; }
 
 inline int adv_variant(const StepParams &P)
 {
-    if (P.dose_every > 0 || P.blpair || P.n_species > 1 || P.langevin) return ADV_EXT;
-    const bool fields = P.khpair || P.drift;
+    if (P.dose_every > 0 || P.blpair || P.n_species > 1 || P.langevin)
+        return P.lut_last < 0 ? ADV_EXT_SEARCH : ADV_EXT;
+    const bool fields = P.khpair || P.drift || P.lut_last < 0;
     if (P.n_modes > 0) return fields ? ADV_MODES_FIELDS : ADV_MODES;
     return fields ? ADV_FIELDS : ADV_PLAIN;
 }
@@ -181,10 +192,10 @@ cudaError_t launch_release(cudaStream_t s, float4 *state, long long first_slot, 
                            long long part_first, long long n_total, int rel_first, int rel_len,
                            float sx, float sy, float sz);
 cudaError_t launch_release_all(cudaStream_t s, const StepParams &P, float4 *state, long long n_slots);
-// Bytes of dynamic shared memory of an advance launch: its copy of the vertical level table.
-inline size_t adv_dyn_smem(int n_lut)
+// Bytes of dynamic shared memory of an advance launch: its level tables.
+inline size_t adv_dyn_smem(int nz, int n_lut)
 {
-    return ((size_t)(n_lut > 0 ? n_lut : 0) + 15) & ~(size_t)15;
+    return (size_t)nz * sizeof(float4) + (((size_t)(n_lut > 0 ? n_lut : 0) + 15) & ~(size_t)15);
 }
 
 cudaError_t launch_advance(const AdvanceLaunch &L);

@@ -47,7 +47,7 @@ __global__ void sort_keys_kernel(const StepParams P, const SortSource S,
                                  unsigned int dead_key)
 {
     __shared__ unsigned char s_lut[MAX_LUT];
-    const Levels LV = load_levels(P, s_lut);
+    const auto LV = load_levels<Levels<false, false>>(P, s_lut);
     __syncthreads();
     const unsigned int live_old = S.has_a ? meta[0] : 0u;
     const long long n = (long long)live_old + ((long long)S.n_b << S.t_shift);
