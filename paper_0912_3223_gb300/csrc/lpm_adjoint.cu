@@ -691,10 +691,12 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
     }
 }
 
-// Reverse sweep of a segment (KHG: gridded K_h, or no level table). Bound by the latency of its gathers at 19
-// warps an SM (96 registers hold the record differences; issue 56 % busy); a uniform K_h's
-// scale is taken out of the loop, its vanishing derivative dropped (571 -> 480 instructions
-// a step with that, the tabled times and the shared round keys).
+// Reverse sweep of a segment (KHG: gridded K_h, or no level table). Bound by the latency of
+// its gathers at 19 warps an SM (96 registers hold the record differences; issue 56 % busy);
+// a uniform K_h's scale is taken out of the loop, its vanishing derivative dropped (571 -> 480
+// instructions a step with that, the tabled times and the shared round keys). The draws come
+// before the gathers with several scenarios too, whose gathers miss the L1 more often
+// (inversion of 16 x 1e5: 35.0 -> 34.2 ms); with one they measured no faster there.
 template <bool KHG, bool MULTI, bool FEW>
 __global__ void __launch_bounds__(SEG_BWD_BLOCK, FEW ? 4 : 5)
 adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
@@ -770,8 +772,8 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, i
             first = false;
             since = since == 0 ? A.every - 1 : since - 1;
             const StepTime T = step_time_from(P, wind, ld_shared4(tab + 16 * (k - G.k_lo)), k);
-            reverse_step<KHG, FEW>(P, A, LV, T, s_rec, s_w, gid, sp, m0, mq, sig_h_uniform, sq2dt,
-                                   X, X.w, Xa, sample, J, wg);
+            reverse_step<KHG, FEW || MULTI>(P, A, LV, T, s_rec, s_w, gid, sp, m0, mq,
+                                            sig_h_uniform, sq2dt, X, X.w, Xa, sample, J, wg);
             Xa = X;
         } while (--k >= kb);
     }
