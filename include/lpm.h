@@ -275,7 +275,9 @@ lpm_status lpm_set_launch(lpm_ctx *ctx, int block, int particles_per_thread, int
  * particles of all scenarios in device memory by the weather cell they occupy, so that
  * the threads of a warp gather from neighbouring cells (a layout change only: every
  * particle keeps its id, hence its random numbers, and all results are bit-identical).
- * 0 turns it off; default 60. A change moves every particle back to its home slot first.
+ * 0 turns it off. Without this call the library sorts by the context's particles: not at
+ * all up to 65536, every 120 steps up to 2^20 (2^19 with dosage, Eq. 3, a decay chain or the
+ * Langevin variant), every 60 above. A change moves every particle back to its home slot.
  * Needs about 60 bytes of extra device memory per particle slot, allocated at the first
  * sort. The sorts do not keep the map from home slots to sorted places: the first
  * lpm_particles, lpm_particle_velocity, lpm_budget or lpm_save after a sort rebuilds it

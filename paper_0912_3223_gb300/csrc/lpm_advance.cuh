@@ -581,8 +581,9 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                 first = tl.first + off;
                 count = max(0, min(32, tl.count - off));
                 tscen = tl.scen;
-                if (!LPM_IN_BOUNDS(P.err, first >= 0 && first + count <= P.slot_cap && tscen >= 0 &&
-                                              tscen < P.n_scen))
+                // (a unit past the end of its tile holds nothing, wherever it would begin)
+                if (!LPM_IN_BOUNDS(P.err, (count == 0 || (first >= 0 && first + count <= P.slot_cap)) &&
+                                              tscen >= 0 && tscen < P.n_scen))
                     count = 0;
             }
             const ScenDev &scg = P.scen[tscen];

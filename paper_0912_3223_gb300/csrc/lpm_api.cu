@@ -114,10 +114,12 @@ struct lpm_ctx {
     bool launch_set = false;                // lpm_set_launch was called; else by size
     int block = 512, ppt = 1, occ = 2;
 
-    // sorting by weather cell (both forms) at the multiples of sort_every: d_state is the
+    // sorting by weather cell (both forms) at the multiples of sort_now: d_state is the
     // home buffer (slot order of the API); the live particles released before sorted_upto
     // sit ordered by cell in d_sorted[cur], the dead ones in d_grave
-    int sort_every = 60;                    // steps between sorts; 0 = off
+    int sort_every = -1;                    // lpm_set_sort's steps between sorts; 0 = off, -1 =
+                                            // not called, by size (sort_interval)
+    int sort_now = 0;                       // the interval that the steps use
     long long sorted_upto = 0;
     int cur = 0;
     float4 *d_sorted[2] = {nullptr, nullptr};
@@ -572,6 +574,22 @@ int tile_particles(const lpm_ctx *c)
     return c->n_slots_used <= (1 << 17) ? 32 : 512;
 }
 
+// Steps between sorts where lpm_set_sort chose none. A sort costs its launches (25 us while
+// few particles move) and cuts the time loop; without it the lanes of a warp drift into other
+// lines of the weather. Up to 2^16 particles, at most 14 warps an SM, the gathers' latency
+// hides either way and the release order itself keeps neighbours together: no sorts (2e4
+// particles x 2880 steps 3.36 ms, 3.88 with one every 120 steps, 4.39 every 60; 65536 x 720
+// 0.83, 0.88 and 1.01; 1.1e5 in 10 scenarios are faster with them, 0.79, 0.72 and 0.80). Up to
+// 2^20, 120 steps (1e5 x 720 1.02 ms against 1.09 at 60; 1e6 4.18 and 4.31; 2e6 7.59 and
+// 7.42), up to 2^19 for the extended step, whose gathers count for more (dose assessment of
+// 5e5 3.95 and 4.13 ms, of 1e6 6.53 and 6.42). Above, 60.
+int sort_interval(const lpm_ctx *c, bool ext)
+{
+    if (c->sort_every >= 0) return c->sort_every;
+    const long long n = c->n_slots_used;
+    return n <= (1 << 16) ? 0 : n <= (ext ? 1 << 19 : 1 << 20) ? 120 : 60;
+}
+
 // Tile table (see lpm_ctx::tiles). A segment [k, e) after the sort at sorted_upto runs
 // the tiles from the interval of sorted_upto up to the last tile whose first particle
 // leaves before e; a sort at a multiple of E takes the tiles of the intervals since the
@@ -580,7 +598,7 @@ lpm_status build_tiles(lpm_ctx *c)
 {
     const int T = tile_particles(c);
     const long long NS = std::max<long long>(1, c->cfg.n_steps);
-    const long long E = c->sort_every > 0 ? c->sort_every : NS;
+    const long long E = c->sort_now > 0 ? c->sort_now : NS;
     const long long n_int = (NS + E - 1) / E;
     c->tiles.clear();
     c->tile_sp.clear();
@@ -1437,13 +1455,20 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
         if (st != LPM_OK) return st;
     }
     const bool ext = (c->d_dose && c->dose_every > 0) || c->kz_model == 1 || c->n_species > 1 ||
-                     c->langevin || c->n_modes > 0;
-    if (ext && c->ppt != 1)
+                     c->langevin;
+    if ((ext || c->n_modes > 0) && c->ppt != 1)
         return fail(c, LPM_E_INVALID, "dosage, K_z from Eq. 3, decay chains, the Langevin "
                                       "variant and perturbation modes run with 1 particle per "
                                       "thread");
     st = upload_tables(c);
     if (st != LPM_OK) return st;
+    if (const int every = sort_interval(c, ext); every != c->sort_now) {
+        // the sort points move: every particle returns home, the next sort starts afresh
+        st = clear_sort_state(c, true);
+        if (st != LPM_OK) return st;
+        c->sort_now = every;
+        c->tiles_valid = false;
+    }
     if (!c->tiles_valid) {
         st = build_tiles(c);
         if (st != LPM_OK) return st;
@@ -1452,7 +1477,7 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
     fill_params(c, P);
     const bool batched = g.n_scenarios > 1;
     const int T = tile_particles(c);
-    const long long E = c->sort_every, Et = c->tiles_E;
+    const long long E = c->sort_now, Et = c->tiles_E;
     const long long k_end = c->k + n;
 
     // ---- plan: segments end at snapshot steps and at multiples of E (sort points) ----------
@@ -2440,7 +2465,7 @@ lpm_status adj_prepare(lpm_ctx *c, const double *rec, int R, double bandwidth, i
         c->adj_tiles_valid = true;
     }
     if (!reuse) {
-        const bool want_sorted = c->sort_every > 0;
+        const bool want_sorted = c->sort_every != 0;
         const lpm_ctx::AdjSorted &S = c->as;
         bool scratch = false;
         lpm_status sst =
