@@ -23,7 +23,8 @@ BUILD = os.path.join(HERE, "_build")
 OUT_CHECKED = os.path.join(HERE, "liblpm_checked.so")
 BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 SOURCES = ["lpm_api.cu", "lpm_kernels.cu", "lpm_advance_b128.cu", "lpm_advance_b256.cu",
-           "lpm_advance_b512.cu", "lpm_adjoint.cu", "lpm_noalloc.cu", "lpm_sort.cu"]
+           "lpm_advance_b512.cu", "lpm_advance_pair.cu", "lpm_adjoint.cu", "lpm_noalloc.cu",
+           "lpm_sort.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

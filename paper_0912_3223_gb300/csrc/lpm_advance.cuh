@@ -205,6 +205,33 @@ __device__ __forceinline__ void dep_words(const StepParams &P, unsigned long lon
     }
 }
 
+// The draws of the steps k and k + 1 of a particle, for DRAWS_GIVEN: the three normals, and in
+// w the deposition tests' outcomes (bit 0 dry, bit 1 wet). dc holds the odd step's words where
+// k is odd (dep_begin) and is left ready for k + 2. Free of branches, so that the two steps'
+// chains overlap.
+__device__ __forceinline__ void draw_pair(const StepParams &P, unsigned long long gid, int k,
+                                          DepCache &dc, float4 &a, float4 &b)
+{
+    const U4 wa = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
+    const U4 wb =
+        philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)(k + 1), 0u, P.rk);
+    normals3(wa, a.x, a.y, a.z);
+    normals3(wb, b.x, b.y, b.z);
+    uint32_t fa = 0u, fb = 0u;
+    if (P.t_dry | P.t_wet) {
+        const bool odd = (k & 1) != 0;
+        const U4 w = dep_block(P, gid, k + 1);   // of the even one of the two steps
+        fa = ((odd ? dc.c : w.a) < P.t_dry ? 1u : 0u) | ((odd ? dc.d : w.b) < P.t_wet ? 2u : 0u);
+        fb = ((odd ? w.a : w.c) < P.t_dry ? 1u : 0u) | ((odd ? w.b : w.d) < P.t_wet ? 2u : 0u);
+        dc.c = w.c;
+        dc.d = w.d;
+    }
+    a.w = __uint_as_float(fa);
+    b.w = __uint_as_float(fb);
+}
+
+enum { DRAWS_LAST = 0, DRAWS_FIRST = 1, DRAWS_GIVEN = 2 };
+
 // Per-step quantities shared by every particle of a tile.
 struct StepTime {
     int k;
@@ -371,33 +398,41 @@ __device__ __forceinline__ Met sample_met_pair(const StepParams &P, const LEV &L
 // particle's scenario plus the bias at t_k. With GRIDS, deposition and exit add their mass
 // to the scenario's grids and counters; *fold receives dz/dz_pre (+-1, 0 when clamped).
 // FIELDS: the run may have a gridded K_h or the drift correction (uniform run-time tests).
-// DRAWS_FIRST: the draws stand before the gathers, so that the two overlap where registers
-// allow it (measured at 128 registers a thread: 2e4 particles over a day 4.55 -> 4.38 ms; at
-// 64 it costs spills: 1e7 particles 40.8 -> 41.9 ms).
+// DRAWS: where the draws come from. DRAWS_FIRST: they stand before the gathers, so that the two
+// overlap where registers allow it (measured at 128 registers a thread: 2e4 particles over a day
+// 4.55 -> 4.38 ms; at 64 it costs spills: 1e7 particles 40.8 -> 41.9 ms); DRAWS_LAST: after
+// them; DRAWS_GIVEN: `given` holds them (draw_pair).
 template <bool GRIDS, bool EXT = false, class LEV, bool MODES = EXT, bool FIELDS = true,
-          bool DRAWS_FIRST = false>
+          int DRAWS = DRAWS_LAST>
 __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV &LV,
                                                   const StepTime &T, const ScenDev &sc,
                                                   const ScenDev *scg, unsigned long long gid,
                                                   int sp, float sig_h_uniform, float du, float dv,
                                                   float &x, float &y, float &z, float *fold,
                                                   float *wv = nullptr, const float *msc = nullptr,
-                                                  DepCache *dc = nullptr)
+                                                  DepCache *dc = nullptr,
+                                                  float4 given = make_float4(0.f, 0.f, 0.f, 0.f))
 {
     const int k = T.k;
     float n0, n1, n2;
     auto draw = [&]() {
+        if (DRAWS == DRAWS_GIVEN) {
+            n0 = given.x;
+            n1 = given.y;
+            n2 = given.z;
+            return;
+        }
         const U4 w = philox4x32_10_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0u, P.rk);
         normals3(w, n0, n1, n2);
     };
-    if (DRAWS_FIRST) draw();
+    if (DRAWS != DRAWS_LAST) draw();
     // 1. weather at the old position and t_k (with the scenario's perturbation modes: msc);
     // 2. diffusivities
     const Met m = sample_met_pair<EXT, LEV, MODES, FIELDS>(P, LV, T, x, y, z, msc);
     const float sig_h = FIELDS && P.khpair ? sqrtf(P.k2 * m.kh * P.dt) : sig_h_uniform;
     const float sig_z = sqrtf(P.k2 * m.kz * P.dt);
     // 3. N(0,1) draws
-    if (!DRAWS_FIRST) draw();
+    if (DRAWS == DRAWS_LAST) draw();
     // 4. Eq. (1)-(2): wind then turbulent displacement
     // (fused multiply-adds, written out: every instantiation rounds alike)
     const float xn = __fmaf_rn(n0, sig_h, __fmaf_rn(m.u + du, P.dt, x));
@@ -462,14 +497,22 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
             return ST_EXITED;
         }
     }
-    if (!(P.t_dry | P.t_wet)) return ST_ACTIVE;
     // 6. dry deposition below the mixing height, then wet where it rains
-    uint32_t w_dry, w_wet;
-    dep_words(P, gid, k, dc, w_dry, w_wet);
-    if (!((w_dry < P.t_dry) | (w_wet < P.t_wet))) return ST_ACTIVE;
+    bool dry, wet;
+    if (DRAWS == DRAWS_GIVEN) {
+        dry = __float_as_uint(given.w) & 1u;
+        wet = __float_as_uint(given.w) & 2u;
+    } else {
+        if (!(P.t_dry | P.t_wet)) return ST_ACTIVE;
+        uint32_t w_dry, w_wet;
+        dep_words(P, gid, k, dc, w_dry, w_wet);
+        dry = w_dry < P.t_dry;
+        wet = w_wet < P.t_wet;
+    }
+    if (!(dry | wet)) return ST_ACTIVE;
     int kind = -1;
-    if (w_dry < P.t_dry && zn < P.h_mix) kind = 0;
-    if (kind < 0 && w_wet < P.t_wet && P.rain) {
+    if (dry && zn < P.h_mix) kind = 0;
+    if (kind < 0 && wet && P.rain) {
         int ir = (int)floorf((xn - P.x0) * P.inv_dx + 0.5f);
         int jr = (int)floorf((yn - P.y0) * P.inv_dy + 0.5f);
         ir = min(max(ir, 0), P.nx - 1);
@@ -497,10 +540,19 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
 }
 
 // Occupancy variants: the register budget per thread is 128 (OCC 0), 80 (OCC 1) or 64
-// (OCC 2), i.e. 16, 24 or 32 resident warps per SM.
+// (OCC 2), i.e. 16, 24 or 32 resident warps per SM. OCC_PAIR: 128, and warps in pairs, one of
+// which draws for the other.
+//
+// With at most two warps of particles a scheduler a step is one chain of dependent instructions
+// (1500 cycles for the 430 of the plain step). 40 % of them are the draws, which depend on the
+// particle's id and the step alone: in an OCC_PAIR block half of the warps compute them up to
+// PAIR_STEPS steps ahead for the other half, through two buffers in shared memory, with one
+// barrier of the pair's 64 threads a buffer. 2160 particles x 2160 steps 1.74 -> 1.32 ms, 2e4 x
+// 2880 3.36 -> 2.93, 38900 x 720 0.76 -> 0.68, 6 members x 240 0.36 -> 0.32; buffers of 4 or 16
+// steps 5 and 1 % slower, a pair on one scheduler 9 %.
 template <int BLOCK, int OCC>
 struct MinBlocks {
-    static constexpr int per_sm_threads = OCC == 0 ? 512 : OCC == 1 ? 768 : 1024;
+    static constexpr int per_sm_threads = OCC == 0 || OCC == OCC_PAIR ? 512 : OCC == 1 ? 768 : 1024;
     static constexpr int value = per_sm_threads / BLOCK > 0 ? per_sm_threads / BLOCK : 1;
 };
 
@@ -533,9 +585,12 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
     __shared__ unsigned long long s_steps;
     __shared__ unsigned int s_tile;
     __shared__ StepTable s_tab;                      // the launch's step times
+    constexpr bool PAIR = OCC == OCC_PAIR;
     // Units of a warp's 32 particles: those of A, then those of the B tiles. (A launch of the
     // pair that has another number of units for its shape has nothing to do.)
-    constexpr unsigned int WARPS = BLOCK / 32;
+    constexpr unsigned int WARPS = BLOCK / (PAIR ? 64 : 32);
+    __shared__ float4 s_draw[PAIR ? WARPS : 1][2][PAIR ? PAIR_STEPS : 1][32];
+    __shared__ int s_stop[PAIR ? WARPS : 1][2];      // the pair's particles have all stopped
     const long long live = R.a_live ? (long long)*R.a_live : 0;
     const unsigned int units_a = (unsigned int)((live + 31) >> 5);
     const unsigned int n_units = units_a + ((unsigned int)R.n_b << R.unit_shift);
@@ -546,7 +601,11 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                                     s_adv_dyn);
     unsigned long long *s_warp = s_acc + (threadIdx.x & ~31);
     const int lane = threadIdx.x & 31;
-    const unsigned int warp = threadIdx.x >> 5;
+    // a pair's warps sit on different schedulers, and two pairs of a block on all four: warps
+    // 0 1 and 6 7 move particles, 2 3 and 4 5 draw for them
+    const unsigned int w = threadIdx.x >> 5;
+    const unsigned int warp = PAIR ? (w & 1u) + 2u * (w >> 2) : w;
+    const bool drawer = PAIR && (((w >> 1) ^ (w >> 2)) & 1u);
     const long long n_cells = (long long)P.cx * P.cy * P.cz;
     // the uniform horizontal diffusivity gives one displacement scale for the run
     const float sig_h_uniform = sqrtf(P.k2 * fmaxf(P.kh_uniform, 0.0f) * P.dt);
@@ -625,9 +684,9 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                 k = sp;
             }
             const int k_own = k;                            // this lane's first step
-            DepCache dc;                                    // odd-step deposition words
+            DepCache dc{0u, 0u};                            // odd-step deposition words
             if (st == ST_ACTIVE) dep_begin(P, gid, k, dc);
-            auto advance = [&](int k) {
+            auto advance = [&](int k, float4 given = make_float4(0.f, 0.f, 0.f, 0.f)) {
                 const StepTime T = step_time_tab<FIELDS || EXT || MIXED>(tab, k - k0, k);
                 float du = T.du, dv = T.dv;
                 if (MIXED && P.woff) {
@@ -641,11 +700,57 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
                     du = P.bias_u + fmaf(T.f, o1.x - o0.x, o0.x);
                     dv = P.bias_v + fmaf(T.f, o1.y - o0.y, o0.y);
                 }
-                return particle_step<true, EXT, Lev, MODES, FIELDS, OCC != 2>(
+                return particle_step<true, EXT, Lev, MODES, FIELDS,
+                                     PAIR ? DRAWS_GIVEN : OCC != 2 ? DRAWS_FIRST : DRAWS_LAST>(
                     P, LV, T, sc, &sc, gid, sp, sig_h_uniform, du, dv, x, y, z, nullptr,
-                    lang ? &wv : nullptr, msc, &dc);
+                    lang ? &wv : nullptr, msc, &dc, given);
             };
-            if (!EXT || !P.dose_every) {
+            if constexpr (PAIR) {
+                // Both warps of the pair loaded the same particles, so both come to the same
+                // number of turns, and to the same barriers; a turn that finds s_stop set ends
+                // both. The drawer reads s_stop[h] between barriers n and n + 1 (n = h mod 2),
+                // its partner writes it next between n + 1 and n + 2; the buffers likewise.
+                const int turns =
+                    (__reduce_max_sync(0xffffffffu, st == ST_ACTIVE ? k1 - k_own : 0) +
+                     PAIR_STEPS - 1) / PAIR_STEPS;
+                float4(*buf)[PAIR_STEPS][32] = s_draw[warp];
+                auto fill = [&](int turn) {
+#pragma unroll 1
+                    for (int j = 0; j < PAIR_STEPS; j += 2) {
+                        float4 a, b;
+                        draw_pair(P, gid, k_own + turn * PAIR_STEPS + j, dc, a, b);
+                        buf[turn & 1][j][lane] = a;
+                        buf[turn & 1][j + 1][lane] = b;
+                    }
+                };
+                if (drawer && turns > 0) fill(0);
+#pragma unroll 1
+                for (int turn = 0; turn < turns; ++turn) {
+                    if (!drawer) {
+                        const bool stop = !__any_sync(0xffffffffu, st == ST_ACTIVE && k < k1);
+                        if (lane == 0) s_stop[warp][turn & 1] = stop;
+                    }
+                    __syncwarp();
+                    asm volatile("bar.sync %0, 64;" ::"r"((int)warp + 1) : "memory");
+                    if (*(volatile int *)&s_stop[warp][turn & 1]) break;
+                    if (drawer) {
+                        if (turn + 1 < turns) fill(turn + 1);
+                    } else {
+#pragma unroll 1
+                        for (int j = 0; j < PAIR_STEPS; ++j) {
+                            if (st == ST_ACTIVE && k < k1) {
+                                st = advance(k, buf[turn & 1][j][lane]);
+                                ++k;
+                            }
+                        }
+                    }
+                }
+                steps = (unsigned int)(k - k_own);
+                if (drawer) {                               // its partner has the results
+                    count = 0;
+                    st = ST_EXITED;
+                }
+            } else if (!EXT || !P.dose_every) {
                 if (st == ST_ACTIVE) {
 #pragma unroll 1
                     do {
@@ -693,7 +798,7 @@ advance_kernel(const StepParams P, const Ranges R, unsigned int *queue, int k0, 
             }
 
             // ---- sort keys for the sort that follows (its inputs: A slots, then B lanes) ----
-            if (R.keys) {
+            if (R.keys && !drawer) {
                 const unsigned int dead_key =
                     (unsigned int)sort_dead_key(P.nx, P.ny, P.nz, R.key_shift, 0);
                 long long idx = -1;
@@ -781,7 +886,8 @@ void adv_prefer_l1()
     // the kernel needs a few KB of shared memory per block: ask for a small carve-out so the
     // rest of the SM's unified L1 serves the weather gathers (measured +0.7 to +1.7 %)
     cudaFuncSetAttribute(advance_kernel<BLOCK, OCC, MIXED, EXT, MODES, FIELDS, TABLE>,
-                         cudaFuncAttributePreferredSharedMemoryCarveout, 10);
+                         cudaFuncAttributePreferredSharedMemoryCarveout,
+                         OCC == OCC_PAIR ? 40 : 10);
     (void)cudaGetLastError();
 }
 
@@ -844,5 +950,36 @@ int occ_adv(size_t smem)
         }                                                                              \
         return 0;                                                                      \
     }
+
+#define LPM_ADVANCE_PAIR_TU(BLOCK)                                                     \
+    cudaError_t launch_advance_pair(const AdvanceLaunch &L)                             \
+    {                                                                                  \
+        switch (L.mixed * 10 + L.variant()) {                                          \
+            LPM_ADV_CASES_PAIR(launch_adv, BLOCK, L)                                   \
+        }                                                                              \
+        return cudaErrorInvalidValue;                                                  \
+    }                                                                                  \
+    int occupancy_pair(bool mixed, int variant, size_t smem)                           \
+    {                                                                                  \
+        switch (mixed * 10 + variant) {                                                \
+            LPM_ADV_CASES_PAIR(occ_adv, BLOCK, smem)                                   \
+        }                                                                              \
+        return 0;                                                                      \
+    }
+#define LPM_ADV_CASE_PAIR(FN, BLOCK, MIX, VAR, ...)                                    \
+    case MIX * 10 + VAR:                                                               \
+        return FN<BLOCK, OCC_PAIR, (MIX != 0), false,                                  \
+                  (VAR == ADV_MODES || VAR == ADV_MODES_FIELDS),                       \
+                  (VAR == ADV_FIELDS || VAR == ADV_MODES_FIELDS),                      \
+                  (VAR == ADV_PLAIN || VAR == ADV_MODES)>(__VA_ARGS__);
+#define LPM_ADV_CASES_PAIR(FN, BLOCK, ...)                                             \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 0, 0, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 0, 2, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 0, 3, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 0, 4, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 1, 0, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 1, 2, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 1, 3, __VA_ARGS__)                                    \
+    LPM_ADV_CASE_PAIR(FN, BLOCK, 1, 4, __VA_ARGS__)
 
 }  // namespace lpm

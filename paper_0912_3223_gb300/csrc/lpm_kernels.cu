@@ -201,6 +201,7 @@ cudaError_t launch_release_all(cudaStream_t s, const StepParams &P, float4 *stat
 
 cudaError_t launch_advance(const AdvanceLaunch &L)
 {
+    if (L.occ == OCC_PAIR) return launch_advance_pair(L);
     switch (L.block) {
     case 128: return launch_advance_b128(L);
     case 256: return launch_advance_b256(L);
@@ -211,6 +212,7 @@ cudaError_t launch_advance(const AdvanceLaunch &L)
 
 int advance_occupancy(int block, int occ, bool mixed, int variant, size_t smem)
 {
+    if (occ == OCC_PAIR) return occupancy_pair(mixed, variant, smem);
     switch (block) {
     case 128: return occupancy_b128(occ, mixed, variant, smem);
     case 256: return occupancy_b256(occ, mixed, variant, smem);

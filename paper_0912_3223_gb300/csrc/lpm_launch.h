@@ -53,6 +53,10 @@ struct Ranges {
 // Longest launch in steps: its step times sit in a table in shared memory.
 constexpr int STEP_TAB = 128;
 
+// AdvanceLaunch::occ of blocks whose warps work in pairs (256 threads, not the extended step),
+// and the steps that one draws ahead for the other.
+constexpr int OCC_PAIR = 3, PAIR_STEPS = 8;
+
 // Options of an advance launch, by the instantiation that carries their code: none; the
 // extended step (dosage, Eq. 3 K_z, a decay chain, the Langevin variant, with anything else);
 // perturbation modes; a gridded K_h, the drift correction or levels without a lookup table;
@@ -202,9 +206,11 @@ cudaError_t launch_advance(const AdvanceLaunch &L);
 int advance_occupancy(int block, int occ, bool mixed, int variant, size_t smem);
 cudaError_t launch_advance_b128(const AdvanceLaunch &L);
 cudaError_t launch_advance_b256(const AdvanceLaunch &L);
+cudaError_t launch_advance_pair(const AdvanceLaunch &L);
 cudaError_t launch_advance_b512(const AdvanceLaunch &L);
 int occupancy_b128(int occ, bool mixed, int variant, size_t smem);
 int occupancy_b256(int occ, bool mixed, int variant, size_t smem);
+int occupancy_pair(bool mixed, int variant, size_t smem);
 int occupancy_b512(int occ, bool mixed, int variant, size_t smem);
 cudaError_t launch_pack(cudaStream_t s, const float4 *a, const float4 *b, const float *ka,
                         const float *kb, float4 *pair, float2 *khpair, int nx, int ny, int nz);
