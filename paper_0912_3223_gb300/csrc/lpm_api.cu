@@ -1250,18 +1250,20 @@ struct Segment {
 //  - up to 8 warps an SM, all that fit at once in pairs: one warp draws for the other (OCC_PAIR;
 //    not the extended step). 500 to 38900 particles over 720 steps 0.62 to 0.68 ms against 0.75
 //    to 0.79 in the next shape;
-//  - up to 20 warps an SM, 128 registers a thread (16 at a time): a step's latency is all that counts, and
-//    its eight gathers fly together. Advance of 2e4 particles over a day: 4.2 ms against 7.2 at
-//    64 registers. From 16 warps an SM on it takes a second round, still the faster one at 20
-//    (2e5 particles x 720 steps 1.70 ms against 1.84 at 80 registers) and no longer at 24.
-//    Blocks of 256 except where there are fewer warps than schedulers;
-//  - up to 1e6 particles, and the extended step at any size, 80 registers (24 warps): 3e5
-//    particles x 720 steps 2.08 ms against 2.22 at 64 registers, dose assessment 3.9 against 4.3
-//    (the extended step spills at 64);
-//  - above, and with mixed scenarios, 64 registers (32 warps): 1e7 particles 40.8 ms against
-//    42.5, 64 scenarios 59 against 66.
-// `units` counts every particle released so far; where the bound leaves open which of the
-// first two is the better one, both are launched and the device's live count lets one of them
+//  - up to 216 warps an SM (1e6 particles), 75 for the extended step and for mixed scenarios,
+//    128 registers a thread (16 warps at a time): a step's latency counts, its eight gathers fly
+//    together, and small blocks share the work out evenly. Runs that released 4e5 particles in
+//    720 steps 1.95 ms against 2.30 at 80 registers and 2.16 at 64; 6e5 2.60, 2.80, 3.03; 1e6
+//    4.05, 4.16, 4.14; 1.5e6 5.83, 5.82, 5.78; dose assessment of 5e5 3.85, 3.98, 4.36, of 1e6
+//    6.69, 6.39, 6.59 (6.46 with the limit at 75, 6.71 at 108); 32 scenarios of together 4e5
+//    1.68, 1.83, 1.84; 24 of 7.6e5 2.85, 2.80, 2.65 (2.67 with the limit, 2.74 at 108). Blocks
+//    of 256 except where there are fewer warps than schedulers;
+//  - the extended step up to 1e6 particles, 80 registers (24 warps);
+//  - above, and with mixed scenarios, 64 registers (32 warps): 3e6 particles 10.5 ms against
+//    10.9 at 80 registers and 11.1 at 128, 64 scenarios 58.1, 63.1 and 65.7, dose assessment of
+//    2e6 11.2, 11.5 and 12.5.
+// `units` counts every particle released so far; where the bound leaves open which of two
+// shapes is the better one, both are launched and the device's live count lets one of them
 // return at once (2 us).
 struct Shape {
     int block, occ, blocks;            // blocks: the persistent grid's limit
@@ -1271,20 +1273,20 @@ struct Shape {
 int launch_shapes(const lpm_ctx *c, const StepParams &P, long long units, Shape h[2])
 {
     constexpr unsigned int ANY = 0xffffffffu;
-    const unsigned int few = 20u * (unsigned int)c->sm_count;
     const int variant = adv_variant(P);
-    const bool mixed = P.n_scen > 1;
+    const bool mixed = P.n_scen > 1, ext = adv_is_ext(variant);
+    const unsigned int few = (mixed || ext ? 75u : 216u) * (unsigned int)c->sm_count;
     int n = 0;
     if (c->launch_set) {
         h[n++] = {c->block, c->occ, 0, 0u, ANY};
-    } else if (units <= 8LL * c->sm_count && !adv_is_ext(variant)) {
+    } else if (units <= 8LL * c->sm_count && !ext) {
         h[n++] = {256, OCC_PAIR, 0, 0u, ANY};
     } else {
         const bool small = units <= few, large = units > 8LL * few;
         if (!large)
             h[n++] = {units <= 4LL * c->sm_count ? 512 : 256, 0, 0, 0u, small ? ANY : few};
         if (!small) {
-            const bool wide = !adv_is_ext(variant) && (mixed || units > 32768);
+            const bool wide = (mixed && !ext) || units > 216LL * c->sm_count;
             h[n++] = {wide ? 512 : 256, wide ? 2 : 1, 0, large ? 0u : few + 1u, ANY};
         }
     }
