@@ -571,8 +571,10 @@ struct MinBlocks {
 // the drift correction. TABLE: the levels have a lookup table. The plain instantiations carry
 // none of that code.
 //
-// Bound by issued instructions (32 warps an SM keep the schedulers 75 % busy, DRAM idle), so
-// the step is kept short of branches and constant loads. A lane's time loop starts at its own
+// Bound by issued instructions and the gathers (at 64 registers 32 warps an SM keep the
+// schedulers 70 % busy and the L1 data pipe 58 %, DRAM idle; 549 -> 399 instructions a warp step,
+// a mid-run launch of 1e7 particles 1.006 -> 0.782 ms), so the step is kept short of branches
+// and constant loads. A lane's time loop starts at its own
 // release step and ends with the particle: no status is tested inside it, and the lanes of a
 // tile of late releases all work from the loop's first turn. (The dosage samples gather a
 // warp's lanes at the same step, so with them the loop runs over common steps.)
