@@ -342,7 +342,7 @@ void fill_params(const lpm_ctx *c, StepParams &P)
         const float z0 = (float)c->zlev[k];
         const float inv = k + 1 < g.nz ? 1.0f / ((float)c->zlev[k + 1] - z0) : 0.0f;
         P.zi[k] = make_float2(z0, inv);
-        P.znext[k] = k < g.nz - 2 ? (float)c->zlev[k + 1] : std::numeric_limits<float>::infinity();
+        P.znext[k] = k < g.nz - 2 ? (float)c->zlev[k + 1] : std::numeric_limits<float>::quiet_NaN();
     }
     P.dt = (float)g.dt;
     P.kh_uniform = (float)g.kh_uniform;
