@@ -105,9 +105,10 @@ __device__ __forceinline__ void sample_met_grad(const StepParams &P, const LEV &
 
 // The time parts of step k as step_time computes them (without an offset), packed for a
 // per-block table: the steps of a segment are the same for every particle.
+template <bool ONCE>
 __device__ __forceinline__ float4 step_time_parts(const StepParams &P, int k)
 {
-    const StepTime T = step_time(P, nullptr, k);
+    const StepTime T = step_time<ONCE>(P, nullptr, k);
     const unsigned long long p = reinterpret_cast<unsigned long long>(T.pair);
     return make_float4(__uint_as_float((unsigned int)p), __uint_as_float((unsigned int)(p >> 32)),
                        T.f, __int_as_float(T.h0));
@@ -215,7 +216,7 @@ adj_forward_kernel(const StepParams P, const AdjParams A)
         for (int k = sp; k < A.n_steps; ++k) {
             if (!TRAJ && k > sp && k % CK == 0)
                 A.ckpt[(long long)(k / CK) * A.n_slots + slot] = pack_state(x, y, z, ST_ACTIVE, sp);
-            const StepTime T = step_time(P, sc.wind_offset, k);
+            const StepTime T = step_time<true>(P, sc.wind_offset, k);
             const float xb = x, yb = y, zb = z;
             float fs = 1.0f;
             st = particle_step<false>(P, LV, T, sc, nullptr, gid, sp, sig_h_uniform, T.du, T.dv,
@@ -418,7 +419,7 @@ adj_backward_kernel(const StepParams P, const AdjParams A)
         for (int k = k_lo; k < k_hi; ++k) {
             if (alive && k >= kstart) {
                 seg[k - k_lo] = make_float4(x, y, z, 0.f);
-                const StepTime T = step_time(P, sc.wind_offset, k);
+                const StepTime T = step_time<true>(P, sc.wind_offset, k);
                 float fs;
                 const uint32_t st = particle_step<false>(P, LV, T, sc, nullptr, gid, sp,
                                                          sig_h_uniform, T.du, T.dv, x, y, z,
@@ -435,7 +436,7 @@ adj_backward_kernel(const StepParams P, const AdjParams A)
             if (!(run && k >= kstart && k <= klast)) continue;
             const int i = k - k_lo;
             const bool sample = (k + 1) % A.every == 0 && !(ev && k == klast);
-            reverse_step<KHG>(P, A, LV, step_time(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0,
+            reverse_step<KHG>(P, A, LV, step_time<true>(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0,
                               mq, sig_h_uniform, sq2dt, seg[i], (float)sfold[i], seg[i + 1],
                               sample, J);
         }
@@ -497,7 +498,7 @@ adj_backward_traj_kernel(const StepParams P, const AdjParams A)
             Xn = __ldcs(row + (long long)(k - 1 - k0) * ADJ_BLOCK);
         if (!act) continue;
         const bool sample = (k + 1) % A.every == 0 && !(ev && k == kn - 1);
-        reverse_step<KHG>(P, A, LV, step_time(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0, mq,
+        reverse_step<KHG>(P, A, LV, step_time<true>(P, sc.wind_offset, k), s_rec, s_w, gid, sp, m0, mq,
                           sig_h_uniform, sq2dt, X, X.w, Xa, sample, J);
         Xa = X;
     }
@@ -617,7 +618,7 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
     __shared__ float4 s_ent[Lev::SMEM ? MAX_LEVELS : 1];
     const Lev LV = load_levels<Lev>(P, s_lut, s_ent);
     for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += BLOCK)
-        s_ta[i] = step_time_parts(P, G.k_lo + i);
+        s_ta[i] = step_time_parts<true>(P, G.k_lo + i);
     if (SAMPLE) {
         for (int r = threadIdx.x; r < A.R; r += BLOCK) s_rec[r] = A.rec[r];
         for (int r = threadIdx.x; r < GROUPS * A.R; r += BLOCK) s_C[r] = 0.0;
@@ -721,7 +722,7 @@ adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, i
     // the segment's step times, once per block
     __shared__ float4 s_ta[CK];
     for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_BWD_BLOCK)
-        s_ta[i] = step_time_parts(P, G.k_lo + i);
+        s_ta[i] = step_time_parts<false>(P, G.k_lo + i);
     const int group = group0 + gi;
     const bool from_a = group < G.tiles_a;
     const bool used = group < n_groups && (!from_a || (long long)group * ADJ_BLOCK < (long long)live);

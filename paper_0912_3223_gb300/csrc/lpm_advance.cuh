@@ -255,11 +255,12 @@ __device__ __forceinline__ float2 step_offset(const StepParams &P, const float2 
     return d;
 }
 
+template <bool ONCE = false>
 __device__ __forceinline__ StepTime step_time(const StepParams &P, const float2 *wind_offset, int k)
 {
     StepTime T;
     T.k = k;
-    TimeSlab ts = time_slab(P, (float)k * P.dt);
+    TimeSlab ts = time_slab(P, step_since<ONCE>(P, k));
     if (!LPM_IN_BOUNDS(P.err, ts.h0 >= 0 && ts.h0 < P.n_pair)) ts.h0 = 0;
     T.h0 = ts.h0;
     T.f = ts.f;
@@ -344,7 +345,7 @@ __device__ __forceinline__ Met sample_met_pair(const StepParams &P, const LEV &L
     m.w = r.z;
     if (MODES && msc) {
         float du, dv;
-        mode_wind(P, msc, k, c, x, y, (float)T.k * P.dt, du, dv);
+        mode_wind(P, msc, k, c, x, y, step_start(P, T.k), du, dv);
         m.u += du;
         m.v += dv;
     }
@@ -517,7 +518,7 @@ __device__ __forceinline__ uint32_t particle_step(const StepParams &P, const LEV
         int jr = (int)floorf((yn - P.y0) * P.inv_dy + 0.5f);
         ir = min(max(ir, 0), P.nx - 1);
         jr = min(max(jr, 0), P.ny - 1);
-        int hr = (int)floorf(__fdiv_rn((float)k * P.dt - P.met_t0, P.met_dt));
+        int hr = (int)floorf(__fdiv_rn(step_since<!GRIDS>(P, k), P.met_dt));
         hr = min(max(hr, 0), P.n_t - 1);
         if (__ldg(P.rain + ((long long)hr * P.ny + jr) * P.nx + ir)) kind = 1;
     }
