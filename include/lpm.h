@@ -18,7 +18,8 @@
  *  - Work is enqueued asynchronously on the CUDA stream given to lpm_create(). The
  *    read-back calls (lpm_concentration, lpm_deposition, lpm_budget, lpm_particles,
  *    lpm_fixed_state, lpm_sync) synchronise that stream and report device-side errors
- *    (LPM_E_NUMERIC for a non-finite particle position).
+ *    (LPM_E_NUMERIC for a non-finite particle position), on which the caller's arrays stay as
+ *    they are.
  *  - A context is used by one host thread at a time.
  *  - Lengths are SI (m, s), masses are in the unit of the emission rate times seconds.
  */

@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <limits>
 #include <string>
 #include <vector>
@@ -517,8 +518,8 @@ lpm_status upload_tables(lpm_ctx *c)
     return LPM_OK;
 }
 
-// Synchronises the context's streams and reports device-side errors: the last call of every
-// read-back, after the copies that it enqueued, so that one wait serves both.
+// Synchronises the context's streams and reports device-side errors: every read-back's wait for
+// the kernels it enqueued, before anything is copied to the caller's arrays (read_back).
 lpm_status check_device_error(lpm_ctx *c)
 {
     LPM_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_err, sizeof(unsigned int), cudaMemcpyDeviceToHost,
@@ -1626,21 +1627,39 @@ lpm_status conv_room(lpm_ctx *c, size_t bytes)
 }
 
 // Enqueues the conversion of n 64-bit fixed-point sums to doubles (x f, / d) at element `at`
-// of the scratch, and the copy of the first n0 of them to out0 and the rest to out1 (either
-// may be nullptr).
-lpm_status read_fixed(lpm_ctx *c, const unsigned long long *src, size_t n, double f, double d,
-                      size_t at, double *out0, size_t n0, double *out1)
+// of the scratch.
+lpm_status convert_fixed(lpm_ctx *c, const unsigned long long *src, size_t n, double f, double d,
+                         size_t at)
 {
-    double *conv = reinterpret_cast<double *>(c->d_conv) + at;
-    LPM_CUDA(c, launch_fixed_to_double(c->stream, src, conv, (long long)n, f, d));
+    LPM_CUDA(c, launch_fixed_to_double(c->stream, src, reinterpret_cast<double *>(c->d_conv) + at,
+                                       (long long)n, f, d));
     c->n_launches++;
-    if (out0)
-        LPM_CUDA(c, cudaMemcpyAsync(out0, conv, n0 * sizeof(double), cudaMemcpyDeviceToHost,
-                                    c->stream));
-    if (out1)
-        LPM_CUDA(c, cudaMemcpyAsync(out1, conv + n0, (n - n0) * sizeof(double),
-                                    cudaMemcpyDeviceToHost, c->stream));
     return LPM_OK;
+}
+
+// A read-back's copies to the caller's arrays (a nullptr is left out), once the device has
+// reported no error: on one, they stay as they are. A failed copy waits for those before it.
+struct CopyOut {
+    void *dst;
+    const void *src;
+    size_t bytes;
+};
+
+lpm_status read_back(lpm_ctx *c, std::initializer_list<CopyOut> copies, bool check = true)
+{
+    if (check) {
+        const lpm_status st = check_device_error(c);
+        if (st != LPM_OK) return st;
+    }
+    cudaError_t e = cudaSuccess;
+    for (const CopyOut &k : copies)
+        if (k.dst && e == cudaSuccess)
+            e = cudaMemcpyAsync(k.dst, k.src, k.bytes, cudaMemcpyDeviceToHost, c->stream);
+    const cudaError_t done = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) e = done;
+    if (e == cudaSuccess) return LPM_OK;
+    (void)cudaGetLastError();
+    return fail(c, LPM_E_CUDA, "copying a read-back failed: %s", cudaGetErrorString(e));
 }
 }  // namespace
 
@@ -1654,8 +1673,8 @@ lpm_status lpm_concentration(lpm_ctx *c, int scenario, double *out, size_t n_out
     const double f = std::ldexp(1.0, -c->scen[(size_t)scenario].shift) / (g.cdx * g.cdy * g.cdz);
     lpm_status st = conv_room(c, n_out * sizeof(double));
     if (st != LPM_OK) return st;
-    st = read_fixed(c, c->d_conc + (size_t)scenario * n_out, n_out, f, 1.0, 0, out, n_out, nullptr);
-    return st != LPM_OK ? st : check_device_error(c);
+    st = convert_fixed(c, c->d_conc + (size_t)scenario * n_out, n_out, f, 1.0, 0);
+    return st != LPM_OK ? st : read_back(c, {{out, c->d_conv, n_out * sizeof(double)}});
 }
 
 lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, size_t n_out)
@@ -1668,11 +1687,11 @@ lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, si
     lpm_status st = conv_room(c, 2 * plane * sizeof(double));
     if (st != LPM_OK) return st;
     if (dry || wet) {
-        st = read_fixed(c, c->d_dep + (size_t)scenario * c->ndep(), 2 * plane, f, 1.0, 0, dry, plane,
-                        wet);
+        st = convert_fixed(c, c->d_dep + (size_t)scenario * c->ndep(), 2 * plane, f, 1.0, 0);
         if (st != LPM_OK) return st;
     }
-    return check_device_error(c);
+    const size_t bytes = plane * sizeof(double);
+    return read_back(c, {{dry, c->d_conv, bytes}, {wet, c->d_conv + bytes, bytes}});
 }
 
 lpm_status lpm_budget(lpm_ctx *c, int scenario, double out[8])
@@ -1745,14 +1764,11 @@ lpm_status lpm_particles(lpm_ctx *c, int64_t first, int64_t count, float *xyz, u
                                       sorted ? c->d_slot_of : nullptr, c->d_grave, first + at, n,
                                       xyz ? d_xyz : nullptr, tag ? d_tag : nullptr));
         c->n_launches++;
-        if (xyz)
-            LPM_CUDA(c, cudaMemcpyAsync(xyz + 3 * at, d_xyz, (size_t)n * 3 * sizeof(float),
-                                        cudaMemcpyDeviceToHost, c->stream));
-        if (tag)
-            LPM_CUDA(c, cudaMemcpyAsync(tag + at, d_tag, (size_t)n * sizeof(uint32_t),
-                                        cudaMemcpyDeviceToHost, c->stream));
+        st = read_back(c, {{xyz ? xyz + 3 * at : nullptr, d_xyz, (size_t)n * 3 * sizeof(float)},
+                           {tag ? tag + at : nullptr, d_tag, (size_t)n * sizeof(uint32_t)}}, at == 0);
+        if (st != LPM_OK) return st;
     }
-    return check_device_error(c);
+    return count == 0 || !(xyz || tag) ? check_device_error(c) : LPM_OK;
 }
 
 lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_conc, uint64_t *dep,
@@ -1763,14 +1779,10 @@ lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_co
     if (conc && n_conc != c->ncell()) return fail(c, LPM_E_INVALID, "n_conc must be %zu", c->ncell());
     if (dep && n_dep != c->ndep()) return fail(c, LPM_E_INVALID, "n_dep must be %zu", c->ndep());
     lpm_status st = LPM_OK;
-    if (conc)
-        LPM_CUDA(c, cudaMemcpyAsync(conc, c->d_conc + (size_t)scenario * c->ncell(),
-                                    n_conc * sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
-    if (dep)
-        LPM_CUDA(c, cudaMemcpyAsync(dep, c->d_dep + (size_t)scenario * c->ndep(),
-                                    n_dep * sizeof(uint64_t), cudaMemcpyDeviceToHost, c->stream));
     if (counters && (st = read_counters(c, scenario)) != LPM_OK) return st;
-    if ((st = check_device_error(c)) != LPM_OK) return st;
+    st = read_back(c, {{conc, c->d_conc + (size_t)scenario * c->ncell(), n_conc * sizeof(uint64_t)},
+                       {dep, c->d_dep + (size_t)scenario * c->ndep(), n_dep * sizeof(uint64_t)}});
+    if (st != LPM_OK) return st;
     if (counters) {
         for (int i = 0; i < 16; ++i) counters[i] = (int64_t)c->h_words[1 + i];
         counters[C_N_BINS] = c->n_bins;
@@ -1931,16 +1943,13 @@ lpm_status lpm_species(lpm_ctx *c, int scenario, int species, double *conc, doub
     const double vol = g.cdx * g.cdy * g.cdz, area = g.cdx * g.cdy;
     lpm_status st = conv_room(c, (c->ncell() + c->ndep()) * sizeof(double));
     if (st != LPM_OK) return st;
-    if (conc && (st = read_fixed(c, dc, c->ncell(), unit, vol, 0, conc, c->ncell(), nullptr)) != LPM_OK)
+    if (conc && (st = convert_fixed(c, dc, c->ncell(), unit, vol, 0)) != LPM_OK) return st;
+    if ((dry || wet) && (st = convert_fixed(c, dd, 2 * plane, unit, area, c->ncell())) != LPM_OK)
         return st;
-    if ((dry || wet) &&
-        (st = read_fixed(c, dd, 2 * plane, unit, area, c->ncell(), dry, plane, wet)) != LPM_OK)
-        return st;
-    if (conc_fixed)
-        LPM_CUDA(c, cudaMemcpyAsync(conc_fixed, dc, c->ncell() * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (dep_fixed)
-        LPM_CUDA(c, cudaMemcpyAsync(dep_fixed, dd, c->ndep() * 8, cudaMemcpyDeviceToHost, c->stream));
-    return check_device_error(c);
+    const char *conv_dep = c->d_conv + c->ncell() * 8;
+    return read_back(c, {{conc, c->d_conv, c->ncell() * 8}, {dry, conv_dep, plane * 8},
+                         {wet, conv_dep + plane * 8, plane * 8}, {conc_fixed, dc, c->ncell() * 8},
+                         {dep_fixed, dd, c->ndep() * 8}});
 }
 
 lpm_status lpm_set_kz_model(lpm_ctx *c, int model, double kz_min)
@@ -2036,17 +2045,16 @@ lpm_status lpm_dosage(lpm_ctx *c, int scenario, double *out, size_t n_out, uint6
         return fail(c, LPM_E_INVALID, "n_out must be cz*cy*cx = %zu", c->ncell());
     lpm_status st = LPM_OK;
     const unsigned long long *src = c->d_dose + (size_t)scenario * c->ncell();
-    if (fixed)
-        LPM_CUDA(c, cudaMemcpyAsync(fixed, src, n_out * sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                                    c->stream));
     if (out) {
         const lpm_config &g = c->cfg;
         const double f = std::ldexp(1.0, c->dose_bits - c->scen[(size_t)scenario].shift) *
                          ((double)c->dose_every * g.dt) / (g.cdx * g.cdy * g.cdz);
         if ((st = conv_room(c, n_out * sizeof(double))) != LPM_OK) return st;
-        if ((st = read_fixed(c, src, n_out, f, 1.0, 0, out, n_out, nullptr)) != LPM_OK) return st;
+        if ((st = convert_fixed(c, src, n_out, f, 1.0, 0)) != LPM_OK) return st;
     }
-    if ((st = check_device_error(c)) != LPM_OK) return st;
+    st = read_back(c, {{out, c->d_conv, n_out * sizeof(double)},
+                       {fixed, src, n_out * sizeof(uint64_t)}});
+    if (st != LPM_OK) return st;
     if (n_samples) *n_samples = c->n_dose;
     return LPM_OK;
 }
