@@ -9,6 +9,8 @@
 #include <cstring>
 #include <initializer_list>
 #include <limits>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 #include <algorithm>
@@ -1613,7 +1615,8 @@ lpm_status lpm_sync(lpm_ctx *c)
 }
 
 namespace {
-// Room for `bytes` of converted read-back data.
+// Room for `bytes` of converted read-back data, if the device has it: else d_conv_cap is less,
+// and the caller converts on the host.
 lpm_status conv_room(lpm_ctx *c, size_t bytes)
 {
     if (bytes <= c->d_conv_cap) return LPM_OK;
@@ -1621,19 +1624,14 @@ lpm_status conv_room(lpm_ctx *c, size_t bytes)
     if (c->d_conv) cudaFree(c->d_conv);
     c->d_conv = nullptr;
     c->d_conv_cap = 0;
-    LPM_CUDA(c, cudaMalloc(&c->d_conv, bytes));
+    const cudaError_t e = cudaMalloc(&c->d_conv, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        c->d_conv = nullptr;
+        return LPM_OK;
+    }
+    LPM_CUDA(c, e);
     c->d_conv_cap = bytes;
-    return LPM_OK;
-}
-
-// Enqueues the conversion of n 64-bit fixed-point sums to doubles (x f, / d) at element `at`
-// of the scratch.
-lpm_status convert_fixed(lpm_ctx *c, const unsigned long long *src, size_t n, double f, double d,
-                         size_t at)
-{
-    LPM_CUDA(c, launch_fixed_to_double(c->stream, src, reinterpret_cast<double *>(c->d_conv) + at,
-                                       (long long)n, f, d));
-    c->n_launches++;
     return LPM_OK;
 }
 
@@ -1645,21 +1643,70 @@ struct CopyOut {
     size_t bytes;
 };
 
-lpm_status read_back(lpm_ctx *c, std::initializer_list<CopyOut> copies, bool check = true)
+lpm_status copy_out(lpm_ctx *c, const CopyOut *copies, size_t n)
 {
-    if (check) {
-        const lpm_status st = check_device_error(c);
-        if (st != LPM_OK) return st;
-    }
     cudaError_t e = cudaSuccess;
-    for (const CopyOut &k : copies)
-        if (k.dst && e == cudaSuccess)
-            e = cudaMemcpyAsync(k.dst, k.src, k.bytes, cudaMemcpyDeviceToHost, c->stream);
+    for (size_t i = 0; i < n; ++i)
+        if (copies[i].dst && e == cudaSuccess)
+            e = cudaMemcpyAsync(copies[i].dst, copies[i].src, copies[i].bytes,
+                                cudaMemcpyDeviceToHost, c->stream);
     const cudaError_t done = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) e = done;
     if (e == cudaSuccess) return LPM_OK;
     (void)cudaGetLastError();
     return fail(c, LPM_E_CUDA, "copying a read-back failed: %s", cudaGetErrorString(e));
+}
+
+// n 64-bit fixed-point sums as doubles, x f, / d.
+struct FixedOut {
+    double *dst;
+    const unsigned long long *src;
+    size_t n;
+    double f, d;
+};
+
+// The read-back of at most 4 fixed-point arrays as doubles and of others as they are. The
+// device converts them (neighbours with one launch); without room for that the host does, in
+// the caller's arrays and with the same arithmetic.
+lpm_status read_back(lpm_ctx *c, std::initializer_list<FixedOut> fixed,
+                     std::initializer_list<CopyOut> plain)
+{
+    size_t need = 0;
+    for (const FixedOut &x : fixed) need += x.dst ? x.n * sizeof(double) : 0;
+    lpm_status st = conv_room(c, need);
+    if (st != LPM_OK) return st;
+    const bool room = need <= c->d_conv_cap;
+    CopyOut copies[8];
+    size_t n = 0, at = 0;
+    for (const FixedOut *x = fixed.begin(); x != fixed.end(); ++x) {
+        if (!x->dst) continue;
+        copies[n++] = {x->dst, room ? (const void *)(c->d_conv + at) : x->src, x->n * sizeof(double)};
+        if (!room) continue;
+        const FixedOut *y = x + 1;
+        size_t m = x->n;
+        if (y != fixed.end() && y->dst && y->src == x->src + x->n && y->f == x->f && y->d == x->d) {
+            copies[n++] = {y->dst, c->d_conv + at + m * sizeof(double), y->n * sizeof(double)};
+            m += y->n;
+        } else {
+            y = x;
+        }
+        LPM_CUDA(c, launch_fixed_to_double(c->stream, x->src, reinterpret_cast<double *>(c->d_conv + at),
+                                           (long long)m, x->f, x->d));
+        c->n_launches++;
+        at += m * sizeof(double);
+        x = y;
+    }
+    for (const CopyOut &x : plain) copies[n++] = x;
+    if ((st = check_device_error(c)) != LPM_OK) return st;
+    if ((st = copy_out(c, copies, n)) != LPM_OK || room) return st;
+    for (const FixedOut &x : fixed)
+        for (size_t i = 0; x.dst && i < x.n; ++i) {
+            unsigned long long v;
+            std::memcpy(&v, x.dst + i, sizeof v);
+            const double w = (double)v * x.f;
+            x.dst[i] = x.d == 1.0 ? w : w / x.d;
+        }
+    return LPM_OK;
 }
 }  // namespace
 
@@ -1671,10 +1718,7 @@ lpm_status lpm_concentration(lpm_ctx *c, int scenario, double *out, size_t n_out
         return fail(c, LPM_E_INVALID, "out must hold cz*cy*cx = %zu doubles", c->ncell());
     const lpm_config &g = c->cfg;
     const double f = std::ldexp(1.0, -c->scen[(size_t)scenario].shift) / (g.cdx * g.cdy * g.cdz);
-    lpm_status st = conv_room(c, n_out * sizeof(double));
-    if (st != LPM_OK) return st;
-    st = convert_fixed(c, c->d_conc + (size_t)scenario * n_out, n_out, f, 1.0, 0);
-    return st != LPM_OK ? st : read_back(c, {{out, c->d_conv, n_out * sizeof(double)}});
+    return read_back(c, {{out, c->d_conc + (size_t)scenario * n_out, n_out, f, 1.0}}, {});
 }
 
 lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, size_t n_out)
@@ -1684,14 +1728,8 @@ lpm_status lpm_deposition(lpm_ctx *c, int scenario, double *dry, double *wet, si
     const size_t plane = (size_t)c->cfg.cx * c->cfg.cy;
     if (n_out != plane) return fail(c, LPM_E_INVALID, "n_out must be cy*cx = %zu", plane);
     const double f = std::ldexp(1.0, -c->scen[(size_t)scenario].shift) / (c->cfg.cdx * c->cfg.cdy);
-    lpm_status st = conv_room(c, 2 * plane * sizeof(double));
-    if (st != LPM_OK) return st;
-    if (dry || wet) {
-        st = convert_fixed(c, c->d_dep + (size_t)scenario * c->ndep(), 2 * plane, f, 1.0, 0);
-        if (st != LPM_OK) return st;
-    }
-    const size_t bytes = plane * sizeof(double);
-    return read_back(c, {{dry, c->d_conv, bytes}, {wet, c->d_conv + bytes, bytes}});
+    const unsigned long long *src = c->d_dep + (size_t)scenario * c->ndep();
+    return read_back(c, {{dry, src, plane, f, 1.0}, {wet, src + plane, plane, f, 1.0}}, {});
 }
 
 lpm_status lpm_budget(lpm_ctx *c, int scenario, double out[8])
@@ -1751,24 +1789,48 @@ lpm_status lpm_particles(lpm_ctx *c, int64_t first, int64_t count, float *xyz, u
                     (long long)first, (long long)(first + count), c->n_slots_used);
     lpm_status st = LPM_OK;
     const bool sorted = c->d_sorted[0] != nullptr;
+    if (!xyz && !tag) return check_device_error(c);
     if (sorted && count > 0 && (st = ensure_slot_map(c)) != LPM_OK) return st;
     // slot order, from the home slots, the sorted set and the dead array, as the caller's two
-    // arrays, a bounded piece at a time
-    const int64_t most = (int64_t)1 << 22;
-    if ((st = conv_room(c, (size_t)std::min(count, most) * 4 * sizeof(float))) != LPM_OK) return st;
-    for (int64_t at = 0; at < count && (xyz || tag); at += most) {
-        const int64_t n = std::min(most, count - at);
-        float *d_xyz = reinterpret_cast<float *>(c->d_conv);
-        unsigned int *d_tag = reinterpret_cast<unsigned int *>(d_xyz + 3 * n);
-        LPM_CUDA(c, launch_gather_xyz(c->stream, c->d_state, sorted ? c->d_sorted[c->cur] : nullptr,
-                                      sorted ? c->d_slot_of : nullptr, c->d_grave, first + at, n,
-                                      xyz ? d_xyz : nullptr, tag ? d_tag : nullptr));
-        c->n_launches++;
-        st = read_back(c, {{xyz ? xyz + 3 * at : nullptr, d_xyz, (size_t)n * 3 * sizeof(float)},
-                           {tag ? tag + at : nullptr, d_tag, (size_t)n * sizeof(uint32_t)}}, at == 0);
-        if (st != LPM_OK) return st;
+    // arrays, a bounded piece at a time: in the spare sorted buffer (free until the next sort),
+    // else in the conversion scratch
+    int64_t most = (int64_t)1 << 22;
+    char *room = reinterpret_cast<char *>(c->d_sorted[1 - c->cur]);
+    if (!room) {
+        if ((st = conv_room(c, (size_t)std::min(count, most) * sizeof(float4))) != LPM_OK) return st;
+        room = c->d_conv;
     }
-    return count == 0 || !(xyz || tag) ? check_device_error(c) : LPM_OK;
+    if (room || count == 0) {
+        for (int64_t at = 0; at < count; at += most) {
+            const int64_t n = std::min(most, count - at);
+            float *d_xyz = reinterpret_cast<float *>(room);
+            unsigned int *d_tag = reinterpret_cast<unsigned int *>(d_xyz + 3 * n);
+            LPM_CUDA(c, launch_gather_xyz(c->stream, c->d_state, sorted ? c->d_sorted[c->cur] : nullptr,
+                                          sorted ? c->d_slot_of : nullptr, c->d_grave, first + at, n,
+                                          xyz ? d_xyz : nullptr, tag ? d_tag : nullptr));
+            c->n_launches++;
+            if (at == 0 && (st = check_device_error(c)) != LPM_OK) return st;
+            const CopyOut out[2] = {{xyz ? xyz + 3 * at : nullptr, d_xyz, (size_t)n * 3 * sizeof(float)},
+                                    {tag ? tag + at : nullptr, d_tag, (size_t)n * sizeof(uint32_t)}};
+            if ((st = copy_out(c, out, 2)) != LPM_OK) return st;
+        }
+        return count == 0 ? check_device_error(c) : LPM_OK;
+    }
+    // no room on the device (so nothing is sorted): the states as they are, parted on the host
+    if ((st = check_device_error(c)) != LPM_OK) return st;
+    most = 1 << 16;
+    std::unique_ptr<float4[]> h(new (std::nothrow) float4[(size_t)std::min(count, most)]);
+    if (!h) return fail(c, LPM_E_OOM, "host allocation failed");
+    for (int64_t at = 0; at < count; at += most) {
+        const int64_t n = std::min(most, count - at);
+        const CopyOut out{h.get(), c->d_state + first + at, (size_t)n * sizeof(float4)};
+        if ((st = copy_out(c, &out, 1)) != LPM_OK) return st;
+        for (int64_t i = 0; i < n; ++i) {
+            if (xyz) std::memcpy(xyz + 3 * (at + i), &h[i], 3 * sizeof(float));
+            if (tag) std::memcpy(tag + at + i, &h[i].w, sizeof(uint32_t));
+        }
+    }
+    return LPM_OK;
 }
 
 lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_conc, uint64_t *dep,
@@ -1780,8 +1842,8 @@ lpm_status lpm_fixed_state(lpm_ctx *c, int scenario, uint64_t *conc, size_t n_co
     if (dep && n_dep != c->ndep()) return fail(c, LPM_E_INVALID, "n_dep must be %zu", c->ndep());
     lpm_status st = LPM_OK;
     if (counters && (st = read_counters(c, scenario)) != LPM_OK) return st;
-    st = read_back(c, {{conc, c->d_conc + (size_t)scenario * c->ncell(), n_conc * sizeof(uint64_t)},
-                       {dep, c->d_dep + (size_t)scenario * c->ndep(), n_dep * sizeof(uint64_t)}});
+    st = read_back(c, {}, {{conc, c->d_conc + (size_t)scenario * c->ncell(), n_conc * sizeof(uint64_t)},
+                           {dep, c->d_dep + (size_t)scenario * c->ndep(), n_dep * sizeof(uint64_t)}});
     if (st != LPM_OK) return st;
     if (counters) {
         for (int i = 0; i < 16; ++i) counters[i] = (int64_t)c->h_words[1 + i];
@@ -1941,15 +2003,9 @@ lpm_status lpm_species(lpm_ctx *c, int scenario, int species, double *conc, doub
     const lpm_config &g = c->cfg;
     const double unit = std::ldexp(1.0, -c->scen[(size_t)scenario].shift);
     const double vol = g.cdx * g.cdy * g.cdz, area = g.cdx * g.cdy;
-    lpm_status st = conv_room(c, (c->ncell() + c->ndep()) * sizeof(double));
-    if (st != LPM_OK) return st;
-    if (conc && (st = convert_fixed(c, dc, c->ncell(), unit, vol, 0)) != LPM_OK) return st;
-    if ((dry || wet) && (st = convert_fixed(c, dd, 2 * plane, unit, area, c->ncell())) != LPM_OK)
-        return st;
-    const char *conv_dep = c->d_conv + c->ncell() * 8;
-    return read_back(c, {{conc, c->d_conv, c->ncell() * 8}, {dry, conv_dep, plane * 8},
-                         {wet, conv_dep + plane * 8, plane * 8}, {conc_fixed, dc, c->ncell() * 8},
-                         {dep_fixed, dd, c->ndep() * 8}});
+    return read_back(c, {{conc, dc, c->ncell(), unit, vol}, {dry, dd, plane, unit, area},
+                         {wet, dd + plane, plane, unit, area}},
+                     {{conc_fixed, dc, c->ncell() * 8}, {dep_fixed, dd, c->ndep() * 8}});
 }
 
 lpm_status lpm_set_kz_model(lpm_ctx *c, int model, double kz_min)
@@ -2043,17 +2099,12 @@ lpm_status lpm_dosage(lpm_ctx *c, int scenario, double *out, size_t n_out, uint6
     if (!c->d_dose) return fail(c, LPM_E_STATE, "dosage was never enabled (lpm_set_dosage)");
     if ((out || fixed) && n_out != c->ncell())
         return fail(c, LPM_E_INVALID, "n_out must be cz*cy*cx = %zu", c->ncell());
-    lpm_status st = LPM_OK;
     const unsigned long long *src = c->d_dose + (size_t)scenario * c->ncell();
-    if (out) {
-        const lpm_config &g = c->cfg;
-        const double f = std::ldexp(1.0, c->dose_bits - c->scen[(size_t)scenario].shift) *
-                         ((double)c->dose_every * g.dt) / (g.cdx * g.cdy * g.cdz);
-        if ((st = conv_room(c, n_out * sizeof(double))) != LPM_OK) return st;
-        if ((st = convert_fixed(c, src, n_out, f, 1.0, 0)) != LPM_OK) return st;
-    }
-    st = read_back(c, {{out, c->d_conv, n_out * sizeof(double)},
-                       {fixed, src, n_out * sizeof(uint64_t)}});
+    const lpm_config &g = c->cfg;
+    const double f = std::ldexp(1.0, c->dose_bits - c->scen[(size_t)scenario].shift) *
+                     ((double)c->dose_every * g.dt) / (g.cdx * g.cdy * g.cdz);
+    const lpm_status st = read_back(c, {{out, src, n_out, f, 1.0}},
+                                    {{fixed, src, n_out * sizeof(uint64_t)}});
     if (st != LPM_OK) return st;
     if (n_samples) *n_samples = c->n_dose;
     return LPM_OK;

@@ -88,3 +88,34 @@ def test_single_outputs(sort_every):
                         assert np.array_equal(x, w), (name, keep)
                     else:
                         assert (x.view(np.uint8) == 0xA5).all(), (name, keep)
+
+
+def test_without_room_on_the_device():
+    """On a full device the read-backs convert on the host and give the same bits."""
+    import torch
+    from paper_0912_3223_gb300 import Sim
+    cfg = dataclasses.replace(_config(release=li.Release(5_000_000, np.array([1.0]), 3600.0, 0, 2)),
+                              cx=400, cy=400, cz=60, cdx=125.0, cdy=125.0, cdz=50.0, n_steps=4,
+                              bin_every=2, langevin=0)
+    need = 4 * min(cfg.n_particles, 1 << 22) * 4          # the smaller of the two scratches
+
+    def outputs(sim):
+        return [*sim.particles(), sim.concentration(), *sim.deposition(), *sim.species(1),
+                *sim.dosage()[:2]]
+
+    sims = [Sim(cfg, sort_every=0).set_dosage(2).step(4) for _ in range(2)]
+    want = outputs(sims[0])                               # (loads the kernels, too)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (32 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        assert torch.cuda.mem_get_info()[0] < need
+        got = outputs(sims[1])
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+        for sim in sims:
+            sim.close()
+    assert want[2].max() > 0 and want[8].max() > 0
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
