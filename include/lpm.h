@@ -285,6 +285,10 @@ lpm_status lpm_set_launch(lpm_ctx *ctx, int block, int particles_per_thread, int
  * (one pass over the slots). */
 lpm_status lpm_set_sort(lpm_ctx *ctx, int every_steps);
 
+/* Takes back lpm_set_launch (launch != 0) and lpm_set_sort (sort != 0): the library picks the
+ * launch shapes and the sort interval by size again, as in a context without these calls. */
+lpm_status lpm_set_auto(lpm_ctx *ctx, int launch, int sort);
+
 /*
  * Vertical Langevin (velocity-memory) variant of the random walk of Eq. 2 (no paper
  * counterpart: the paper moves particles by Eq. 1-2 only). Each particle carries a

@@ -1,11 +1,11 @@
 """Launch-shape and sort-interval autotuner for the particle kernels.
 
 Times complete runs (lpm_reset + lpm_step over the whole horizon, so the release ramp,
-the exits and the end-of-run binning are all represented) for every supported
-(threads per block, particles per thread, occupancy variant), and with
-``autotune_with_sort`` also for several intervals of the re-ordering of the particles by
-weather cell (the steps fused between two sorts), with CUDA events on the context stream,
-and keeps the fastest. Results are cached per (GPU name, workload signature) in a JSON file
+the exits and the end-of-run binning are all represented) for the library's own choice by
+size and for every (threads per block, occupancy variant), and with ``autotune_with_sort``
+also for several intervals of the re-ordering of the particles by weather cell (the steps
+fused between two sorts), with CUDA events on the context stream, and keeps the fastest.
+The library's choice is written ``None``, as in ``Sim``'s arguments. Results are cached per (GPU name, workload signature) in a JSON file
 (``$LPM_AUTOTUNE_CACHE`` or ``~/.cache/lpm_gb300/autotune.json``). Every shape and sort
 interval gives bit-identical results, so tuning never changes what is computed.
 """
@@ -19,10 +19,11 @@ from typing import Dict, Iterable, Optional, Tuple
 from . import lpm
 
 BLOCKS = (128, 256, 512)
-PPTS = (1, 2, 4)
 OCCS = (0, 1, 2)
-# shapes tried by default: every (block, particles per thread, occupancy variant)
-DEFAULT_SHAPES = [(b, p, o) for b in BLOCKS for p in PPTS for o in OCCS]
+# shapes tried by default: the choice by size, which has shapes of its own (warps in pairs,
+# several in one run), and every (block, tile factor 1, occupancy variant); the factor
+# reaches no kernel
+DEFAULT_SHAPES = [None] + [(b, 1, o) for b in BLOCKS for o in OCCS]
 
 
 def cache_path() -> str:
@@ -62,10 +63,31 @@ def _store(d: Dict) -> None:
         pass
 
 
-def time_shape(sim, shape, reps: int = 2) -> float:
+Shape = Optional[Tuple[int, int, int]]
+
+
+def _set_launch(sim, shape: Shape) -> None:
+    if shape is None:
+        lpm.lpm_set_auto(sim.ctx, launch=True, sort=False)
+    else:
+        lpm.lpm_set_launch(sim.ctx, *shape)
+
+
+def _set_sort(sim, every: Optional[int]) -> None:
+    if every is None:
+        lpm.lpm_set_auto(sim.ctx, launch=False, sort=True)
+    else:
+        lpm.lpm_set_sort(sim.ctx, every)
+
+
+def _label(shape: Shape) -> str:
+    return "auto" if shape is None else "x".join(map(str, shape))
+
+
+def time_shape(sim, shape: Shape, reps: int = 2) -> float:
     """Milliseconds of one complete run with the given launch shape (best of ``reps``)."""
     import torch
-    lpm.lpm_set_launch(sim.ctx, *shape)
+    _set_launch(sim, shape)
     stream = sim.stream
     best = float("inf")
     for _ in range(reps + 1):                # the first run builds graphs and warms up
@@ -80,78 +102,86 @@ def time_shape(sim, shape, reps: int = 2) -> float:
     return best
 
 
-def autotune(sim, shapes: Optional[Iterable[Tuple[int, int, int]]] = None, use_cache: bool = True,
-             reps: int = 2) -> Tuple[int, int, int]:
-    """Picks and applies the fastest launch shape for ``sim`` (a ``Sim``); returns it."""
-    import torch
-    key = f"{torch.cuda.get_device_name()}|{signature(sim.cfg)}"
-    cache = _load() if use_cache else {}
-    if key in cache:
-        shape = tuple(cache[key]["shape"])
-        lpm.lpm_set_launch(sim.ctx, *shape)
-        return shape
-    shapes = [tuple(v) for v in shapes] if shapes is not None else DEFAULT_SHAPES
-    results = {}
-    for shape in shapes:
+def _fastest(sim, candidates, reps: int):
+    """Times (label, shape, interval) candidates in turn (interval "keep": the context's);
+    returns the fastest and the milliseconds of each."""
+    results, chosen = {}, {}
+    for label, shape, every in candidates:
+        if every != "keep":
+            _set_sort(sim, every)
         try:
-            results["x".join(map(str, shape))] = time_shape(sim, shape, reps)
+            results[label] = time_shape(sim, shape, reps)
+            chosen[label] = shape, every
         except lpm.LpmError as e:
-            # shapes the context's options do not run with (e.g. dosage, Eq. 3 K_z or a
-            # decay chain need one particle per thread)
+            # shapes the context's options do not run with (dosage, Eq. 3 K_z, a decay chain,
+            # the Langevin variant and perturbation modes need a tile factor of 1)
             if e.status != lpm.LPM_E_INVALID:
                 raise
     if not results:
         raise RuntimeError("no launch shape runs with this context's options")
-    best = min(results, key=results.get)
-    shape = tuple(int(v) for v in best.split("x"))
-    lpm.lpm_set_launch(sim.ctx, *shape)
+    return chosen[min(results, key=results.get)], results
+
+
+def _shape(v) -> Shape:
+    return None if v is None else tuple(int(x) for x in v)
+
+
+# (the key names the candidates' generation: answers kept from before the choice by size was
+# one of them are not served)
+def _key(sim) -> str:
+    import torch
+    return f"{torch.cuda.get_device_name()}|{signature(sim.cfg)}|auto"
+
+
+def autotune(sim, shapes: Optional[Iterable[Shape]] = None, use_cache: bool = True,
+             reps: int = 2) -> Shape:
+    """Picks and applies the fastest launch shape for ``sim`` (a ``Sim``); returns it (None:
+    the library's choice by size)."""
+    key = _key(sim)
+    cache = _load() if use_cache else {}
+    if key in cache:
+        shape = _shape(cache[key]["shape"])
+        _set_launch(sim, shape)
+        return shape
+    shapes = [_shape(v) for v in shapes] if shapes is not None else DEFAULT_SHAPES
+    (shape, _), results = _fastest(sim, [(_label(v), v, "keep") for v in shapes], reps)
+    _set_launch(sim, shape)
     sim.reset()
     if use_cache:
         cache = _load()
-        cache[key] = {"shape": list(shape), "ms": results}
+        cache[key] = {"shape": shape, "ms": results}
         _store(cache)
     return shape
 
 
-SORT_INTERVALS = (30, 60, 90)
+# intervals tried by default: the choice by size, and none (0), 30, 60, 90 and 120 steps
+SORT_INTERVALS = (None, 0, 30, 60, 90, 120)
 
 
-def autotune_with_sort(sim, shapes: Optional[Iterable[Tuple[int, int, int]]] = None,
-                       sort_intervals: Iterable[int] = SORT_INTERVALS, use_cache: bool = True,
-                       reps: int = 2) -> Tuple[Tuple[int, int, int], int, Dict[str, float]]:
+def autotune_with_sort(sim, shapes: Optional[Iterable[Shape]] = None,
+                       sort_intervals: Iterable[Optional[int]] = SORT_INTERVALS,
+                       use_cache: bool = True,
+                       reps: int = 2) -> Tuple[Shape, Optional[int], Dict[str, float]]:
     """Picks and applies the fastest (launch shape, sort interval) for ``sim``; returns the
-    shape, the interval and the measured milliseconds of every combination tried."""
-    import torch
-    intervals = [int(e) for e in sort_intervals]
-    key = f"{torch.cuda.get_device_name()}|{signature(sim.cfg)}|sort{intervals}"
+    shape, the interval (None: the library's choice by size) and the measured milliseconds of
+    every combination tried."""
+    intervals = [None if e is None else int(e) for e in sort_intervals]
+    key = f"{_key(sim)}|sort{intervals}"
     cache = _load() if use_cache else {}
     if key in cache:
-        shape = tuple(cache[key]["shape"])
-        every = int(cache[key]["sort_every"])
-        lpm.lpm_set_launch(sim.ctx, *shape)
-        lpm.lpm_set_sort(sim.ctx, every)
+        shape, every = _shape(cache[key]["shape"]), cache[key]["sort_every"]
+        _set_launch(sim, shape)
+        _set_sort(sim, every)
         return shape, every, cache[key]["ms"]
-    shapes = [tuple(v) for v in shapes] if shapes is not None else DEFAULT_SHAPES
-    results = {}
-    for every in intervals:
-        lpm.lpm_set_sort(sim.ctx, every)
-        for shape in shapes:
-            try:
-                results["x".join(map(str, shape)) + f"/sort{every}"] = time_shape(sim, shape, reps)
-            except lpm.LpmError as e:
-                if e.status != lpm.LPM_E_INVALID:
-                    raise
-    if not results:
-        raise RuntimeError("no launch shape runs with this context's options")
-    best = min(results, key=results.get)
-    shape_s, every_s = best.split("/sort")
-    shape = tuple(int(v) for v in shape_s.split("x"))
-    every = int(every_s)
-    lpm.lpm_set_launch(sim.ctx, *shape)
-    lpm.lpm_set_sort(sim.ctx, every)
+    shapes = [_shape(v) for v in shapes] if shapes is not None else DEFAULT_SHAPES
+    (shape, every), results = _fastest(
+        sim, [(f"{_label(v)}/sort{'auto' if e is None else e}", v, e)
+              for e in intervals for v in shapes], reps)
+    _set_launch(sim, shape)
+    _set_sort(sim, every)
     sim.reset()
     if use_cache:
         cache = _load()
-        cache[key] = {"shape": list(shape), "sort_every": every, "ms": results}
+        cache[key] = {"shape": shape, "sort_every": every, "ms": results}
         _store(cache)
     return shape, every, results

@@ -1880,6 +1880,27 @@ lpm_status lpm_set_sort(lpm_ctx *c, int every_steps)
     return LPM_OK;
 }
 
+lpm_status lpm_set_auto(lpm_ctx *c, int launch, int sort)
+{
+    if (!c) return LPM_E_INVALID;
+    if (sort && c->sort_every >= 0) {
+        const lpm_status st = clear_sort_state(c, true);     // as in lpm_set_sort
+        if (st != LPM_OK) return st;
+        c->sort_every = -1;
+        c->tiles_valid = false;
+        drop_graphs(c);
+    }
+    if (launch && c->launch_set) {
+        c->launch_set = false;
+        c->block = 512;
+        c->ppt = 1;
+        c->occ = 2;
+        c->tiles_valid = false;
+        drop_graphs(c);
+    }
+    return LPM_OK;
+}
+
 lpm_status lpm_set_langevin(lpm_ctx *c, int on, double t_lagr)
 {
     if (!c) return LPM_E_INVALID;

@@ -39,7 +39,7 @@ SYMBOLS = ["lpm_create", "lpm_destroy", "lpm_last_error", "lpm_set_met", "lpm_se
            "lpm_load", "lpm_set_dosage", "lpm_dosage", "lpm_set_kz_model",
            "lpm_set_boundary_layer", "lpm_set_decay_chain", "lpm_species", "lpm_set_langevin",
            "lpm_particle_velocity", "lpm_set_adjoint_storage", "lpm_adjoint_storage",
-           "lpm_set_modes", "lpm_set_mode_phases", "lpm_device_state"]
+           "lpm_set_modes", "lpm_set_mode_phases", "lpm_device_state", "lpm_set_auto"]
 
 
 class LpmError(RuntimeError):
@@ -110,6 +110,7 @@ def load() -> C.CDLL:
     L.lpm_stats.argtypes = [vp, C.POINTER(i64), C.POINTER(i64), dp]
     L.lpm_set_params.argtypes = [vp, C.c_double, C.c_double, C.c_double]
     L.lpm_set_sort.argtypes = [vp, C.c_int]
+    L.lpm_set_auto.argtypes = [vp, C.c_int, C.c_int]
     L.lpm_set_dosage.argtypes = [vp, C.c_int]
     L.lpm_set_kz_model.argtypes = [vp, C.c_int, C.c_double]
     L.lpm_set_decay_chain.argtypes = [vp, C.c_int, dp]
@@ -139,8 +140,8 @@ def load() -> C.CDLL:
                  "lpm_particles", "lpm_fixed_state", "lpm_set_launch", "lpm_sync",
                  "lpm_draws", "lpm_release_range", "lpm_reset", "lpm_set_profiling",
                  "lpm_stats", "lpm_set_params", "lpm_set_emission", "lpm_receptors",
-                 "lpm_adjoint", "lpm_draws_static", "lpm_set_sort", "lpm_save", "lpm_load",
-                 "lpm_set_dosage", "lpm_dosage", "lpm_set_kz_model", "lpm_set_boundary_layer",
+                 "lpm_adjoint", "lpm_draws_static", "lpm_set_sort", "lpm_set_auto", "lpm_save",
+                 "lpm_load", "lpm_set_dosage", "lpm_dosage", "lpm_set_kz_model", "lpm_set_boundary_layer",
                  "lpm_set_decay_chain", "lpm_species", "lpm_set_langevin",
                  "lpm_particle_velocity", "lpm_set_adjoint_storage", "lpm_adjoint_storage",
                  "lpm_set_modes", "lpm_set_mode_phases", "lpm_device_state"):
@@ -302,6 +303,11 @@ def lpm_load(ctx, state: bytes) -> None:
 
 def lpm_set_sort(ctx, every_steps: int) -> None:
     _check(ctx, load().lpm_set_sort(C.c_void_p(ctx), int(every_steps)))
+
+
+def lpm_set_auto(ctx, launch: bool = True, sort: bool = True) -> None:
+    """Takes back ``lpm_set_launch`` and ``lpm_set_sort``: shapes and interval by size."""
+    _check(ctx, load().lpm_set_auto(C.c_void_p(ctx), int(bool(launch)), int(bool(sort))))
 
 
 def lpm_set_params(ctx, k_scale: float = 1.0, bias_u: float = 0.0, bias_v: float = 0.0) -> None:
