@@ -153,7 +153,7 @@ lpm_status lpm_set_source(lpm_ctx *ctx, int scenario, double x, double y, double
  * eu, ev); the field is non-divergent when (eu, ev) is perpendicular to (fx, fy).
  * profile: host [nz] scale at the levels. 0 <= n_modes <= LPM_MAX_MODES (0 turns the
  * modes off); every scenario starts with zero amplitudes. Copied; applies to the next
- * lpm_step. Runs in the extended step kernel (1 particle per thread); lpm_adjoint and
+ * lpm_step (which then takes a tile factor of 1 only, see lpm_set_launch); lpm_adjoint and
  * lpm_receptors reject a context with modes (LPM_E_INVALID). Like the met and the
  * source, the modes are inputs, not part of lpm_save's state.
  * Errors: LPM_E_INVALID for n_modes out of range, NULL or non-finite arrays.
@@ -264,9 +264,12 @@ lpm_status lpm_device_state(lpm_ctx *ctx, int scenario, const uint64_t **conc,
                             const uint64_t **dep, const uint64_t **counters,
                             int64_t *counter_stride);
 
-/* Launch shape of the particle kernels: threads per block (128, 256 or 512), particles
- * per thread (1, 2 or 4) and occupancy variant (0, 1, 2: at most 128, 80 or 64 registers
- * per thread, i.e. 16, 24 or 32 resident warps per SM). Without this call the library picks
+/* Launch shape of the particle kernels: threads per block (128, 256 or 512), tile factor (1, 2
+ * or 4) and occupancy variant (0, 1, 2: at most 128, 80 or 64 registers per thread, i.e. 16,
+ * 24 or 32 resident warps per SM). Every thread moves one particle at a time; particles not
+ * yet sorted are listed in runs of block x particles_per_thread. With dosage, Eq. 3, a decay
+ * chain, the Langevin variant or perturbation modes lpm_step takes a tile factor of 1 only
+ * (else LPM_E_INVALID). Without this call the library picks
  * a shape for every launch by its number of particles and its options. Results do not
  * depend on it. The paper tuned its launch (32 blocks of 256 threads) with the
  * occupancy calculator (Sec. 3.2); here the autotuner picks among these shapes. */
@@ -301,8 +304,8 @@ lpm_status lpm_set_auto(lpm_ctx *ctx, int launch, int sort);
  * dt >> T_L the model reduces to the random walk with the same K_z.
  *
  * lpm_set_langevin: on (0/1) and T_L (s, > 0); before the first step or after lpm_reset
- * (LPM_E_STATE otherwise). Allocates 12 bytes per particle slot. Runs with one particle
- * per thread; not supported by lpm_adjoint (LPM_E_INVALID).
+ * (LPM_E_STATE otherwise). Allocates 12 bytes per particle slot. Takes a tile
+ * factor of 1 (lpm_set_launch); not supported by lpm_adjoint (LPM_E_INVALID).
  * lpm_particle_velocity: w' (m/s) of slots [first, first+count) to host (0 for deposited or
  * exited particles). Synchronises.
  */
@@ -344,8 +347,8 @@ lpm_status lpm_species(lpm_ctx *ctx, int scenario, int species, double *conc, do
  * weather records is then ignored.
  *
  * lpm_set_kz_model: model 0 = the gridded K_z of lpm_set_met (default), 1 = Eq. 3
- * (allocates the column buffers: 48 bytes per column and hour). Model 1 runs with one
- * particle per thread and is not supported by lpm_adjoint (LPM_E_INVALID).
+ * (allocates the column buffers: 48 bytes per column and hour). Model 1 takes a
+ * tile factor of 1 (lpm_set_launch) and is not supported by lpm_adjoint (LPM_E_INVALID).
  * lpm_set_boundary_layer: hour t_index of the columns, bl [ny][nx][4] float =
  * (u* (m/s) >= 0, 1/L (1/m), H_z (m) > 0, unused), host memory (validated, copied before
  * return) or device memory (on_device != 0, read on the context stream, not validated).

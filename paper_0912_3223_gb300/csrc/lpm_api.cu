@@ -115,7 +115,7 @@ struct lpm_ctx {
     long long k = 0;                        // steps taken
     long long n_bins = 0;                   // snapshots taken
     bool launch_set = false;                // lpm_set_launch was called; else by size
-    int block = 512, ppt = 1, occ = 2;
+    int block = 512, ppt = 1, occ = 2;      // (ppt: the tile factor)
 
     // sorting by weather cell (both forms) at the multiples of sort_now: d_state is the
     // home buffer (slot order of the API); the live particles released before sorted_upto
@@ -226,7 +226,7 @@ struct lpm_ctx {
     };
     std::vector<Graph> graphs;
 
-    // tile table: runs of at most block*ppt particles of one scenario, grouped by the sort
+    // tile table: runs of at most tile_particles() of one scenario, grouped by the sort
     // interval [j*E, (j+1)*E) their particles leave in (one interval when sorting is off),
     // ordered by the release step of their first particle within an interval
     std::vector<Tile> tiles;
@@ -1468,8 +1468,8 @@ lpm_status lpm_step(lpm_ctx *c, int64_t n)
                      c->langevin;
     if ((ext || c->n_modes > 0) && c->ppt != 1)
         return fail(c, LPM_E_INVALID, "dosage, K_z from Eq. 3, decay chains, the Langevin "
-                                      "variant and perturbation modes run with 1 particle per "
-                                      "thread");
+                                      "variant and perturbation modes take a tile factor of 1 "
+                                      "(lpm_set_launch)");
     st = upload_tables(c);
     if (st != LPM_OK) return st;
     if (const int every = sort_interval(c, ext); every != c->sort_now) {

@@ -468,6 +468,7 @@ def lpm_dosage(ctx, scenario: int, shape):
 
 
 def lpm_set_launch(ctx, block: int, particles_per_thread: int, occupancy: int = 1) -> None:
+    """Launch shape; ``particles_per_thread`` is the tile factor (see include/lpm.h)."""
     _check(ctx, load().lpm_set_launch(C.c_void_p(ctx), int(block), int(particles_per_thread),
                                       int(occupancy)))
 
