@@ -520,12 +520,19 @@ lpm_status upload_tables(lpm_ctx *c)
     return LPM_OK;
 }
 
-// Synchronises the context's streams and reports device-side errors: every read-back's wait for
-// the kernels it enqueued, before anything is copied to the caller's arrays (read_back).
-lpm_status check_device_error(lpm_ctx *c)
+ErrOut err_out(const lpm_ctx *c)
 {
-    LPM_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_err, sizeof(unsigned int), cudaMemcpyDeviceToHost,
-                                c->stream));
+    return {c->d_err, reinterpret_cast<unsigned int *>(c->h_words)};
+}
+
+// Synchronises the context's streams and reports device-side errors: every read-back's wait for
+// the kernels it enqueued, before anything is copied to the caller's arrays (read_back). told:
+// one of those kernels, the last that was enqueued, has the error word in err_out.
+lpm_status check_device_error(lpm_ctx *c, bool told = false)
+{
+    if (!told)
+        LPM_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_err, sizeof(unsigned int),
+                                    cudaMemcpyDeviceToHost, c->stream));
     LPM_CUDA(c, cudaStreamSynchronize(c->stream));
     if (c->copy_stream) LPM_CUDA(c, cudaStreamSynchronize(c->copy_stream));
     unsigned int e;
@@ -1691,13 +1698,13 @@ lpm_status read_back(lpm_ctx *c, std::initializer_list<FixedOut> fixed,
             y = x;
         }
         LPM_CUDA(c, launch_fixed_to_double(c->stream, x->src, reinterpret_cast<double *>(c->d_conv + at),
-                                           (long long)m, x->f, x->d));
+                                           (long long)m, x->f, x->d, err_out(c)));
         c->n_launches++;
         at += m * sizeof(double);
         x = y;
     }
     for (const CopyOut &x : plain) copies[n++] = x;
-    if ((st = check_device_error(c)) != LPM_OK) return st;
+    if ((st = check_device_error(c, at > 0)) != LPM_OK) return st;
     if ((st = copy_out(c, copies, n)) != LPM_OK || room) return st;
     for (const FixedOut &x : fixed)
         for (size_t i = 0; x.dst && i < x.n; ++i) {
@@ -1807,9 +1814,10 @@ lpm_status lpm_particles(lpm_ctx *c, int64_t first, int64_t count, float *xyz, u
             unsigned int *d_tag = reinterpret_cast<unsigned int *>(d_xyz + 3 * n);
             LPM_CUDA(c, launch_gather_xyz(c->stream, c->d_state, sorted ? c->d_sorted[c->cur] : nullptr,
                                           sorted ? c->d_slot_of : nullptr, c->d_grave, first + at, n,
-                                          xyz ? d_xyz : nullptr, tag ? d_tag : nullptr));
+                                          xyz ? d_xyz : nullptr, tag ? d_tag : nullptr,
+                                          err_out(c)));
             c->n_launches++;
-            if (at == 0 && (st = check_device_error(c)) != LPM_OK) return st;
+            if (at == 0 && (st = check_device_error(c, true)) != LPM_OK) return st;
             const CopyOut out[2] = {{xyz ? xyz + 3 * at : nullptr, d_xyz, (size_t)n * 3 * sizeof(float)},
                                     {tag ? tag + at : nullptr, d_tag, (size_t)n * sizeof(uint32_t)}};
             if ((st = copy_out(c, out, 2)) != LPM_OK) return st;

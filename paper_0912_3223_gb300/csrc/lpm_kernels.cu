@@ -222,11 +222,14 @@ int advance_occupancy(int block, int occ, bool mixed, int variant, size_t smem)
 }
 
 // Read-back of a 64-bit fixed-point grid as physical values, in the host's arithmetic (the
-// conversion rounds to nearest): out[i] = in[i] * f, or with DIV in[i] * f / d.
+// conversion rounds to nearest): out[i] = in[i] * f, or with DIV in[i] * f / d. The first thread
+// leaves the error word in page-locked host memory (see ErrOut).
 template <bool DIV>
 __global__ void fixed_to_double_kernel(const unsigned long long *__restrict__ in,
-                                       double *__restrict__ out, long long n, double f, double d)
+                                       double *__restrict__ out, long long n, double f, double d,
+                                       ErrOut err)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err.host = *err.device;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const double v = __ull2double_rn(in[i]) * f;
@@ -235,16 +238,16 @@ __global__ void fixed_to_double_kernel(const unsigned long long *__restrict__ in
 }
 
 cudaError_t launch_fixed_to_double(cudaStream_t s, const unsigned long long *in, double *out,
-                                   long long n, double f, double d)
+                                   long long n, double f, double d, ErrOut err)
 {
     if (n <= 0) return cudaSuccess;
     const int block = 256;
     long long blocks = (n + block - 1) / block;
     if (blocks > 152 * 16) blocks = 152 * 16;
     if (d == 1.0)
-        fixed_to_double_kernel<false><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d);
+        fixed_to_double_kernel<false><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d, err);
     else
-        fixed_to_double_kernel<true><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d);
+        fixed_to_double_kernel<true><<<(unsigned)blocks, block, 0, s>>>(in, out, n, f, d, err);
     return cudaGetLastError();
 }
 

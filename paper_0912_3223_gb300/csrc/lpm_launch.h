@@ -17,6 +17,15 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// The device's error word and a page-locked host word: the kernels of a read-back copy the one to
+// the other, so that one wait tells the error before anything goes to the caller's arrays, with
+// no copy of its own (1e4 particles x 360 steps and their read-backs: 370 us with it, 358 without;
+// the copies before the error is known 362).
+struct ErrOut {
+    const unsigned int *device;
+    unsigned int *host;
+};
+
 // Counts of a sort: particles per key, and per tile of SCAN_TILE keys. Zero except between
 // the pass that writes the keys and the sort that uses them up. Both padded to whole tiles.
 constexpr int SCAN_TILE_BITS = 12;
@@ -223,7 +232,7 @@ cudaError_t launch_gather(cudaStream_t s, const float4 *home, const float4 *sort
                           long long count, float4 *out);
 cudaError_t launch_gather_xyz(cudaStream_t s, const float4 *home, const float4 *sorted,
                               const unsigned int *slot_of, const float4 *grave, long long first,
-                              long long count, float *xyz, unsigned int *tag);
+                              long long count, float *xyz, unsigned int *tag, ErrOut err);
 cudaError_t launch_gather_w(cudaStream_t s, const float *home, const float *sorted,
                             const unsigned int *slot_of, long long first, long long count,
                             float *out);
@@ -239,7 +248,7 @@ cudaError_t launch_budget(cudaStream_t s, const StepParams &P, const float4 *hom
                           int k_now);
 
 cudaError_t launch_fixed_to_double(cudaStream_t s, const unsigned long long *in, double *out,
-                                   long long n, double f, double d = 1.0);
+                                   long long n, double f, double d, ErrOut err);
 void set_global_error(const char *msg);
 
 struct AdjParams;

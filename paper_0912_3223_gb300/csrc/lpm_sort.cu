@@ -279,12 +279,15 @@ __global__ void gather_kernel(const float4 *__restrict__ home, const float4 *__r
         out[i] = locate(home, sorted, slot_of, grave, first + i);
 }
 
-// The same as separate positions [count][3] and tags [count] (either may be nullptr).
+// The same as separate positions [count][3] and tags [count] (either may be nullptr); the first
+// thread leaves the error word in page-locked host memory.
 __global__ void gather_xyz_kernel(const float4 *__restrict__ home, const float4 *__restrict__ sorted,
                                   const unsigned int *__restrict__ slot_of,
                                   const float4 *__restrict__ grave, long long first, long long count,
-                                  float *__restrict__ xyz, unsigned int *__restrict__ tag)
+                                  float *__restrict__ xyz, unsigned int *__restrict__ tag,
+                                  ErrOut err)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err.host = *err.device;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
         const float4 s = locate(home, sorted, slot_of, grave, first + i);
@@ -379,11 +382,11 @@ cudaError_t launch_gather(cudaStream_t s, const float4 *home, const float4 *sort
 
 cudaError_t launch_gather_xyz(cudaStream_t s, const float4 *home, const float4 *sorted,
                               const unsigned int *slot_of, const float4 *grave, long long first,
-                              long long count, float *xyz, unsigned int *tag)
+                              long long count, float *xyz, unsigned int *tag, ErrOut err)
 {
     if (count <= 0) return cudaSuccess;
     gather_xyz_kernel<<<grid_for(count, 256), 256, 0, s>>>(home, sorted, slot_of, grave, first,
-                                                           count, xyz, tag);
+                                                           count, xyz, tag, err);
     return cudaGetLastError();
 }
 
