@@ -327,7 +327,7 @@ __device__ __forceinline__ void reverse_step(const StepParams &P, const AdjParam
     J.mu2 = mz + nm[2];
 }
 
-// Sums of a block's particles (FP64) and one atomic per parameter and block: the source
+// Sums of a group's particles (FP64) and one atomic per parameter and group: the source
 // partials are the sum of mu at release.
 __device__ __forceinline__ void reduce_gradient(const AdjParams &A, const Tile &tile, Adjoint J,
                                                 bool valid, int qidx, double *s_g, double *s_gq)
@@ -344,22 +344,24 @@ __device__ __forceinline__ void reduce_gradient(const AdjParams &A, const Tile &
     if (J.gq != 0.f) atomicAdd(&s_gq[qidx], (double)J.gq);
     __syncthreads();
     double *G = A.grad + (long long)tile.scen * A.ng;
-    const int t = threadIdx.x;
-    if (t < 6 && s_g[t] != 0.0) atomicAdd(G + (t < 3 ? t : A.nq + t), s_g[t]);
-    for (int i = t; i < A.nq; i += ADJ_BLOCK)
+    const int lane = threadIdx.x % ADJ_BLOCK;
+    if (lane < 6 && s_g[lane] != 0.0)
+        atomicAdd(G + (lane < 3 ? lane : A.nq + lane), s_g[lane]);
+    for (int i = lane; i < A.nq; i += ADJ_BLOCK)
         if (s_gq[i] != 0.0) atomicAdd(G + 3 + i, s_gq[i]);
 }
 
-// Receptors and the tile's scenario's dL/dC (scaled by 1 / samples) into shared memory.
+// Receptors and the group's scenario's dL/dC (scaled by 1 / samples) into shared memory.
 __device__ __forceinline__ void load_receptors(const AdjParams &A, const Tile &tile, float4 *s_rec,
                                                float *s_w, double *s_g, double *s_gq)
 {
-    for (int r = threadIdx.x; r < A.R; r += ADJ_BLOCK) {
-        s_rec[r] = A.rec[r];
+    const int lane = threadIdx.x % ADJ_BLOCK;
+    for (int r = lane; r < A.R; r += ADJ_BLOCK) {
+        if (threadIdx.x < ADJ_BLOCK) s_rec[r] = A.rec[r];
         s_w[r] = (float)(A.w[(long long)tile.scen * A.R + r] * (double)A.inv_ns);
     }
-    for (int i = threadIdx.x; i < A.nq; i += ADJ_BLOCK) s_gq[i] = 0.0;
-    if (threadIdx.x < 6) s_g[threadIdx.x] = 0.0;
+    for (int i = lane; i < A.nq; i += ADJ_BLOCK) s_gq[i] = 0.0;
+    if (lane < 6) s_g[lane] = 0.0;
     __syncthreads();
 }
 
@@ -512,10 +514,10 @@ static size_t adj_smem_forward(const StepParams &P, const AdjParams &A, int grou
     return (size_t)A.R * (sizeof(float4) + groups * sizeof(double)) + (size_t)P.n_lut;
 }
 
-static size_t adj_smem_backward(const StepParams &P, const AdjParams &A)
+static size_t adj_smem_backward(const StepParams &P, const AdjParams &A, int groups = 1)
 {
-    return (size_t)A.R * (sizeof(float4) + sizeof(float)) + (size_t)(6 + A.nq) * sizeof(double) +
-           (size_t)P.n_lut;
+    return (size_t)A.R * (sizeof(float4) + groups * sizeof(float)) +
+           (size_t)groups * (6 + A.nq) * sizeof(double) + (size_t)P.n_lut;
 }
 
 // ---------------------------------------------------------------------------------
@@ -530,7 +532,7 @@ static size_t adj_smem_backward(const StepParams &P, const AdjParams &A)
 // ---------------------------------------------------------------------------------
 
 // Threads of the segment kernels' blocks, in groups of ADJ_BLOCK entries with receptor sums of
-// their own, one a block in the reverse sweep. The forwards take two: neighbours in the sorted order then share
+// their own. The forwards take two groups a block: neighbours in the sorted order then share
 // the SM's L1 at nearly the same step (hits 86 -> 92 %) and one copy of the tables, of which
 // more would cost blocks; 4 a SM (64 registers) with the trajectory, 3 (80) without, where
 // the row stores do not hold it up (1e6 x 1080 and 2e5 x 720 with checkpoints, whole gradients:
@@ -540,6 +542,7 @@ static size_t adj_smem_backward(const StepParams &P, const AdjParams &A)
 //
 // FEW: segments of at most 4 groups an SM are bound by a step's latency: one group a block, 128
 // registers a thread, the draws before the gathers so that the two overlap.
+constexpr int SEG_BWD_BLOCK = 128;
 constexpr int seg_fwd_block(bool few) { return few ? 128 : 256; }
 constexpr int SEG_FEW = 4;
 
@@ -593,9 +596,9 @@ __device__ __forceinline__ bool seg_block_empty(const AdjSeg &G, int group0, int
 }
 
 // Receptor forward of a segment (MODE: SegMode). MULTI: entries of several scenarios (else
-// all of scenario 0); FIELDS: a gridded K_h, or no level table. Instructions bound it as they do
-// the advance kernel: the step times come from a table, the deposition words from one block for
-// two steps, the samples by a countdown.
+// all of scenario 0); FIELDS: a gridded K_h, or no level table. Instructions bound it as they do the advance
+// kernel: the step times come from a table, the deposition words from one block for two
+// steps, the samples by a countdown.
 template <int MODE, bool MULTI, bool FIELDS, bool FEW>
 __global__ void __launch_bounds__(seg_fwd_block(FEW), seg_fwd_blocks(MODE, FEW))
 adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
@@ -696,36 +699,43 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
 // before the gathers with several scenarios too, whose gathers miss the L1 more often
 // (inversion of 16 x 1e5: 35.0 -> 34.2 ms); with one they measured no faster there.
 template <bool KHG, bool MULTI, bool FEW>
-__global__ void __launch_bounds__(ADJ_BLOCK, FEW ? 4 : 5)
-adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G)
+__global__ void __launch_bounds__(SEG_BWD_BLOCK, FEW ? 4 : 5)
+adj_backward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
 {
-    const int group = blockIdx.x;
-    const bool from_a = group < G.tiles_a;
-    const unsigned int live = from_a ? *G.live : 0u;
-    if (from_a && (long long)group * ADJ_BLOCK >= (long long)live) return;
+    constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
+    const int group0 = blockIdx.x * GROUPS;
+    const unsigned int live = group0 < G.tiles_a ? *G.live : 0u;
+    if (seg_block_empty(G, group0, GROUPS, n_groups, live)) return;
     extern __shared__ float4 s_dyn[];             // sized by the launch: adj_smem_backward
+    const int gi = threadIdx.x / ADJ_BLOCK;
     float4 *s_rec = s_dyn;                        // [R]
-    double *s_g = reinterpret_cast<double *>(s_rec + A.R);    // [6]
-    double *s_gq = s_g + 6;                       // [nq]
-    float *s_w = reinterpret_cast<float *>(s_gq + A.nq);      // [R]
-    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + A.R);   // [n_lut]
+    double *s_g = reinterpret_cast<double *>(s_rec + A.R);    // [GROUPS][6]
+    double *s_gq = s_g + 6 * GROUPS;              // [GROUPS][nq]
+    float *s_w = reinterpret_cast<float *>(s_gq + GROUPS * A.nq);      // [GROUPS][R]
+    unsigned char *s_lut = reinterpret_cast<unsigned char *>(s_w + GROUPS * A.R);   // [n_lut]
+    s_g += 6 * gi;
+    s_gq += A.nq * gi;
+    s_w += A.R * gi;
     using Lev = Levels<MULTI, !KHG>;              // (the rule is at Levels)
     __shared__ float4 s_ent[Lev::SMEM ? MAX_LEVELS : 1];
     const Lev LV = load_levels<Lev>(P, s_lut, s_ent);
     // the segment's step times, once per block
     __shared__ float4 s_ta[CK];
-    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += ADJ_BLOCK)
+    for (int i = threadIdx.x; i < G.k_hi - G.k_lo; i += SEG_BWD_BLOCK)
         s_ta[i] = step_time_parts<false>(P, G.k_lo + i);
+    const int group = group0 + gi;
+    const bool from_a = group < G.tiles_a;
+    const bool used = group < n_groups && (!from_a || (long long)group * ADJ_BLOCK < (long long)live);
     Tile tb{0, 0, 0};
-    tb.scen = seg_group_scen<MULTI>(P, G, group, from_a);
+    if (used) tb.scen = seg_group_scen<MULTI>(P, G, group, from_a);
     load_receptors(A, tb, s_rec, s_w, s_g, s_gq);     // (ends with a barrier)
     const float sig_h_uniform = sqrtf(P.k2 * fmaxf(P.kh_uniform, 0.0f) * P.dt);
     const float sq2dt = sqrtf(2.0f * P.k_scale * P.dt);
     const uint32_t tab = shared_addr(s_ta);
-    const long long e = (long long)group * ADJ_BLOCK + threadIdx.x;
-    long long home;
-    int scen;
-    const bool valid = seg_entry<MULTI>(P, G, group, from_a, live, home, scen);
+    const long long e = (long long)group * ADJ_BLOCK + threadIdx.x % ADJ_BLOCK;
+    long long home = P.scen[0].first_slot;
+    int scen = 0;
+    const bool valid = used && seg_entry<MULTI>(P, G, group, from_a, live, home, scen);
     const ScenDev &sc = P.scen[scen];
     const float2 *wind = sc.wind_offset;
     // receptor weights of another scenario than the group's come from global memory
@@ -863,11 +873,13 @@ cudaError_t launch_adj_backward_seg(cudaStream_t s, const StepParams &P, const A
     if (n_groups <= 0) return cudaSuccess;
     adj_prefer_l1();
     const bool few = n_groups <= SEG_FEW * n_sm;
-    const size_t sm = adj_smem_backward(P, A);
+    constexpr int GROUPS = SEG_BWD_BLOCK / ADJ_BLOCK;
+    const int n = (n_groups + GROUPS - 1) / GROUPS;
+    const size_t sm = adj_smem_backward(P, A, GROUPS);
     const bool multi = P.n_scen > 1, fields = P.khpair || P.lut_last < 0;
 #define LPM_SEG_BWD(K, U)                                                                 \
-    (few ? adj_backward_seg_kernel<K, U, true><<<n_groups, ADJ_BLOCK, sm, s>>>(P, A, G)    \
-         : adj_backward_seg_kernel<K, U, false><<<n_groups, ADJ_BLOCK, sm, s>>>(P, A, G))
+    (few ? adj_backward_seg_kernel<K, U, true><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups) \
+         : adj_backward_seg_kernel<K, U, false><<<n, SEG_BWD_BLOCK, sm, s>>>(P, A, G, n_groups))
     if (fields && multi)
         LPM_SEG_BWD(true, true);
     else if (fields)
