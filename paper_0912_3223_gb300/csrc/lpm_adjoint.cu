@@ -538,7 +538,10 @@ static size_t adj_smem_backward(const StepParams &P, const AdjParams &A, int gro
 // the row stores do not hold it up (1e6 x 1080 and 2e5 x 720 with checkpoints, whole gradients:
 // 15.8 and 5.3 ms; 4 and 4: 15.8 and 5.7; 3 and 3: 16.0 and 5.4; blocks of 512: 15.9 and 5.7).
 // The reverse sweep at 5 blocks of 128 a SM (96 registers): blocks of 256 at 2 or 3 a SM 16.1 and
-// 16.7 ms, of 384 16.4, of 640 16.6.
+// 16.7 ms, of 384 16.4, of 640 16.6. Its one group a block is indexed as several would be: written
+// for one alone it measured 15.28 -> 15.12 ms with one scenario (1e6 x 1080) and 33.35 -> 33.86
+// with several (inversion of 16 x 1e5; start of the block, entries and sums changed one by one
+// made no difference).
 //
 // FEW: segments of at most 4 groups an SM are bound by a step's latency: one group a block, 128
 // registers a thread, the draws before the gathers so that the two overlap.
@@ -596,9 +599,9 @@ __device__ __forceinline__ bool seg_block_empty(const AdjSeg &G, int group0, int
 }
 
 // Receptor forward of a segment (MODE: SegMode). MULTI: entries of several scenarios (else
-// all of scenario 0); FIELDS: a gridded K_h, or no level table. Instructions bound it as they do the advance
-// kernel: the step times come from a table, the deposition words from one block for two
-// steps, the samples by a countdown.
+// all of scenario 0); FIELDS: a gridded K_h, or no level table. Instructions bound it as they do
+// the advance kernel: the step times come from a table, the deposition words from one block for
+// two steps, the samples by a countdown.
 template <int MODE, bool MULTI, bool FIELDS, bool FEW>
 __global__ void __launch_bounds__(seg_fwd_block(FEW), seg_fwd_blocks(MODE, FEW))
 adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, int n_groups)
@@ -695,7 +698,7 @@ adj_forward_seg_kernel(const StepParams P, const AdjParams A, const AdjSeg G, in
 // Reverse sweep of a segment (KHG: gridded K_h, or no level table). Bound by the latency of
 // its gathers at 19 warps an SM (96 registers hold the record differences; issue 56 % busy);
 // a uniform K_h's scale is taken out of the loop, its vanishing derivative dropped (571 -> 480
-// instructions a step with that, the tabled times and the shared round keys). The draws come
+// executed instructions a step with that, the tabled times and the shared round keys). The draws come
 // before the gathers with several scenarios too, whose gathers miss the L1 more often
 // (inversion of 16 x 1e5: 35.0 -> 34.2 ms); with one they measured no faster there.
 template <bool KHG, bool MULTI, bool FEW>
