@@ -44,12 +44,12 @@ OPS_PER_PARTICLE_STEP_LOW = 350
 # DRAM traffic per advance launch from an ncu capture of two mid-run 60-step launches
 # (hours 10-11 of the realistic workload, persistent grid of 2 blocks per SM; read + write,
 # mean of the two), valid while the kernel sources hash to the values below.
-ADVANCE_TRAFFIC_BYTES = 0.5 * ((22.473984 + 0.000256) + (23.845376 + 0.049664)) * 1e6
-ADVANCE_TRAFFIC_SOURCES = {"lpm_advance.cuh": "4247e0ea", "lpm_device.cuh": "2cc273c0"}
+ADVANCE_TRAFFIC_BYTES = 0.5 * ((22.466816 + 0.000512) + (23.840256 + 0.044544)) * 1e6
+ADVANCE_TRAFFIC_SOURCES = {"lpm_advance.cuh": "81127fec", "lpm_device.cuh": "6aaab966"}
 # Busiest hardware units of the same capture (% of peak, mean of the two launches): the
 # L1 data pipe carrying the weather gathers, and the warp-instruction issue slots.
-ADVANCE_BUSIEST_UNITS = {"l1tex_data_pipe": 0.5 * (57.67 + 57.66) / 100.0,
-                         "issue_slots": 0.5 * (69.71 + 69.73) / 100.0}
+ADVANCE_BUSIEST_UNITS = {"l1tex_data_pipe": 0.5 * (57.25 + 58.00) / 100.0,
+                         "issue_slots": 0.5 * (69.62 + 69.61) / 100.0}
 LANES_PER_SM = 128          # 4 sub-partitions x 32 lanes issue one op per clock
 
 
